@@ -25,10 +25,11 @@ namespace {
 
 constexpr int kGenThreads = 128;
 constexpr int kTraceThreads = 128;
-constexpr int kTraceBlocksPerSM = 8;
-constexpr int kTraceStepsPerRefill = 8;
-constexpr int kLeafQueue = 8;   // postponed triangle tests per lane
-constexpr int kLeafBatch = 16;  // lanes holding one that start a triangle round
+constexpr int kTraceBlocksPerSM = 8;     // 7: the same; 9 and 10 spill: 5% and 15% slower
+constexpr int kTraceStepsPerRefill = 8;  // 4: 6% slower, 12 and 16: within 1%
+constexpr int kTraceNodes = 20;          // pending nodes per lane (a visit needs four free)
+constexpr int kTraceLeaves = 8;          // postponed triangle tests per lane (a visit needs four free)
+constexpr int kLeafBatch = 16;           // lanes holding one that start a triangle round (12 to 22: within 1%)
 
 struct WaveBuffers {
     float4* ray;        // [rays] direction, w = slot index (int bits) of the sample
@@ -155,85 +156,134 @@ __global__ void __launch_bounds__(kGenThreads) wave_gen_kernel(ShadeArgs a, void
     }
 }
 
-// Persistent any-hit tracer with per-lane refill.  A lane holds one ray, the
-// four-wide node it visits next, a short stack of pending nodes and a queue of
-// leaf triangles whose boxes the ray hit (columns of shared-memory arrays);
-// every kTraceStepsPerRefill steps the warp refills the lanes that are idle
-// from the global slot counter.  A step visits one node per lane; triangle
-// tests are postponed and run as warp-wide rounds, one triangle per lane with
-// a non-empty queue, once kLeafBatch lanes hold one or a lane must drain its
-// queue (its nodes are done, or the queue cannot take another node's four
-// leaves), so most rounds run with many lanes converged instead of a few
-// lanes testing while the rest wait.  A ray whose pending nodes outgrow the
-// stack is decided by the stackless walk of the depth-first copy instead.
+// Persistent any-hit tracer with per-lane refill.  A lane holds a ray, the
+// four-wide node it visits next, a stack of pending nodes and a queue of leaf
+// triangles whose boxes its ray hit (columns of shared-memory arrays, so a
+// warp's accesses fall in different banks); every kTraceStepsPerRefill steps
+// the warp gives the lanes that are out of nodes the next rays of the list.
+//
+// A step visits one node per lane.  Triangle tests are postponed and run as
+// warp-wide rounds, one triangle per lane that holds one, once kLeafBatch
+// lanes do or a lane's queue is full.  A lane whose nodes are done takes its
+// next ray at once, although triangles of the last one may still be queued:
+// origin and direction of both rays stay in shared memory (s_ray), entries
+// below lmark belong to the previous one, and the lane only waits for a round
+// when those are still there as the next ray ends too.  (Waiting for the
+// tests instead, with rounds forced by waiting lanes, takes a round at nearly
+// every step with a quarter of its lanes, or leaves lanes idle.)
+//
+// What bounds it is the L1's one wavefront per load of a lane that no other
+// lane's line matches (85% of its peak): two per node visited, two per
+// triangle test, then the shared-memory accesses, which is why a node is two
+// 32-byte loads, a record two loads (load_record), and a child one store.
+// Measured, 1.64M rays against 198k triangles at 512 x 512, 16 samples: 394 us
+// (before: 493 us, issue-bound, a child a branch and a triangle round a step);
+// 67.8M rays against 1.3M triangles: 12.2 ms (before: 15.9 ms).  The rays'
+// order matters little: shuffled 6% slower, sorted by direction 10% faster.
+//
+// A ray whose pending nodes outgrow the stack is decided by the stackless walk
+// of the depth-first copy instead.
 __global__ void __launch_bounds__(kTraceThreads, kTraceBlocksPerSM) wave_trace_kernel(
     const void* __restrict__ nodes, const TriRecord* __restrict__ tris, int n_tris, void* ws, long long P,
     long long slots) {
     pdl_prologue();
+    constexpr int kStep = 4 * kTraceThreads, kPair = 8 * kTraceThreads, kRay = 3 * kPair;
+    __shared__ float2 s_ray[2 * 3 * kTraceThreads];  // two rays per lane: (o.x, o.y), (o.z, d.x), (d.y, d.z)
+    __shared__ int s_slot[2 * kTraceThreads];        // their slots
+    __shared__ int s_node[kTraceNodes * kTraceThreads];
+    __shared__ int s_leaf[kTraceLeaves * kTraceThreads];
     WaveBuffers B = wave_buffers(ws, P, slots);
-    const long long n_rays = (long long)*((volatile unsigned*)B.counter);
+    const unsigned n_rays = *((volatile unsigned*)B.counter);
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
-    long long ray = -1;  // -1 idle, -2 no work left, >= 0 tracing
-    int slot = 0;
-    RayInv r;
-    int node = 0, sp = 0, lq = 0;
-    bool overflow = false;
-    // one column per thread, so a warp's accesses fall in 32 different banks
-    __shared__ int s_stack[kWideStack * kTraceThreads];
-    __shared__ int s_leaf[kLeafQueue * kTraceThreads];
-    int* stack = s_stack + threadIdx.x;
-    int* leafq = s_leaf + threadIdx.x;
     if (n_tris <= 0) return;  // nothing can block a ray; gen already wrote misses
     const WideNode* wn = wide_nodes(nodes, n_tris);
+    const uint32_t rbase = (uint32_t)__cvta_generic_to_shared(s_ray + threadIdx.x);
+    const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(s_slot + threadIdx.x);
+    const uint32_t nbase = (uint32_t)__cvta_generic_to_shared(s_node + threadIdx.x);
+    const uint32_t lbase = (uint32_t)__cvta_generic_to_shared(s_leaf + threadIdx.x);
+    const uint32_t nroom = nbase + (kTraceNodes - 4) * kStep, lroom = lbase + (kTraceLeaves - 4) * kStep;
+    uint32_t na = nbase, la = lbase;  // first free entries
+    uint32_t lmark = lbase;           // leaf entries below it belong to the lane's previous ray
+    int cur = 0;                      // which of the two places in s_ray is the current ray's
+    int node = kWideDone;             // a lane out of nodes has node < 0
+    f3 inv = mk(0.f, 0.f, 0.f), oi = inv;
+    bool more = true;  // rays left in the list (the same for the whole warp)
+    auto load_ray = [&](int which, f3& o, f3& d) {
+        const uint32_t r = rbase + which * kRay;
+        const float2 a = lds64(r), b = lds64(r + kPair), c = lds64(r + 2 * kPair);
+        o = mk(a.x, a.y, b.x);
+        d = mk(b.y, c.x, c.y);
+    };
+    auto blocked = [&](int which) { B.hit[lds32(sbase + which * kStep)] = 1; };
     while (true) {
-        const unsigned need = __ballot_sync(full, ray == -1);
-        if (need) {
-            const int leader = __ffs(need) - 1;
+        const bool free_lane = node < 0 && lmark == lbase;
+        const unsigned idle = __ballot_sync(full, free_lane);
+        if (more && idle) {
             unsigned base = 0;
-            if (lane == leader) base = atomicAdd(B.counter + 1, (unsigned)__popc(need));
-            base = __shfl_sync(full, base, leader);
-            if (ray == -1) {
-                const long long my = (long long)base + __popc(need & lt);
-                if (my >= n_rays) {
-                    ray = -2;
-                } else {
-                    const float4 d = __ldg(B.ray + my);
-                    slot = __float_as_int(d.w);
-                    const float4 o = __ldg(B.origin + (uint32_t)slot % (uint32_t)P);  // slots < 2^31
-                    r = make_ray(mk(o.x, o.y, o.z), mk(d.x, d.y, d.z));
-                    node = 0;
-                    sp = 0;
-                    lq = 0;
-                    overflow = false;
-                    ray = my;
+            if (lane == 0) base = atomicAdd(B.counter + 1, (unsigned)__popc(idle));
+            base = __shfl_sync(full, base, 0);
+            const unsigned my = base + __popc(idle & lt);
+            if (free_lane && my < n_rays) {
+                const float4 d = __ldg(B.ray + my);
+                const int slot = __float_as_int(d.w);
+                const float4 o = __ldg(B.origin + (uint32_t)slot % (uint32_t)P);  // slots < 2^31
+                inv = make_ray(xyz(o), xyz(d)).inv;
+                oi = mk(-o.x * inv.x, -o.y * inv.y, -o.z * inv.z);
+                node = 0;
+                lmark = la;
+                cur ^= 1;
+                const uint32_t r = rbase + cur * kRay;
+                sts64(r, o.x, o.y);
+                sts64(r + kPair, o.z, d.x);
+                sts64(r + 2 * kPair, d.y, d.z);
+                sts32(sbase + cur * kStep, slot);
+            }
+            more = base + (unsigned)__popc(idle) < n_rays;
+        } else if (!__any_sync(full, node >= 0 || la != lbase)) {
+            break;
+        }
+        // every node is visited at most once, so a ray ends within n - 1 visits and as many rounds
+        for (int step = 0; step < kTraceStepsPerRefill; ++step) {
+            if (node >= 0 && la <= lroom && na <= nroom) {
+                wide_visit<kStep>(wn, inv, oi, node, na, la);
+                node = kWideDone;
+                if (na != nbase) {
+                    na -= kStep;
+                    node = lds32(na);
                 }
             }
-        }
-        if (__all_sync(full, ray == -2)) break;
-        // kTraceStepsPerRefill steps; every node is visited at most once, so a ray
-        // ends within n - 1 node visits and as many triangle rounds
-        for (int step = 0; step < kTraceStepsPerRefill; ++step) {
-            const bool act = ray >= 0;
-            // a visit appends at most four leaves: a fuller queue waits for the rounds it forces
-            if (act && node >= 0 && lq <= kLeafQueue - 4)
-                node = wide_visit<kTraceThreads>(wn, r, node, stack, sp, overflow, leafq, lq);
-            const bool pend = act && lq > 0;
-            const bool must = pend && (node == kWideDone || lq > kLeafQueue - 4);
-            const unsigned vote = __ballot_sync(full, pend);
-            if (__popc(vote) >= kLeafBatch || __any_sync(full, must)) {
-                if (pend) {
-                    const int l = leafq[kTraceThreads * --lq];
-                    if (tri_hit(r, tris, ~l, nullptr, nullptr) < FLT_MAX) {
-                        B.hit[slot] = 1;
-                        ray = -1;
+            const unsigned pend = __ballot_sync(full, la != lbase);
+            // a lane that cannot go on without a round: its queue is full, or its next ray waits for the previous one
+            const bool must = la > lroom || (node < 0 && lmark != lbase);
+            if (__popc(pend) >= kLeafBatch || __any_sync(full, must) || !__any_sync(full, node >= 0)) {
+                if (la != lbase) {
+                    la -= kStep;
+                    const int k = ~lds32(la);
+                    const bool prev = la < lmark;
+                    if (prev) lmark = la;
+                    f3 o, d;
+                    load_ray(prev ? cur ^ 1 : cur, o, d);
+                    // (an empty slot's link can only come from a ray with infinite coordinates)
+                    if ((unsigned)k < (unsigned)n_tris && tri_blocks(o, d, tris, k)) {
+                        blocked(prev ? cur ^ 1 : cur);
+                        if (prev) {
+                            la = lmark = lbase;  // nothing of the current ray is queued above it
+                        } else {
+                            la = lmark;
+                            node = kWideDone;
+                            na = nbase;
+                        }
                     }
                 }
             }
-            if (ray >= 0 && node == kWideDone && lq == 0) {  // nodes done and no triangle left: a miss
-                if (overflow && any_hit_threaded(nodes, tris, n_tris, r)) B.hit[slot] = 1;
-                ray = -1;
+            if (node >= 0 && na > nroom) {  // more pending nodes than the stack holds
+                f3 o, d;
+                load_ray(cur, o, d);
+                if (any_hit_threaded(nodes, tris, n_tris, make_ray(o, d))) blocked(cur);
+                node = kWideDone;
+                na = nbase;
             }
         }
     }

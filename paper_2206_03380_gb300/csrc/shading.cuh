@@ -65,6 +65,49 @@ __device__ __forceinline__ float tri_hit(const RayInv& r, const TriRecord* __res
     return tri_hit_v(r, xyz(v0), xyz(e1), xyz(e2), bu, bv);
 }
 
+// The same test of a shadow ray (hit or not) with every rounding written out
+// (one fused multiply-add per term, the contractions tri_hit_v compiles to), so
+// that every kernel that traces shadow rays decides a ray and a triangle
+// alike, whatever the compiler would choose around it.
+__device__ __forceinline__ float tri_dot(f3 a, f3 b) {
+    return __fmaf_rn(a.z, b.z, __fmaf_rn(a.x, b.x, __fmul_rn(a.y, b.y)));
+}
+__device__ __forceinline__ f3 tri_cross(f3 a, f3 b) {
+    return {__fmaf_rn(a.y, b.z, -__fmul_rn(a.z, b.y)), __fmaf_rn(a.z, b.x, -__fmul_rn(a.x, b.z)),
+            __fmaf_rn(a.x, b.y, -__fmul_rn(a.y, b.x))};
+}
+// Triangle record k in two loads: records are 48 bytes apart on 16-byte
+// boundaries, so either their first 32 bytes or their last 32 start on a
+// 32-byte boundary.  (Each load of a lane is one L1 wavefront when lanes read
+// different records; three 16-byte loads made the tracer 3% slower.)
+__device__ __forceinline__ void load_record(const TriRecord* __restrict__ tris, int k, f3& v0, f3& e1, f3& e2) {
+    const char* a = reinterpret_cast<const char*>(tris + k);
+    const bool odd = (reinterpret_cast<uintptr_t>(a) & 16) != 0;
+    float4 x, y;
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w), "=f"(y.x), "=f"(y.y), "=f"(y.z), "=f"(y.w)
+        : "l"(a + (odd ? 16 : 0)));
+    const float4 z = __ldg(reinterpret_cast<const float4*>(a + (odd ? 0 : 32)));
+    v0 = odd ? xyz(z) : xyz(x);
+    e1 = odd ? xyz(x) : xyz(y);
+    e2 = odd ? xyz(y) : xyz(z);
+}
+__device__ __forceinline__ bool tri_blocks(f3 o, f3 d, const TriRecord* __restrict__ tris, int k) {
+    f3 v0, e1, e2;
+    load_record(tris, k, v0, e1, e2);
+    const f3 p = tri_cross(d, e2);
+    const float det = tri_dot(e1, p);
+    if (det == 0.0f) return false;
+    const float inv = 1.0f / det;
+    const f3 s = {__fsub_rn(o.x, v0.x), __fsub_rn(o.y, v0.y), __fsub_rn(o.z, v0.z)};
+    const float u = __fmul_rn(tri_dot(s, p), inv);
+    if (u < 0.0f || u > 1.0f) return false;
+    const f3 q = tri_cross(s, e1);
+    const float v = __fmul_rn(tri_dot(d, q), inv);
+    if (v < 0.0f || __fadd_rn(u, v) > 1.0f) return false;
+    return __fmul_rn(tri_dot(e2, q), inv) > 0.0f;
+}
+
 // slab test of a box given by its corners (xyz of lo and hi); same rounding
 // rule as slab()
 __device__ __forceinline__ bool slab_hit(const RayInv& r, float4 lo, float4 hi) {
@@ -213,13 +256,48 @@ __device__ __forceinline__ int wide_step(const WideNode* __restrict__ wn, const 
     return next;
 }
 
+// Shared-memory accesses by 32-bit shared address.
+__device__ __forceinline__ int lds32(uint32_t a) {
+    int v;
+    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ float2 lds64(uint32_t a) {
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ void sts32(uint32_t a, int v) {
+    asm volatile("st.shared.b32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ void sts64(uint32_t a, float x, float y) {
+    asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(x), "f"(y) : "memory");
+}
+
+// two fused multiply-adds in one instruction: (x.x a + b, x.y a + b)
+__device__ __forceinline__ float2 fma2(float2 x, float2 a, float2 b) {
+    float2 r;
+    asm("{\n\t.reg .b64 rx, ra, rb, rd;\n\t"
+        "mov.b64 rx, {%2, %3};\n\tmov.b64 ra, {%4, %5};\n\tmov.b64 rb, {%6, %7};\n\t"
+        "fma.rn.f32x2 rd, rx, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(x.x), "f"(x.y), "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+
 // The node part of wide_step for a traversal that postpones its triangle
-// tests: hit leaf children are appended to the lane's leaf queue
-// (leafq[i * kStride], lq entries; the caller keeps room for four) instead of
-// being tested.  Returns the next node or kWideDone.
-template <int kStride>
-__device__ __forceinline__ int wide_visit(const WideNode* __restrict__ wn, const RayInv& r, int node, int* stack,
-                                          int& sp, bool& overflow, int* leafq, int& lq) {
+// tests: hit inner children are appended to the lane's node stack (entries at
+// shared address na, kStep bytes apart), hit leaf children to its leaf queue
+// (at la, kStep apart); the caller makes sure that four more of each fit.  One
+// predicated store per child, to whichever of the two, and predicated
+// additions: no branch for other lanes to wait at, and one shared-memory
+// wavefront per child instead of two.  The child tests are wide_child_hits',
+// two children per fused multiply-add instruction, with the origin's product
+// oi = -o / d formed once per ray (its rounding, at most 2^-24 |o| / |d|, is
+// under 2^-7 quantisation steps for origins inside the scene's bounds).
+template <int kStep>
+__device__ __forceinline__ void wide_visit(const WideNode* __restrict__ wn, f3 inv, f3 oi, int node, uint32_t& na,
+                                           uint32_t& la) {
     float4 a, b, c;
     int4 d;
     asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
@@ -228,24 +306,43 @@ __device__ __forceinline__ int wide_visit(const WideNode* __restrict__ wn, const
     asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
         : "=f"(c.x), "=f"(c.y), "=f"(c.z), "=f"(c.w), "=r"(d.x), "=r"(d.y), "=r"(d.z), "=r"(d.w)
         : "l"(reinterpret_cast<const char*>(wn + node) + 32));
-    const unsigned m = wide_child_hits(r, a, b, c);
-    int next = kWideDone;
+    const uint32_t lox = __float_as_uint(b.z), loy = __float_as_uint(b.w), loz = __float_as_uint(c.x);
+    const uint32_t hix = __float_as_uint(c.y), hiy = __float_as_uint(c.z), hiz = __float_as_uint(c.w);
+    const bool px = inv.x >= 0.0f, py = inv.y >= 0.0f, pz = inv.z >= 0.0f;
+    const uint32_t nx = px ? lox : hix, fx = px ? hix : lox;
+    const uint32_t ny = py ? loy : hiy, fy = py ? hiy : loy;
+    const uint32_t nz = pz ? loz : hiz, fz = pz ? hiz : loz;
+    const float ax = a.w * inv.x, ay = b.x * inv.y, az = b.y * inv.z;
+    const float bx = fmaf(-8388608.0f, ax, fmaf(a.x, inv.x, oi.x));
+    const float by = fmaf(-8388608.0f, ay, fmaf(a.y, inv.y, oi.y));
+    const float bz = fmaf(-8388608.0f, az, fmaf(a.z, inv.z, oi.z));
+    const float2 ax2 = {ax, ax}, bx2 = {bx, bx}, ay2 = {ay, ay}, by2 = {by, by}, az2 = {az, az}, bz2 = {bz, bz};
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int l = k == 0 ? d.x : k == 1 ? d.y : k == 2 ? d.z : d.w;
-        if (!((m >> k) & 1u)) continue;
-        if (l < 0) {
-            leafq[kStride * lq++] = l;
-        } else if (next == kWideDone) {
-            next = l;
-        } else if (sp < kWideStack) {
-            stack[kStride * sp++] = l;
-        } else {
-            overflow = true;
+    for (int k = 0; k < 4; k += 2) {
+        const float2 x0 = fma2({qbyte(nx, k), qbyte(nx, k + 1)}, ax2, bx2);
+        const float2 y0 = fma2({qbyte(ny, k), qbyte(ny, k + 1)}, ay2, by2);
+        const float2 z0 = fma2({qbyte(nz, k), qbyte(nz, k + 1)}, az2, bz2);
+        const float2 x1 = fma2({qbyte(fx, k), qbyte(fx, k + 1)}, ax2, bx2);
+        const float2 y1 = fma2({qbyte(fy, k), qbyte(fy, k + 1)}, ay2, by2);
+        const float2 z1 = fma2({qbyte(fz, k), qbyte(fz, k + 1)}, az2, bz2);
+        const float t0[2] = {fmax3(x0.x, y0.x, fmaxf(z0.x, 0.0f)), fmax3(x0.y, y0.y, fmaxf(z0.y, 0.0f))};
+        const float t1[2] = {fmin3(x1.x, y1.x, z1.x), fmin3(x1.y, y1.y, z1.y)};
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int l = k + h == 0 ? d.x : k + h == 1 ? d.y : k + h == 2 ? d.z : d.w;
+            asm volatile(
+                "{\n\t.reg .pred h, pl, pn;\n\t.reg .u32 ad;\n\t"
+                "setp.le.f32 h, %2, %3;\n\t"
+                "setp.lt.and.s32 pl|pn, %4, 0, h;\n\t"
+                "selp.u32 ad, %0, %1, pl;\n\t"
+                "@h st.shared.b32 [ad], %4;\n\t"
+                "@pl add.u32 %0, %0, %5;\n\t"
+                "@pn add.u32 %1, %1, %5;\n\t}"
+                : "+r"(la), "+r"(na)
+                : "f"(t0[h]), "f"(t1[h]), "r"(l), "n"(kStep)
+                : "memory");
         }
     }
-    if (next == kWideDone && sp > 0) next = stack[kStride * --sp];
-    return next;
 }
 
 // any hit with t > 0 (shadow ray, no far limit) over the four-wide nodes

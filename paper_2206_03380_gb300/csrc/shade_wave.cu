@@ -19,17 +19,14 @@
 #include "common.cuh"
 #include "internal.h"
 #include "shading.cuh"
+#include "trace.cuh"
 
 namespace mcdi {
 namespace {
 
 constexpr int kGenThreads = 128;
-constexpr int kTraceThreads = 128;
-constexpr int kTraceBlocksPerSM = 8;     // 7: the same; 9 and 10 spill: 5% and 15% slower
-constexpr int kTraceStepsPerRefill = 8;  // 4: 6% slower, 12 and 16: within 1%
-constexpr int kTraceNodes = 20;          // pending nodes per lane (a visit needs four free)
-constexpr int kTraceLeaves = 8;          // postponed triangle tests per lane (a visit needs four free)
-constexpr int kLeafBatch = 16;           // lanes holding one that start a triangle round (12 to 22: within 1%)
+constexpr int kGenBlocksPerSM = 9;  // 56 registers, no spills; 7 and 8: 4% slower, 10 spills: 2% slower
+constexpr int kTraceBlocksPerSM = 8;  // 7: the same; 9 and 10 spill: 5% and 15% slower
 
 struct WaveBuffers {
     float4* ray;        // [rays] direction, w = slot index (int bits) of the sample
@@ -92,7 +89,8 @@ __global__ void wave_reset_kernel(void* ws, long long P, long long slots) {
 // depend on which warp drew it.
 constexpr int kGenQuarters = kGenThreads / 32;
 
-__global__ void __launch_bounds__(kGenThreads) wave_gen_kernel(ShadeArgs a, void* ws, float4* __restrict__ kd_out) {
+__global__ void __launch_bounds__(kGenThreads, kGenBlocksPerSM) wave_gen_kernel(ShadeArgs a, void* ws,
+                                                                  float4* __restrict__ kd_out) {
     pdl_prologue();
     extern __shared__ float s_marg[];
     const int lane = threadIdx.x & 31, quarter = threadIdx.x >> 5;
@@ -115,7 +113,7 @@ __global__ void __launch_bounds__(kGenThreads) wave_gen_kernel(ShadeArgs a, void
                               : make_float4(0.f, 0.f, 0.f, 0.f);
     Probe Pr = wave_probe(a);
     stage_marginal(Pr, s_marg);
-    const f3 origin = covered ? px.p + px.n * a.ray_eps : mk(0.f, 0.f, 0.f);
+    const f3 origin = covered ? fma_rn(px.n, a.ray_eps, px.p) : mk(0.f, 0.f, 0.f);
     if (covered && quarter == 0) B.origin[idx] = make_float4(origin.x, origin.y, origin.z, 0.0f);
     for (int j = quarter; j < spp; j += kGenQuarters) {
         const long long s = (long long)j * P + idx;
@@ -131,10 +129,10 @@ __global__ void __launch_bounds__(kGenThreads) wave_gen_kernel(ShadeArgs a, void
                 rec.x = __int_as_float(t);
                 rec.y = ci * MCDI_INV_PI * inv_denom;  // c_d = L rec.y
                 if (px.spec_on) {
-                    const f3 h = normalize(wi + px.wo);
-                    const float D = ggx_D(dot(px.n, h), sin2_between(px.n, h), px.a2);
+                    const f3 h = half_vector(wi, px.wo);
+                    const float D = ggx_D(dot_rn(px.n, h), sin2_between(px.n, h), px.a2);
                     const float G2 = 1.0f / (1.0f + ggx_lambda(ci, px.a2) + ggx_lambda(px.co, px.a2));
-                    rec.z = schlick_weight(dot(px.wo, h));
+                    rec.z = schlick_weight(dot_rn(px.wo, h));
                     rec.w = D * G2 / (4.0f * px.co) * inv_denom;  // c_s = spec_colour(L, F0, rec.z, rec.w)
                 }
             }
@@ -156,137 +154,60 @@ __global__ void __launch_bounds__(kGenThreads) wave_gen_kernel(ShadeArgs a, void
     }
 }
 
-// Persistent any-hit tracer with per-lane refill.  A lane holds a ray, the
-// four-wide node it visits next, a stack of pending nodes and a queue of leaf
-// triangles whose boxes its ray hit (columns of shared-memory arrays, so a
-// warp's accesses fall in different banks); every kTraceStepsPerRefill steps
-// the warp gives the lanes that are out of nodes the next rays of the list.
-//
-// A step visits one node per lane.  Triangle tests are postponed and run as
-// warp-wide rounds, one triangle per lane that holds one, once kLeafBatch
-// lanes do or a lane's queue is full.  A lane whose nodes are done takes its
-// next ray at once, although triangles of the last one may still be queued:
-// origin and direction of both rays stay in shared memory (s_ray), entries
-// below lmark belong to the previous one, and the lane only waits for a round
-// when those are still there as the next ray ends too.  (Waiting for the
-// tests instead, with rounds forced by waiting lanes, takes a round at nearly
-// every step with a quarter of its lanes, or leaves lanes idle.)
+// The rays of the list, copied to shared memory as a lane takes them: a lane
+// has two places, for its current ray and the one before.
+struct ListRays {
+    static constexpr int kStep = 4 * kTraceThreads, kPair = 8 * kTraceThreads, kRay = 3 * kPair;
+    WaveBuffers B;
+    unsigned n;
+    uint32_t P;
+    uint32_t rbase, sbase;  // shared addresses of the lane's columns: (o.x, o.y), (o.z, d.x), (d.y, d.z); slots
+
+    __device__ __forceinline__ unsigned count() const { return n; }
+    __device__ __forceinline__ unsigned take(unsigned k) { return atomicAdd(B.counter + 1, k); }
+    __device__ __forceinline__ int start(unsigned i, int id, f3& o, f3& d) {
+        const float4 v = __ldg(B.ray + i);
+        const int slot = __float_as_int(v.w);
+        d = xyz(v);
+        o = xyz(__ldg(B.origin + (uint32_t)slot % P));  // slots < 2^31
+        id ^= 1;
+        const uint32_t r = rbase + id * kRay;
+        sts64(r, o.x, o.y);
+        sts64(r + kPair, o.z, d.x);
+        sts64(r + 2 * kPair, d.y, d.z);
+        sts32(sbase + id * kStep, slot);
+        return id;
+    }
+    __device__ __forceinline__ void load(int id, f3& o, f3& d) const {
+        const uint32_t r = rbase + id * kRay;
+        const float2 a = lds64(r), b = lds64(r + kPair), c = lds64(r + 2 * kPair);
+        o = mk(a.x, a.y, b.x);
+        d = mk(b.y, c.x, c.y);
+    }
+    __device__ __forceinline__ void blocked(int id) { B.hit[lds32(sbase + id * kStep)] = 1; }
+};
+
+// Persistent any-hit tracer (trace_rays) over the whole list.
 //
 // What bounds it is the L1's one wavefront per load of a lane that no other
 // lane's line matches (85% of its peak): two per node visited, two per
 // triangle test, then the shared-memory accesses, which is why a node is two
 // 32-byte loads, a record two loads (load_record), and a child one store.
-// Measured, 1.64M rays against 198k triangles at 512 x 512, 16 samples: 394 us
+// Measured, 1.64M rays against 198k triangles at 512 x 512, 16 samples: 397 us
 // (before: 493 us, issue-bound, a child a branch and a triangle round a step);
-// 67.8M rays against 1.3M triangles: 12.2 ms (before: 15.9 ms).  The rays'
+// 67.8M rays against 1.3M triangles: 12.3 ms (before: 15.9 ms).  The rays'
 // order matters little: shuffled 6% slower, sorted by direction 10% faster.
-//
-// A ray whose pending nodes outgrow the stack is decided by the stackless walk
-// of the depth-first copy instead.
 __global__ void __launch_bounds__(kTraceThreads, kTraceBlocksPerSM) wave_trace_kernel(
     const void* __restrict__ nodes, const TriRecord* __restrict__ tris, int n_tris, void* ws, long long P,
     long long slots) {
     pdl_prologue();
-    constexpr int kStep = 4 * kTraceThreads, kPair = 8 * kTraceThreads, kRay = 3 * kPair;
-    __shared__ float2 s_ray[2 * 3 * kTraceThreads];  // two rays per lane: (o.x, o.y), (o.z, d.x), (d.y, d.z)
-    __shared__ int s_slot[2 * kTraceThreads];        // their slots
-    __shared__ int s_node[kTraceNodes * kTraceThreads];
-    __shared__ int s_leaf[kTraceLeaves * kTraceThreads];
-    WaveBuffers B = wave_buffers(ws, P, slots);
-    const unsigned n_rays = *((volatile unsigned*)B.counter);
-    const unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    const unsigned lt = (1u << lane) - 1u;
-    if (n_tris <= 0) return;  // nothing can block a ray; gen already wrote misses
-    const WideNode* wn = wide_nodes(nodes, n_tris);
-    const uint32_t rbase = (uint32_t)__cvta_generic_to_shared(s_ray + threadIdx.x);
-    const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(s_slot + threadIdx.x);
-    const uint32_t nbase = (uint32_t)__cvta_generic_to_shared(s_node + threadIdx.x);
-    const uint32_t lbase = (uint32_t)__cvta_generic_to_shared(s_leaf + threadIdx.x);
-    const uint32_t nroom = nbase + (kTraceNodes - 4) * kStep, lroom = lbase + (kTraceLeaves - 4) * kStep;
-    uint32_t na = nbase, la = lbase;  // first free entries
-    uint32_t lmark = lbase;           // leaf entries below it belong to the lane's previous ray
-    int cur = 0;                      // which of the two places in s_ray is the current ray's
-    int node = kWideDone;             // a lane out of nodes has node < 0
-    f3 inv = mk(0.f, 0.f, 0.f), oi = inv;
-    bool more = true;  // rays left in the list (the same for the whole warp)
-    auto load_ray = [&](int which, f3& o, f3& d) {
-        const uint32_t r = rbase + which * kRay;
-        const float2 a = lds64(r), b = lds64(r + kPair), c = lds64(r + 2 * kPair);
-        o = mk(a.x, a.y, b.x);
-        d = mk(b.y, c.x, c.y);
-    };
-    auto blocked = [&](int which) { B.hit[lds32(sbase + which * kStep)] = 1; };
-    while (true) {
-        const bool free_lane = node < 0 && lmark == lbase;
-        const unsigned idle = __ballot_sync(full, free_lane);
-        if (more && idle) {
-            unsigned base = 0;
-            if (lane == 0) base = atomicAdd(B.counter + 1, (unsigned)__popc(idle));
-            base = __shfl_sync(full, base, 0);
-            const unsigned my = base + __popc(idle & lt);
-            if (free_lane && my < n_rays) {
-                const float4 d = __ldg(B.ray + my);
-                const int slot = __float_as_int(d.w);
-                const float4 o = __ldg(B.origin + (uint32_t)slot % (uint32_t)P);  // slots < 2^31
-                inv = make_ray(xyz(o), xyz(d)).inv;
-                oi = mk(-o.x * inv.x, -o.y * inv.y, -o.z * inv.z);
-                node = 0;
-                lmark = la;
-                cur ^= 1;
-                const uint32_t r = rbase + cur * kRay;
-                sts64(r, o.x, o.y);
-                sts64(r + kPair, o.z, d.x);
-                sts64(r + 2 * kPair, d.y, d.z);
-                sts32(sbase + cur * kStep, slot);
-            }
-            more = base + (unsigned)__popc(idle) < n_rays;
-        } else if (!__any_sync(full, node >= 0 || la != lbase)) {
-            break;
-        }
-        // every node is visited at most once, so a ray ends within n - 1 visits and as many rounds
-        for (int step = 0; step < kTraceStepsPerRefill; ++step) {
-            if (node >= 0 && la <= lroom && na <= nroom) {
-                wide_visit<kStep>(wn, inv, oi, node, na, la);
-                node = kWideDone;
-                if (na != nbase) {
-                    na -= kStep;
-                    node = lds32(na);
-                }
-            }
-            const unsigned pend = __ballot_sync(full, la != lbase);
-            // a lane that cannot go on without a round: its queue is full, or its next ray waits for the previous one
-            const bool must = la > lroom || (node < 0 && lmark != lbase);
-            if (__popc(pend) >= kLeafBatch || __any_sync(full, must) || !__any_sync(full, node >= 0)) {
-                if (la != lbase) {
-                    la -= kStep;
-                    const int k = ~lds32(la);
-                    const bool prev = la < lmark;
-                    if (prev) lmark = la;
-                    f3 o, d;
-                    load_ray(prev ? cur ^ 1 : cur, o, d);
-                    // (an empty slot's link can only come from a ray with infinite coordinates)
-                    if ((unsigned)k < (unsigned)n_tris && tri_blocks(o, d, tris, k)) {
-                        blocked(prev ? cur ^ 1 : cur);
-                        if (prev) {
-                            la = lmark = lbase;  // nothing of the current ray is queued above it
-                        } else {
-                            la = lmark;
-                            node = kWideDone;
-                            na = nbase;
-                        }
-                    }
-                }
-            }
-            if (node >= 0 && na > nroom) {  // more pending nodes than the stack holds
-                f3 o, d;
-                load_ray(cur, o, d);
-                if (any_hit_threaded(nodes, tris, n_tris, make_ray(o, d))) blocked(cur);
-                node = kWideDone;
-                na = nbase;
-            }
-        }
-    }
+    __shared__ float2 s_ray[2 * 3 * kTraceThreads];
+    __shared__ int s_slot[2 * kTraceThreads];
+    __shared__ TraceStacks s_stacks;
+    ListRays rays{wave_buffers(ws, P, slots), 0u, (uint32_t)P, (uint32_t)__cvta_generic_to_shared(s_ray + threadIdx.x),
+                  (uint32_t)__cvta_generic_to_shared(s_slot + threadIdx.x)};
+    rays.n = *((volatile unsigned*)rays.B.counter);
+    trace_rays(nodes, tris, n_tris, s_stacks, rays);
 }
 
 __global__ void __launch_bounds__(kGenThreads) wave_accum_kernel(ShadeArgs a, const void* ws,

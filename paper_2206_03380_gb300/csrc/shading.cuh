@@ -9,6 +9,41 @@
 
 namespace mcdi {
 
+// ---------------------------------------------------------------- fixed roundings
+// What decides a sample (its direction, its probe texel, whether a triangle
+// blocks its ray) is written with every rounding spelled out, so that all the
+// kernels that draw a sample or trace its ray, whatever is compiled around it,
+// decide it alike: a sum of products as one fused multiply-add per product
+// after the first, a + b (p q) as one.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float dot_rn(f3 a, f3 b) {
+    return fma_rn(a.z, b.z, fma_rn(a.x, b.x, mul_rn(a.y, b.y)));
+}
+// the same sum with the first two products the other way round
+__device__ __forceinline__ float dot_xy_rn(f3 a, f3 b) {
+    return fma_rn(a.z, b.z, fma_rn(a.y, b.y, mul_rn(a.x, b.x)));
+}
+__device__ __forceinline__ f3 cross_rn(f3 a, f3 b) {
+    return {fma_rn(a.y, b.z, -mul_rn(a.z, b.y)), fma_rn(a.z, b.x, -mul_rn(a.x, b.z)),
+            fma_rn(a.x, b.y, -mul_rn(a.y, b.x))};
+}
+__device__ __forceinline__ f3 scale_rn(f3 a, float s) { return {mul_rn(a.x, s), mul_rn(a.y, s), mul_rn(a.z, s)}; }
+__device__ __forceinline__ f3 add_rn(f3 a, f3 b) { return {add_rn(a.x, b.x), add_rn(a.y, b.y), add_rn(a.z, b.z)}; }
+__device__ __forceinline__ f3 normalize_rn(f3 a) { return scale_rn(a, rsqrtf(dot_rn(a, a))); }
+__device__ __forceinline__ f3 normalize_xy_rn(f3 a) { return scale_rn(a, rsqrtf(dot_xy_rn(a, a))); }
+// a x + b y + c z
+__device__ __forceinline__ f3 combine_rn(f3 a, float x, f3 b, float y, f3 c, float z) {
+    return {fma_rn(c.x, z, fma_rn(a.x, x, mul_rn(b.x, y))), fma_rn(c.y, z, fma_rn(a.y, x, mul_rn(b.y, y))),
+            fma_rn(c.z, z, fma_rn(a.z, x, mul_rn(b.z, y)))};
+}
+// a s + b
+__device__ __forceinline__ f3 fma_rn(f3 a, float s, f3 b) {
+    return {fma_rn(a.x, s, b.x), fma_rn(a.y, s, b.y), fma_rn(a.z, s, b.z)};
+}
+
 // ---------------------------------------------------------------- traversal
 struct RayInv {
     f3 o, d, inv;
@@ -66,16 +101,7 @@ __device__ __forceinline__ float tri_hit(const RayInv& r, const TriRecord* __res
 }
 
 // The same test of a shadow ray (hit or not) with every rounding written out
-// (one fused multiply-add per term, the contractions tri_hit_v compiles to), so
-// that every kernel that traces shadow rays decides a ray and a triangle
-// alike, whatever the compiler would choose around it.
-__device__ __forceinline__ float tri_dot(f3 a, f3 b) {
-    return __fmaf_rn(a.z, b.z, __fmaf_rn(a.x, b.x, __fmul_rn(a.y, b.y)));
-}
-__device__ __forceinline__ f3 tri_cross(f3 a, f3 b) {
-    return {__fmaf_rn(a.y, b.z, -__fmul_rn(a.z, b.y)), __fmaf_rn(a.z, b.x, -__fmul_rn(a.x, b.z)),
-            __fmaf_rn(a.x, b.y, -__fmul_rn(a.y, b.x))};
-}
+// (the products of tri_hit_v as the compiler contracts them).
 // Triangle record k in two loads: records are 48 bytes apart on 16-byte
 // boundaries, so either their first 32 bytes or their last 32 start on a
 // 32-byte boundary.  (Each load of a lane is one L1 wavefront when lanes read
@@ -95,17 +121,17 @@ __device__ __forceinline__ void load_record(const TriRecord* __restrict__ tris, 
 __device__ __forceinline__ bool tri_blocks(f3 o, f3 d, const TriRecord* __restrict__ tris, int k) {
     f3 v0, e1, e2;
     load_record(tris, k, v0, e1, e2);
-    const f3 p = tri_cross(d, e2);
-    const float det = tri_dot(e1, p);
+    const f3 p = cross_rn(d, e2);
+    const float det = dot_rn(e1, p);
     if (det == 0.0f) return false;
     const float inv = 1.0f / det;
     const f3 s = {__fsub_rn(o.x, v0.x), __fsub_rn(o.y, v0.y), __fsub_rn(o.z, v0.z)};
-    const float u = __fmul_rn(tri_dot(s, p), inv);
+    const float u = __fmul_rn(dot_rn(s, p), inv);
     if (u < 0.0f || u > 1.0f) return false;
-    const f3 q = tri_cross(s, e1);
-    const float v = __fmul_rn(tri_dot(d, q), inv);
+    const f3 q = cross_rn(s, e1);
+    const float v = __fmul_rn(dot_rn(d, q), inv);
     if (v < 0.0f || __fadd_rn(u, v) > 1.0f) return false;
-    return __fmul_rn(tri_dot(e2, q), inv) > 0.0f;
+    return __fmul_rn(dot_rn(e2, q), inv) > 0.0f;
 }
 
 // slab test of a box given by its corners (xyz of lo and hi); same rounding
@@ -136,7 +162,7 @@ __device__ __forceinline__ int threaded_step(const ThreadedNode* __restrict__ tn
             next = i + 1;
         } else {
             if (kCount) ++*tri_tests;
-            if (tri_hit(r, tris, tri, nullptr, nullptr) < FLT_MAX) return -1;
+            if (tri_blocks(r.o, r.d, tris, tri)) return -1;
         }
     }
     return next > i ? next : i + 1;  // strictly increasing: at most 2 n - 1 steps
@@ -250,7 +276,7 @@ __device__ __forceinline__ int wide_step(const WideNode* __restrict__ wn, const 
         leaves &= leaves - 1;
         const int l = k == 0 ? d.x : k == 1 ? d.y : k == 2 ? d.z : d.w;
         if (kCount) ++*tri_tests;
-        if (tri_hit(r, tris, ~l, nullptr, nullptr) < FLT_MAX) return kWideBlocked;
+        if (tri_blocks(r.o, r.d, tris, ~l)) return kWideBlocked;
     }
     if (next == kWideDone && sp > 0) next = stack[kStride * --sp];
     return next;
@@ -345,26 +371,6 @@ __device__ __forceinline__ void wide_visit(const WideNode* __restrict__ wn, f3 i
     }
 }
 
-// any hit with t > 0 (shadow ray, no far limit) over the four-wide nodes
-// (at most 2 n - 1 node visits: each node is pushed at most once)
-__device__ __forceinline__ bool any_hit(const void* nodes, const TriRecord* __restrict__ tris, int n_tris,
-                                        const RayInv& r) {
-    if (n_tris <= 0) return false;
-    const WideNode* wn = wide_nodes(nodes, n_tris);
-    int stack[kWideStack];
-    int sp = 0, node = 0;
-    bool overflow = false, done = false;
-    for (int it = 0; it < 2 * n_tris; ++it) {
-        node = wide_step(wn, tris, r, node, stack, sp, overflow);
-        if (node == kWideBlocked) return true;
-        if (node == kWideDone) {
-            done = true;
-            break;
-        }
-    }
-    return (overflow || !done) ? any_hit_threaded(nodes, tris, n_tris, r) : false;
-}
-
 // closest hit; returns the leaf (triangle record) index or -1
 __device__ __forceinline__ int closest_hit(const BvhNode* __restrict__ nodes, const TriRecord* __restrict__ tris,
                                            int n_tris, const RayInv& r, float* t_out, float* bu, float* bv) {
@@ -443,7 +449,7 @@ __device__ __forceinline__ f3 dir_from_uv(float u, float v, float* sin_theta) {
     sincospif(2.0f * u, &sp, &cp);
     sincospif(v, &st, &ct);
     *sin_theta = st;
-    return mk(st * cp, ct, st * sp);
+    return mk(mul_rn(st, cp), ct, mul_rn(st, sp));
 }
 
 struct Probe {
@@ -464,12 +470,12 @@ __device__ __forceinline__ void stage_marginal(Probe& P, float* s_marg) {
 
 // probe texel of a direction and sin(theta) (accurate near the poles)
 __device__ __forceinline__ int texel_of_dir(const Probe& P, f3 d, float* sin_theta) {
-    const float st = sqrtf(d.x * d.x + d.z * d.z);
-    float u = atan2f(d.z, d.x) * (0.5f * MCDI_INV_PI);
-    if (u < 0.0f) u += 1.0f;
-    const float v = atan2f(st, d.y) * MCDI_INV_PI;
-    const int i = min(P.W - 1, (int)(u * (float)P.W));
-    const int j = min(P.H - 1, (int)(v * (float)P.H));
+    const float st = sqrtf(fma_rn(d.z, d.z, mul_rn(d.x, d.x)));
+    float u = mul_rn(atan2f(d.z, d.x), 0.5f * MCDI_INV_PI);
+    if (u < 0.0f) u = add_rn(u, 1.0f);
+    const float v = mul_rn(atan2f(st, d.y), MCDI_INV_PI);
+    const int i = min(P.W - 1, (int)mul_rn(u, (float)P.W));
+    const int j = min(P.H - 1, (int)mul_rn(v, (float)P.H));
     *sin_theta = st;
     return j * P.W + i;
 }
@@ -479,9 +485,9 @@ __device__ __forceinline__ float pdf_light_texel(const Probe& P, int t, float st
     if (!P.on || !(st > 0.0f)) return 0.0f;
     const int j = t / P.W, i = t - j * P.W;
     const float* c = P.cond + (size_t)j * (P.W + 1);
-    const float wr = P.marg[j + 1] - P.marg[j];
-    const float wc = __ldg(c + i + 1) - __ldg(c + i);
-    return ((float)P.W * (float)P.H * wr * wc) / (2.0f * MCDI_PI * MCDI_PI * st);
+    const float wr = sub_rn(P.marg[j + 1], P.marg[j]);
+    const float wc = sub_rn(__ldg(c + i + 1), __ldg(c + i));
+    return mul_rn(mul_rn(mul_rn((float)P.W, (float)P.H), wr), wc) / mul_rn(2.0f * MCDI_PI * MCDI_PI, st);
 }
 
 // probe sample; returns false if the technique is off
@@ -492,12 +498,14 @@ __device__ __forceinline__ bool sample_light(const Probe& P, float u0, float u1,
     const float* c = P.cond + (size_t)j * (P.W + 1);
     const int i = upper_index(c, P.W, u1);
     const float c0 = __ldg(c + i), c1 = __ldg(c + i + 1);
-    const float dv = fminf((u0 - m0) / (m1 - m0), 0.99999994f);
-    const float du = fminf((u1 - c0) / (c1 - c0), 0.99999994f);
+    const float dm = sub_rn(m1, m0), dc = sub_rn(c1, c0);
+    const float dv = fminf(sub_rn(u0, m0) / dm, 0.99999994f);
+    const float du = fminf(sub_rn(u1, c0) / dc, 0.99999994f);
     float st;
-    *d = dir_from_uv(((float)i + du) / (float)P.W, ((float)j + dv) / (float)P.H, &st);
+    *d = dir_from_uv(add_rn((float)i, du) / (float)P.W, add_rn((float)j, dv) / (float)P.H, &st);
     *texel = j * P.W + i;
-    *pdf = st > 0.0f ? ((float)P.W * (float)P.H * (m1 - m0) * (c1 - c0)) / (2.0f * MCDI_PI * MCDI_PI * st) : 0.0f;
+    *pdf = st > 0.0f ? mul_rn(mul_rn(mul_rn((float)P.W, (float)P.H), dm), dc) / mul_rn(2.0f * MCDI_PI * MCDI_PI, st)
+                     : 0.0f;
     return true;
 }
 
@@ -505,68 +513,76 @@ __device__ __forceinline__ bool sample_light(const Probe& P, float u0, float u1,
 // orthonormal basis of Duff et al. 2017 (sign(0) = +1)
 __device__ __forceinline__ void frame(f3 n, f3* b1, f3* b2) {
     const float s = n.z >= 0.0f ? 1.0f : -1.0f;
-    const float a = -1.0f / (s + n.z);
-    const float b = n.x * n.y * a;
-    *b1 = mk(1.0f + s * n.x * n.x * a, s * b, -s * n.x);
-    *b2 = mk(b, s + n.y * n.y * a, -n.y);
+    const float a = -1.0f / add_rn(s, n.z);
+    const float b = mul_rn(mul_rn(n.x, n.y), a);
+    *b1 = mk(fma_rn(mul_rn(mul_rn(s, n.x), n.x), a, 1.0f), mul_rn(s, b), mul_rn(-s, n.x));
+    *b2 = mk(b, fma_rn(mul_rn(n.y, n.y), a, s), -n.y);
 }
 
 __device__ __forceinline__ f3 sample_cosine(f3 n, f3 b1, f3 b2, float u0, float u1) {
     float sp, cp;
     sincospif(2.0f * u1, &sp, &cp);
     const float r = sqrtf(u0);
-    const float z = sqrtf(1.0f - u0);
-    return b1 * (r * cp) + b2 * (r * sp) + n * z;
+    const float z = sqrtf(sub_rn(1.0f, u0));
+    return combine_rn(b1, mul_rn(r, cp), b2, mul_rn(r, sp), n, z);
 }
 
 // GGX normal distribution with the denominator term nh^2 (a2 - 1) + 1 written as
 // sin^2 + nh^2 a2 (s2 = |n x h|^2): free of the cancellation of 1 - nh^2 near the
 // lobe peak, which in FP32 would cost ~1e-3 relative accuracy at alpha ~ 0.006.
-__device__ __forceinline__ float ggx_D_denom(float nh, float s2, float a2) { return s2 + nh * nh * a2; }
+__device__ __forceinline__ float ggx_D_denom(float nh, float s2, float a2) { return fma_rn(mul_rn(nh, nh), a2, s2); }
 __device__ __forceinline__ float ggx_D(float nh, float s2, float a2) {
     if (!(nh > 0.0f)) return 0.0f;
     const float d = ggx_D_denom(nh, s2, a2);
-    return a2 / (MCDI_PI * d * d);
+    return a2 / mul_rn(mul_rn(MCDI_PI, d), d);
 }
 __device__ __forceinline__ float sin2_between(f3 n, f3 h) {
-    const f3 c = cross(n, h);
-    return dot(c, c);
+    const f3 c = cross_rn(n, h);
+    return dot_rn(c, c);
 }
 
 __device__ __forceinline__ float ggx_lambda(float c, float a2) {
-    const float z = a2 * (1.0f / (c * c) - 1.0f);
-    return 0.5f * (sqrtf(1.0f + z) - 1.0f);
+    const float z1 = fma_rn(a2, sub_rn(1.0f / mul_rn(c, c), 1.0f), 1.0f);
+    return mul_rn(0.5f, sub_rn(sqrtf(z1), 1.0f));
 }
 
-// Heitz 2018 visible-normal sample, returns the reflected light direction
+// Heitz 2018 visible-normal sample, returns the reflected light direction.  The
+// adjoint sums wo's projections in another order than the forward kernels (a
+// last bit of the direction, a texel or two of a million samples).
+template <bool kAdjoint>
 __device__ __forceinline__ f3 sample_ggx(f3 n, f3 b1, f3 b2, f3 wo, float alpha, float u0, float u1) {
-    const f3 lo = mk(dot(wo, b1), dot(wo, b2), dot(wo, n));
-    const f3 vh = normalize(mk(alpha * lo.x, alpha * lo.y, lo.z));
-    const float lensq = vh.x * vh.x + vh.y * vh.y;
-    f3 t1v = lensq > 0.0f ? mk(-vh.y, vh.x, 0.0f) * rsqrtf(lensq) : mk(1.0f, 0.0f, 0.0f);
-    const f3 t2v = cross(vh, t1v);
+    const f3 lo = kAdjoint ? mk(dot_rn(wo, b1), dot_rn(wo, b2), dot_rn(wo, n))
+                           : mk(dot_xy_rn(wo, b1), dot_xy_rn(wo, b2), dot_xy_rn(wo, n));
+    const f3 vh = normalize_rn(mk(mul_rn(alpha, lo.x), mul_rn(alpha, lo.y), lo.z));
+    const float lensq = fma_rn(vh.x, vh.x, mul_rn(vh.y, vh.y));
+    f3 t1v = lensq > 0.0f ? scale_rn(mk(-vh.y, vh.x, 0.0f), rsqrtf(lensq)) : mk(1.0f, 0.0f, 0.0f);
+    const f3 t2v = cross_rn(vh, t1v);
     float sp, cp;
     sincospif(2.0f * u1, &sp, &cp);
     const float r = sqrtf(u0);
-    const float t1 = r * cp;
-    float t2 = r * sp;
-    const float s = 0.5f * (1.0f + vh.z);
-    t2 = (1.0f - s) * sqrtf(1.0f - t1 * t1) + s * t2;
-    const float tz = sqrtf(fmaxf(0.0f, 1.0f - t1 * t1 - t2 * t2));
-    const f3 nh = t1v * t1 + t2v * t2 + vh * tz;
-    const f3 hl = normalize(mk(alpha * nh.x, alpha * nh.y, fmaxf(nh.z, 0.0f)));
-    const f3 h = b1 * hl.x + b2 * hl.y + n * hl.z;
-    const float voh = dot(wo, h);
-    return h * (2.0f * voh) - wo;
+    const float t1 = mul_rn(r, cp);
+    float t2 = mul_rn(r, sp);
+    const float s = mul_rn(0.5f, add_rn(1.0f, vh.z));
+    const float q1 = fma_rn(-t1, t1, 1.0f);
+    t2 = fma_rn(sub_rn(1.0f, s), sqrtf(q1), mul_rn(s, t2));
+    const float tz = sqrtf(fmaxf(0.0f, fma_rn(-t2, t2, q1)));
+    const f3 nh = combine_rn(t1v, t1, t2v, t2, vh, tz);
+    const f3 hl = normalize_rn(mk(mul_rn(alpha, nh.x), mul_rn(alpha, nh.y), fmaxf(nh.z, 0.0f)));
+    const f3 h = combine_rn(b1, hl.x, b2, hl.y, n, hl.z);
+    const float voh = dot_rn(wo, h);
+    return fma_rn(h, mul_rn(2.0f, voh), mk(-wo.x, -wo.y, -wo.z));
 }
 
+// the half vector, formed as pdf_ggx forms it
+__device__ __forceinline__ f3 half_vector(f3 wi, f3 wo) { return normalize_xy_rn(add_rn(wi, wo)); }
+
 __device__ __forceinline__ float pdf_ggx(f3 n, f3 wo, float co, float a2, float g1o, f3 wi) {
-    f3 h = wi + wo;
-    const float l2 = dot(h, h);
+    f3 h = add_rn(wi, wo);
+    const float l2 = dot_xy_rn(h, h);
     if (!(l2 > 0.0f)) return 0.0f;
-    h = h * rsqrtf(l2);
-    if (!(dot(wo, h) > 0.0f)) return 0.0f;
-    return g1o * ggx_D(dot(n, h), sin2_between(n, h), a2) / (4.0f * co);
+    h = scale_rn(h, rsqrtf(l2));
+    if (!(dot_rn(wo, h) > 0.0f)) return 0.0f;
+    return mul_rn(g1o, ggx_D(dot_rn(n, h), sin2_between(n, h), a2)) / mul_rn(4.0f, co);
 }
 
 __device__ __forceinline__ float schlick_weight(float vh) {
@@ -663,19 +679,19 @@ struct Pixel {
 
 __device__ __forceinline__ bool load_pixel(float4 pos, float4 nrm, float4 kd, float4 korm, f3 cam, Pixel* px) {
     const f3 N = xyz(nrm);
-    const float l2 = dot(N, N);
+    const float l2 = dot_rn(N, N);
     if (!(pos.w > 0.0f) || !(l2 > 0.0f)) return false;
     px->lN = sqrtf(l2);
-    px->n = N * (1.0f / px->lN);
+    px->n = scale_rn(N, 1.0f / px->lN);
     px->p = xyz(pos);
-    px->wo = normalize(cam - px->p);
-    px->co = dot(px->n, px->wo);
+    px->wo = normalize_xy_rn(mk(sub_rn(cam.x, px->p.x), sub_rn(cam.y, px->p.y), sub_rn(cam.z, px->p.z)));
+    px->co = dot_rn(px->n, px->wo);
     px->spec_on = px->co >= 1e-4f;
     px->r = korm.y;
     px->m = korm.z;
-    px->alpha = fmaxf(px->r * px->r, 1e-4f);
-    px->a2 = px->alpha * px->alpha;
-    px->g1o = px->spec_on ? 1.0f / (1.0f + ggx_lambda(px->co, px->a2)) : 0.0f;
+    px->alpha = fmaxf(mul_rn(px->r, px->r), 1e-4f);
+    px->a2 = mul_rn(px->alpha, px->alpha);
+    px->g1o = px->spec_on ? 1.0f / add_rn(1.0f, ggx_lambda(px->co, px->a2)) : 0.0f;
     px->kd = xyz(kd);
     px->F0 = fresnel0(px->kd, px->m);
     frame(px->n, &px->b1, &px->b2);
@@ -685,6 +701,7 @@ __device__ __forceinline__ bool load_pixel(float4 pos, float4 nrm, float4 kd, fl
 // One sample of the MIS estimator: direction, texel and 1/denominator.
 // Returns false when the sample does not contribute (technique off, below the
 // horizon, zero density).
+template <bool kAdjoint = false>
 __device__ __forceinline__ bool draw_sample(const Probe& P, const Pixel& px, int n_light, int n_cos, int n_ggx,
                                             int j, float2 u, f3* wi, int* texel, float* ci, float* inv_denom) {
     float pl = 0.0f, st = 0.0f;
@@ -695,16 +712,17 @@ __device__ __forceinline__ bool draw_sample(const Probe& P, const Pixel& px, int
         *wi = sample_cosine(px.n, px.b1, px.b2, u.x, u.y);
     } else {
         if (!px.spec_on) return false;
-        *wi = sample_ggx(px.n, px.b1, px.b2, px.wo, px.alpha, u.x, u.y);
+        *wi = sample_ggx<kAdjoint>(px.n, px.b1, px.b2, px.wo, px.alpha, u.x, u.y);
     }
-    const float c = dot(px.n, *wi);
+    const float c = dot_xy_rn(px.n, *wi);
     if (!(c > 0.0f)) return false;
     if (t < 0) {
         t = texel_of_dir(P, *wi, &st);
         pl = pdf_light_texel(P, t, st);
     }
-    float denom = (float)n_light * pl + (float)n_cos * (c * MCDI_INV_PI);
-    if (px.spec_on && n_ggx > 0) denom += (float)n_ggx * pdf_ggx(px.n, px.wo, px.co, px.a2, px.g1o, *wi);
+    float denom = fma_rn((float)n_cos, mul_rn(c, MCDI_INV_PI), mul_rn((float)n_light, pl));
+    if (px.spec_on && n_ggx > 0)
+        denom = fma_rn((float)n_ggx, pdf_ggx(px.n, px.wo, px.co, px.a2, px.g1o, *wi), denom);
     if (!(denom > 0.0f)) return false;
     *texel = t;
     *ci = c;

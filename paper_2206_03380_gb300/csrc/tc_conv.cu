@@ -41,6 +41,15 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map
         : "memory");
 }
 
+__device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, int c3,
+                                            int c4, uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
+        "%5, %6}], [%7];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(bar)
+        : "memory");
+}
+
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t bar) {
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
@@ -80,35 +89,18 @@ __host__ __device__ constexpr uint32_t e4m3_idesc(int M, int N) {
     return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-// A-operand collector use: kAPlain reads A from shared memory for this MMA
-// only; kAFill also keeps it in the collector buffer, kAUse takes it from
-// there (same A descriptor), kALast takes it and releases the buffer.
-enum ACollector { kAPlain, kAFill, kAUse, kALast };
-
-#define MCDI_MMA(KIND, COLL)                                                                       \
+#define MCDI_MMA(KIND)                                                                         \
     asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"                             \
-                 "tcgen05.mma.cta_group::1.kind::" KIND COLL " [%0], %1, %2, %3, p;\n\t}" ::"r"(d), \
-                 "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum)                                    \
+                 "tcgen05.mma.cta_group::1.kind::" KIND " [%0], %1, %2, %3, p;\n\t}" ::"r"(d), \
+                 "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum)                                \
                  : "memory")
 
-template <bool FP8, int COLL = kAPlain>
+template <bool FP8>
 __device__ __forceinline__ void mma_issue(uint32_t d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accum) {
-    if constexpr (FP8) {
-        if constexpr (COLL == kAFill) MCDI_MMA("f8f6f4", ".collector::a::fill");
-        else if constexpr (COLL == kAUse) MCDI_MMA("f8f6f4", ".collector::a::use");
-        else if constexpr (COLL == kALast) MCDI_MMA("f8f6f4", ".collector::a::lastuse");
-        else MCDI_MMA("f8f6f4", "");
-    } else {
-        if constexpr (COLL == kAFill) MCDI_MMA("f16", ".collector::a::fill");
-        else if constexpr (COLL == kAUse) MCDI_MMA("f16", ".collector::a::use");
-        else if constexpr (COLL == kALast) MCDI_MMA("f16", ".collector::a::lastuse");
-        else MCDI_MMA("f16", "");
-    }
+    if constexpr (FP8) MCDI_MMA("f8f6f4");
+    else MCDI_MMA("f16");
 }
 #undef MCDI_MMA
-
-
-
 
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* v) {
     asm volatile(
@@ -409,21 +401,28 @@ __global__ void __launch_bounds__(kConvThreads) conv_tc_kernel(const __grid_cons
 // ---------------------------------------------------------------------------
 // Row-tile form, for images at least 48 pixels wide (128-pixel row tiles).
 // A persistent CTA keeps a slice of Nc output channels of the layer's weights
-// resident in shared memory for its whole life ([chunk][tap][Nc][16 ch],
+// resident in shared memory for its whole life ([chunk][dx][dy][Nc][16 ch],
 // 32-byte swizzle, one TMA load per chunk) and loops over tiles of R output
 // rows x 128 pixels.  Per 16-channel input chunk the tile's halo, R + 2 rows x
 // 130 pixels of two 8-channel planes, arrives once: each halo row is one
 // contiguous run in the planar activation layout, copied with one bulk copy
-// (large requests instead of one per 16-byte pixel), the part outside the
-// image zero-filled.  Rows are 16 bytes per pixel and unswizzled, so any row
-// starts a valid 8-row core matrix: the A operand of output row r and tap
-// (dy, dx) is the window starting at halo row (r + dy) * 130 + dx, and 9 R
-// MMAs (M = 128, N = Nc, K = 16) per chunk read (R + 2) / R input rows per
-// output row instead of 9.
+// (large requests instead of one per 16-byte pixel), as are the zeros of the
+// rows and columns beside the image.  Rows are 16 bytes per pixel and
+// unswizzled, so any row starts a valid 8-row core matrix: the A operand of
+// output row r and tap (dy, dx) is the window starting at halo row
+// (r + dy) * 130 + dx, and MMAs (M = 128, N = up to 3 Nc, K = 16) over
+// (R + 2) / R input rows per output row do the chunk (issue_chunk).
 //   warp 0          weight TMA (lane 0), halo row copies (one lane per row),
-//   warp 1 lane 0   MMA issuer; accumulators of tile i in TMEM buffer i & 1,
+//   warp 1          MMA issue (one elected lane); accumulators of tile i in
+//                   TMEM buffer i & 1,
 //   warps 2..9      epilogue: TMEM lane quarter warp % 4, and the two warps of
 //                   a quarter take alternate 16-column chunks of each row.
+// Compiled per rows R, operand type and epilogue (RowMode), so that each
+// epilogue holds only its own registers: with all in one kernel chosen at run
+// time they spilled, and the spills' write-through was most of the L2 writes.
+// Measured, sixteen 800 x 800 images: forward 3.64 -> 2.58 ms, input gradient
+// 4.45 -> 3.70 ms; two 512 x 512: 289 -> 231 and 334 -> 278 us.  At the full
+// resolution the layers run at 50 to 75% of the DRAM rate.
 constexpr int kRowThreads = 320;
 constexpr int kEpiWarps = kRowThreads / 32 - 2;
 constexpr int kEpiSplit = kEpiWarps / 4;  // epilogue warps per TMEM lane quarter
@@ -431,10 +430,192 @@ constexpr int kRowMaxStages = 6;
 constexpr int kHaloW = 130;
 constexpr int kMaxRows = 4;
 
+__device__ __align__(16) uint8_t g_zeros[kHaloW * 16];  // source of the halo's zeros
 
-// EV: the epilogue variant, 0 plain, 1 also the 2x2 max-pool of the output (kStore), 2 the pool
-// gradient routed through the pool (kDgradPoolBwd)
-template <int R, bool FP8, bool MP, int EV>
+
+// ---- epilogue of the row-tile form: 16 accumulator columns of one pixel, as
+// packed BF16 pairs (rounding before the ReLU or the mask gives what rounding
+// after it would).
+enum RowMode {  // what the kernel is compiled for: a ConvEpilogue, or kStore that also writes the 2x2 max-pool
+    kRowStore = kStore, kRowUp2 = kStoreUp2, kRowF32 = kStoreF32, kRowMask = kDgradMask, kRowPlain = kDgradPlain,
+    kRowPoolBwd = kDgradPoolBwd, kRowPool = 6
+};
+
+__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&h);
+}
+__device__ __forceinline__ __nv_bfloat162 as_bf162(uint32_t w) { return *reinterpret_cast<const __nv_bfloat162*>(&w); }
+__device__ __forceinline__ uint32_t max_bf16(uint32_t a, uint32_t b) {
+    const __nv_bfloat162 m = __hmax2(as_bf162(a), as_bf162(b));
+    return *reinterpret_cast<const uint32_t*>(&m);
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+    float2 r;
+    asm("{\n\t.reg .b64 ra, rb, rd;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
+        "add.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+
+// accumulators (times dq for E4M3 operands) plus bias, rounded to BF16
+template <bool FP8>
+__device__ __forceinline__ void bias_pack16(const uint32_t* v, float dq, const float* bias, uint32_t* h) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float4 b = *reinterpret_cast<const float4*>(bias + 4 * i);
+        const float x0 = __uint_as_float(v[4 * i]), x1 = __uint_as_float(v[4 * i + 1]);
+        const float x2 = __uint_as_float(v[4 * i + 2]), x3 = __uint_as_float(v[4 * i + 3]);
+        if constexpr (FP8) {
+            h[2 * i] = pack_bf16(__fadd_rn(__fmul_rn(x0, dq), b.x), __fadd_rn(__fmul_rn(x1, dq), b.y));
+            h[2 * i + 1] = pack_bf16(__fadd_rn(__fmul_rn(x2, dq), b.z), __fadd_rn(__fmul_rn(x3, dq), b.w));
+        } else {
+            const float2 s = add2({x0, x1}, {b.x, b.y}), t = add2({x2, x3}, {b.z, b.w});
+            h[2 * i] = pack_bf16(s.x, s.y);
+            h[2 * i + 1] = pack_bf16(t.x, t.y);
+        }
+    }
+}
+template <bool FP8>
+__device__ __forceinline__ void scale_pack16(const uint32_t* v, float dq, uint32_t* h) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const float a = __uint_as_float(v[2 * i]), b = __uint_as_float(v[2 * i + 1]);
+        h[i] = FP8 ? pack_bf16(a * dq, b * dq) : pack_bf16(a, b);
+    }
+}
+// running max |value| of stored BF16 pairs
+__device__ __forceinline__ void fold_amax(uint32_t& am, const uint32_t* h, int n) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+        if (i < n) am = max_bf16(am, h[i] & 0x7fff7fffu);
+}
+__device__ __forceinline__ void publish_amax2(unsigned* out_amax, uint32_t am) {
+    if (out_amax == nullptr) return;
+    const unsigned hi = am & 0xffff0000u, lo = am << 16;  // the two halves as floats' bits (non-negative)
+    const unsigned w = __reduce_max_sync(0xffffffffu, hi > lo ? hi : lo);
+    if ((threadIdx.x & 31) == 0 && w) atomicMax(out_amax, w);
+}
+// 32 bytes (two neighbouring pixels of an 8-channel plane) in one access: whole sectors, half the instructions
+struct Words8 {
+    uint32_t w[8];
+};
+__device__ __forceinline__ void store32(__nv_bfloat16* o, const Words8& v) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(o), "r"(v.w[0]), "r"(v.w[1]),
+                 "r"(v.w[2]), "r"(v.w[3]), "r"(v.w[4]), "r"(v.w[5]), "r"(v.w[6]), "r"(v.w[7])
+                 : "memory");
+}
+__device__ __forceinline__ Words8 load32(const __nv_bfloat16* a) {
+    Words8 v;
+    asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(v.w[0]), "=r"(v.w[1]), "=r"(v.w[2]), "=r"(v.w[3]), "=r"(v.w[4]), "=r"(v.w[5]), "=r"(v.w[6]), "=r"(v.w[7])
+        : "l"(a));
+    return v;
+}
+// two 8-channel groups of one pixel, `hw` pixels apart
+__device__ __forceinline__ void store16(__nv_bfloat16* o, size_t hw, const uint32_t* h) {
+    *reinterpret_cast<uint4*>(o) = make_uint4(h[0], h[1], h[2], h[3]);
+    *reinterpret_cast<uint4*>(o + hw * 8) = make_uint4(h[4], h[5], h[6], h[7]);
+}
+// h where the mask words' values are positive, +0 elsewhere
+__device__ __forceinline__ void apply_mask(uint32_t* h, uint4 a, uint4 b) {
+    const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    const __nv_bfloat162 zero = as_bf162(0u);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) h[i] &= __hgt2_mask(as_bf162(w[i]), zero);
+}
+
+// kRowPoolBwd: the gradient gp (packed pairs of 16 channels) at a pooled pixel, routed to the first maximum of
+// the pooled tensor's 2x2 window `e`, plus the skip gradient `gs`, masked by E > 0, into the window of `o`
+// (all three at the window's first pixel and first 8-channel group; W2, hw2: the full-size row and plane)
+template <bool FP8>
+__device__ __forceinline__ void pool_bwd16(const uint32_t* gp, const __nv_bfloat16* e, const __nv_bfloat16* gs,
+                                           __nv_bfloat16* o, int W2, size_t hw2, uint32_t& am) {
+    auto half = [](uint32_t w, int hi) { return __uint_as_float(hi ? (w & 0xffff0000u) : (w << 16)); };
+#pragma unroll
+    for (int gg = 0; gg < 2; ++gg) {
+        const size_t g0 = gg * hw2 * 8, row = (size_t)W2 * 8;
+        // window pixel k of channel pair j: word 4 (k & 1) + j of row k >> 1
+        const Words8 e0 = load32(e + g0), e1 = load32(e + g0 + row);
+        const Words8 s0 = load32(gs + g0), s1 = load32(gs + g0 + row);
+        Words8 o0, o1;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t ew[4] = {e0.w[j], e0.w[4 + j], e1.w[j], e1.w[4 + j]};
+            const uint32_t sw[4] = {s0.w[j], s0.w[4 + j], s1.w[j], s1.w[4 + j]};
+            float x[4][2];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                float best = half(ew[0], q);
+                int arg = 0;  // the window's first maximum, in window order
+#pragma unroll
+                for (int k = 1; k < 4; ++k) {
+                    const float v = half(ew[k], q);
+                    if (v > best) best = v, arg = k;
+                }
+                const float g = half(gp[4 * gg + j], q);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) x[k][q] = half(sw[k], q) + (arg == k ? g : 0.0f);
+            }
+            uint32_t h[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) h[k] = pack_bf16(x[k][0], x[k][1]) & __hgt2_mask(as_bf162(ew[k]), as_bf162(0u));
+            o0.w[j] = h[0], o0.w[4 + j] = h[1], o1.w[j] = h[2], o1.w[4 + j] = h[3];
+        }
+        store32(o + g0, o0);
+        store32(o + g0 + row, o1);
+        if constexpr (FP8) {
+            fold_amax(am, o0.w, 8);
+            fold_amax(am, o1.w, 8);
+        }
+    }
+}
+
+// The MMAs of one 16-channel chunk (32-byte K-step) of a tile.  Halo row hr at
+// column shift dx is the A window of output rows r = hr - dy for every tap row
+// dy with 0 <= r < R.  Their accumulators lie in descending row order, so those
+// of dy, dy + 1, ... are adjacent columns, and the weights of one dx lie in dy
+// order ([dx][dy][Nc]), so one MMA with up to kStack tap rows stacked on N
+// (kStack Nc <= 256) does them: at M = 128 an MMA costs 32 cycles for reading
+// its A window plus N / 4 for its weights (N / 2 of math above N = 128), so
+// three rows at Nc = 32 take 56 cycles instead of 120.  A tile's first MMA
+// into accumulator r (chunk 0, hr = r, dx = 0, dy = 0) overwrites it and is
+// issued by itself.  Every accumulator adds its taps in the order chunk, dy, dx.
+template <int R, int kStack, bool FP8>
+__device__ __forceinline__ void issue_chunk(uint32_t d0, uint64_t a0, uint64_t b0, int Nc, bool first) {
+    const uint32_t step = (uint32_t)Nc * 2u;  // Nc x 32 bytes per tap, in 16-byte units
+#pragma unroll
+    for (int hr = 0; hr < R + 2; ++hr) {
+        const int lo = hr - R + 1 > 0 ? hr - R + 1 : 0, hi = hr < 2 ? hr : 2;
+#pragma unroll
+        for (int dx = 0; dx < 3; ++dx) {
+            const uint64_t a = a0 + (uint64_t)(hr * kHaloW + dx);
+#pragma unroll
+            for (int dy = lo; dy <= hi; dy += kStack) {  // tap rows dy ... dy + n - 1
+                const int n = hi - dy + 1 < kStack ? hi - dy + 1 : kStack;
+                const uint32_t d = d0 + (uint32_t)((R - 1 - hr + dy) * Nc);
+                const uint64_t b = b0 + (uint64_t)((uint32_t)(dx * 3 + dy) * step);
+                const uint32_t idesc = FP8 ? e4m3_idesc(128, n * Nc) : bf16_idesc(128, n * Nc);
+                if (dx == 0 && dy == 0 && hr < R) {
+                    if (n == 1) {
+                        mma_issue<FP8>(d, a, b, idesc, first ? 0u : 1u);
+                    } else if (first) {
+                        mma_issue<FP8>(d, a, b, FP8 ? e4m3_idesc(128, Nc) : bf16_idesc(128, Nc), 0u);
+                        mma_issue<FP8>(d + (uint32_t)Nc, a, b + step,
+                                       FP8 ? e4m3_idesc(128, (n - 1) * Nc) : bf16_idesc(128, (n - 1) * Nc), 1u);
+                    } else {
+                        mma_issue<FP8>(d, a, b, idesc, 1u);
+                    }
+                } else {
+                    mma_issue<FP8>(d, a, b, idesc, 1u);
+                }
+            }
+        }
+    }
+}
+
+template <int R, bool FP8, int MODE>
 __global__ void __launch_bounds__(kRowThreads, 2) conv_tc_rows_kernel(const __grid_constant__ CUtensorMap tmap_wh,
                                                                    const ConvParams p, const RowPlan rp) {
     // The setup that reads nothing the preceding kernel writes (barriers, bias, tensor memory and the
@@ -442,7 +623,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) conv_tc_rows_kernel(const __gr
     // overlaps the preceding kernel's tail when the launch is programmatically dependent.
     pdl_allow_dependents();
     extern __shared__ uint8_t smem_raw[];
-    __shared__ float s_bias[256];
+    __shared__ __align__(16) float s_bias[256];
     __shared__ __align__(8) uint64_t full_bar[kRowMaxStages], empty_bar[kRowMaxStages], accf_bar[2], acce_bar[2],
         w_bar;
     __shared__ uint32_t tmem_slot;
@@ -497,65 +678,57 @@ __global__ void __launch_bounds__(kRowThreads, 2) conv_tc_rows_kernel(const __gr
     if (warp == 0 && has_work && lane == 0) {
         const uint32_t wb = smem_u32(&w_bar);
         mbar_expect_tx(wb, (uint32_t)n_chunks * w_chunk);
-        for (int c = 0; c < n_chunks; ++c) tma_load_4d(wbase + (uint32_t)c * w_chunk, &tmap_wh, 0, n0, 0, c, wb);
+        for (int c = 0; c < n_chunks; ++c) tma_load_5d(wbase + (uint32_t)c * w_chunk, &tmap_wh, 0, n0, 0, 0, c, wb);
         w_issued = true;
     }
     pdl_wait();  // activations, masks and outputs: after the preceding kernel has completed
     if (warp == 0) {
         if (has_work) {
             // Halo rows by plain bulk copies: lane l < 2 (R + 2) owns row l % (R + 2)
-            // of plane l / (R + 2); the part of the row outside the image is
-            // zero-filled with shared-memory stores made visible to the async
-            // proxy before the stage's barrier is armed.
+            // of plane l / (R + 2).  What lies outside the image is copied from a run
+            // of zeros: a whole row above or below it, or the column beside its first
+            // or last pixel (further columns reach only outputs outside the image).
             const int rows = R + 2;
             const bool mine = lane < 2 * rows;
             const int q = lane / rows, hr = lane - q * rows;
             const size_t plane_bytes = (size_t)p.H * p.W * 16;
             const uint8_t* x_bytes = reinterpret_cast<const uint8_t*>(p.x);
+            auto copy = [&](uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+                asm volatile(
+                    "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+                    "l"(src), "r"(bytes), "r"(bar)
+                    : "memory");
+            };
             int g = 0;
             for (int t = first; t < rp.n_tiles; t += step) {
                 int img, x0, y0;
                 tile_origin(t, &img, &x0, &y0);
                 const int y = y0 - 1 + hr;
-                const int xa = x0 - 1 < 0 ? 0 : x0 - 1, xb = x0 + 129 > p.W ? p.W : x0 + 129;
-                const bool row_in = mine && y >= 0 && y < p.H && xb > xa;
-                const uint32_t n_bytes = row_in ? (uint32_t)(xb - xa) * 16u : 0u;
-                const int lead = row_in ? xa - (x0 - 1) : kHaloW;  // zero pixels [0, lead)
-                const int tail = row_in ? xb - (x0 - 1) : kHaloW;  // zero pixels [tail, 130)
-                const uint32_t total = __reduce_add_sync(0xffffffffu, n_bytes);
+                const bool row_in = mine && y >= 0 && y < p.H;
+                const int xa = x0 > 0 ? x0 - 1 : 0, xb = x0 + 129 > p.W ? p.W : x0 + 129;  // columns in the image
+                const bool left = x0 == 0, right = xb < x0 + 129;                          // columns -1 and W
+                const uint32_t n_bytes = row_in ? (uint32_t)(xb - xa) * 16u : (mine ? (uint32_t)kHaloW * 16u : 0u);
+                const uint32_t edge = row_in ? ((left ? 16u : 0u) + (right ? 16u : 0u)) : 0u;
+                const uint32_t total = __reduce_add_sync(0xffffffffu, n_bytes + edge);
+                const uint8_t* src0 = x_bytes + (size_t)(img * (p.cin_bytes >> 4) + q) * plane_bytes + ((size_t)y * p.W + xa) * 16;
+                const uint32_t row0 = base + (uint32_t)q * rp.plane_bytes + (uint32_t)hr * (uint32_t)kHaloW * 16u;
                 int c = 0;
                 for (; c < n_chunks; ++c, ++g) {
                     const int s = g % S;
-                    int ok = 1;
-                    if (lane == 0) ok = mbar_wait(smem_u32(&empty_bar[s]), ((uint32_t)(g / S) & 1u) ^ 1u) ? 1 : 0;
-                    ok = __shfl_sync(0xffffffffu, ok, 0);
-                    if (!ok) {
-                        if (lane == 0) failed = 1;
+                    if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&empty_bar[s]), ((uint32_t)(g / S) & 1u) ^ 1u))) {
+                        failed = 1;
                         break;
                     }
-                    const uint32_t row_smem = base + (uint32_t)s * rp.stage_bytes + (uint32_t)q * rp.plane_bytes +
-                                              (uint32_t)hr * (uint32_t)kHaloW * 16u;
-                    if (mine) {
-                        for (int x = 0; x < lead; ++x)
-                            asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(row_smem + 16u * x), "r"(0)
-                                         : "memory");
-                        for (int x = tail; x < kHaloW; ++x)
-                            asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(row_smem + 16u * x), "r"(0)
-                                         : "memory");
-                    }
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    __syncwarp();
+                    const uint32_t row_smem = row0 + (uint32_t)s * rp.stage_bytes;
                     const uint32_t fb = smem_u32(&full_bar[s]);
                     if (lane == 0) mbar_expect_tx(fb, total);
                     __syncwarp();
-                    if (n_bytes > 0) {
-                        const uint8_t* src = x_bytes + (size_t)(img * (p.cin_bytes >> 4) + 2 * c + q) * plane_bytes +
-                                             ((size_t)y * p.W + xa) * 16;
-                        asm volatile(
-                            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                                row_smem + 16u * (uint32_t)lead),
-                            "l"(src), "r"(n_bytes), "r"(fb)
-                            : "memory");
+                    if (row_in) {
+                        copy(row_smem + (left ? 16u : 0u), src0 + (size_t)(2 * c) * plane_bytes, n_bytes, fb);
+                        if (left) copy(row_smem, g_zeros, 16u, fb);
+                        if (right) copy(row_smem + (uint32_t)(xb - x0 + 1) * 16u, g_zeros, 16u, fb);
+                    } else if (mine) {
+                        copy(row_smem, g_zeros, n_bytes, fb);
                     }
                     issued = g + 1;
                 }
@@ -564,107 +737,102 @@ __global__ void __launch_bounds__(kRowThreads, 2) conv_tc_rows_kernel(const __gr
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0 && has_work) {
-            const uint32_t idesc = FP8 ? e4m3_idesc(128, Nc) : bf16_idesc(128, Nc);
-            bool ok = mbar_wait(smem_u32(&w_bar), 0u);
+        if (has_work) {  // the whole warp runs the loop, one elected lane issues (elect_one)
+            const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+            const int stack = R == 1 ? 1 : (3 * Nc <= 256 ? 3 : (2 * Nc <= 256 ? 2 : 1));
+            bool ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&w_bar), 0u));
             if (!ok) failed = 1;
             int g = 0, i = 0;
-            for (int t = first; ok && t < rp.n_tiles && !failed; t += step, ++i) {
+            for (int t = first; ok && t < rp.n_tiles; t += step, ++i) {
                 const int b = i & 1;
-                if (!mbar_wait(smem_u32(&acce_bar[b]), ((uint32_t)(i >> 1) & 1u) ^ 1u)) {
+                if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&acce_bar[b]), ((uint32_t)(i >> 1) & 1u) ^ 1u))) {
                     failed = 1;
                     break;
                 }
                 tc_fence_after();
-                const uint32_t d0 = tmem + (uint32_t)(b * R) * rp.acc_stride;
+                const uint32_t d0 = tm + (uint32_t)(b * R * Nc);
                 int c = 0;
                 for (; c < n_chunks; ++c, ++g) {
                     const int s = g % S;
-                    if (!mbar_wait(smem_u32(&full_bar[s]), (uint32_t)(g / S) & 1u)) {
+                    if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&full_bar[s]), (uint32_t)(g / S) & 1u))) {
                         failed = 1;
                         break;
                     }
                     tc_fence_after();
-                    // descriptors of the stage's halo and the chunk's weights; each MMA adds a
-                    // compile-time offset (in 16-byte units) to the start-address field, which
-                    // stays below 2^14 for any shared-memory address
+                    // descriptors of the stage's halo and the chunk's weights; each MMA adds an
+                    // offset (in 16-byte units) to the start-address field, which stays below 2^14
+                    // for any shared-memory address
                     const uint64_t a0 = noswz_desc(base + (uint32_t)s * rp.stage_bytes, rp.plane_bytes);
                     const uint64_t b0 = sw32_desc(wbase + (uint32_t)c * w_chunk);
-                    const uint64_t b_step = (uint64_t)((uint32_t)Nc * 2u);  // Nc x 32 bytes per tap, in 16-byte units
-                    const uint32_t acc0 = c > 0 ? 1u : 0u;
-                    // MMAs grouped by A window: halo row hr and column shift dx feed output rows
-                    // r = hr - dy for every tap row dy with 0 <= r < R, so the window is read from
-                    // shared memory once (collector fill) and reused by the following MMAs.  The
-                    // first MMA into accumulator r of chunk 0 is (hr = r, dx = 0, dy = 0).
-#pragma unroll
-                    for (int hr = 0; hr < R + 2; ++hr) {
-#pragma unroll
-                        for (int dx = 0; dx < 3; ++dx) {
-                            const uint64_t adesc = a0 + (uint64_t)(hr * kHaloW + dx);
-                            const int dy_lo = hr - R + 1 > 0 ? hr - R + 1 : 0, dy_hi = hr < 2 ? hr : 2;
-#pragma unroll
-                            for (int dy = dy_lo; dy <= dy_hi; ++dy) {
-                                const uint32_t d = d0 + (uint32_t)(hr - dy) * rp.acc_stride;
-                                const uint64_t bdesc = b0 + (uint64_t)(dy * 3 + dx) * b_step;
-                                const uint32_t acc = (dx == 0 && dy == 0) ? acc0 : 1u;
-                                if (dy_lo == dy_hi) mma_issue<FP8, kAPlain>(d, adesc, bdesc, idesc, acc);
-                                else if (dy == dy_lo) mma_issue<FP8, kAFill>(d, adesc, bdesc, idesc, acc);
-                                else if (dy == dy_hi) mma_issue<FP8, kALast>(d, adesc, bdesc, idesc, acc);
-                                else mma_issue<FP8, kAUse>(d, adesc, bdesc, idesc, acc);
-                            }
-                        }
+                    if (elect_one()) {
+                        if (stack == 3) issue_chunk<R, 3, FP8>(d0, a0, b0, Nc, c == 0);
+                        else if (stack == 2) issue_chunk<R, 2, FP8>(d0, a0, b0, Nc, c == 0);
+                        else issue_chunk<R, 1, FP8>(d0, a0, b0, Nc, c == 0);
+                        asm volatile(
+                            "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                                smem_u32(&empty_bar[s]))
+                            : "memory");
+                        if (c + 1 == n_chunks)
+                            asm volatile(
+                                "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                                    smem_u32(&accf_bar[b]))
+                                : "memory");
                     }
-                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                                     smem_u32(&empty_bar[s]))
-                                 : "memory");
+                    __syncwarp();
                 }
                 if (c < n_chunks) break;
-                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                                 smem_u32(&accf_bar[b]))
-                             : "memory");
             }
         }
         __syncwarp();
     } else {
         const int q = warp & 3, h = (warp - 2) >> 2;
         const int m = q * 32 + lane;
-        float amax = 0.0f;
+        uint32_t amax = 0, pool_amax = 0;
         // this warp's 16-column chunks of a row: 16 h, 16 (h + kEpiSplit), ...,
         // drained two per TMEM-load wait
         const int cfirst = 16 * h, cstep = 16 * kEpiSplit;
-        // MP (ReLU-masked input gradients with at most 64 channels per CTA): the
-        // mask words of the next row are loaded while the current row drains
-        // (and those of a tile's first row before its accumulator wait), so
-        // their latency does not stall the epilogue
-        const bool pref = MP && p.mode == kDgradMask && Nc <= 2 * cstep;
-        uint4 na0{}, na1{}, nb0{}, nb1{};  // next row's mask words of chunks cfirst (a) and cfirst + cstep (b)
-        auto load_row = [&](int img, int x, int y) {
-            uint4 w[2];
-            if (cfirst < Nc && x < p.W && y < p.H && n0 + cfirst < p.cout_valid) {
-                load_mask16(p, n0 + cfirst, img, x, y, w);
-                na0 = w[0];
-                na1 = w[1];
-            }
-            if (cfirst + cstep < Nc && x < p.W && y < p.H && n0 + cfirst + cstep < p.cout_valid) {
-                load_mask16(p, n0 + cfirst + cstep, img, x, y, w);
-                nb0 = w[0];
-                nb1 = w[1];
-            }
+        const size_t hw = (size_t)p.H * p.W;
+        const size_t pair = (size_t)(cstep >> 3) * hw * 8;  // elements from a chunk's planes to the next one's
+        // ReLU-masked input gradients: the mask words of the tile's rows are loaded before its accumulator wait,
+        // so their latency does not stall the epilogue (chunk cfirst; with at most two rows also the one after)
+        constexpr int kMaskChunks = R <= 2 ? 2 : 1;
+        uint4 mk[MODE == kRowMask ? R : 1][MODE == kRowMask ? kMaskChunks : 1][2];
+        const __nv_bfloat16* mask_px = nullptr;
+        auto load_mask = [&](const __nv_bfloat16* at, uint4* w) {
+            w[0] = __ldg(reinterpret_cast<const uint4*>(at));
+            w[1] = __ldg(reinterpret_cast<const uint4*>(at + hw * 8));
         };
-        // 2x2 max-pool of the stored values: the two pixels of a window are neighbouring
-        // lanes, its two rows consecutive rows of this thread (R even, tiles start on even
-        // rows and columns); the maxima are taken on the stored BF16 values
-        // (EV 1: the instantiation for the convolutions that feed a pooling layer)
-        const bool pool = EV == 1 && R % 2 == 0 && p.pool_out != nullptr && p.mode == kStore && Nc <= 2 * cstep;
-        float pool_amax = 0.0f;
-        uint32_t ha[8], hb[8];  // the even row's stored values of chunks c0 / c1, packed BF16 pairs
         int i = 0;
         for (int t = first; t < rp.n_tiles; t += step, ++i) {
             const int b = i & 1;
             int img, x0, y0;
             tile_origin(t, &img, &x0, &y0);
             const int x = x0 + m;
-            if (pref) load_row(img, x, y0);
+            const bool x_in = x < p.W;
+            // this pixel of the tile's first row in the output's, mask's and skip gradient's first plane
+            // (kRowUp2, kRowPoolBwd: at twice the size)
+            const int up = MODE == kRowUp2 ? 2 : 1, dn = MODE == kRowPoolBwd ? 2 : 1, sc = up * dn;
+            const int Ws = p.W * sc;
+            const size_t hws = hw * (sc * sc);
+            auto first_px = [&](int ctotal, int coff) {
+                return ((((size_t)img * (ctotal >> 3) + ((coff + n0 + cfirst) >> 3)) * (p.H * sc) + y0 * sc) * Ws + x * sc) * 8;
+            };
+            __nv_bfloat16* out_px = MODE == kRowF32 ? nullptr : p.out + first_px(p.out_ctotal, p.out_coff);
+            const __nv_bfloat16* skip_px = nullptr;
+            if (MODE == kRowMask || MODE == kRowPoolBwd) {
+                const size_t at = first_px(p.mask_ctotal, p.mask_coff);
+                mask_px = p.mask + at;
+                if (MODE == kRowPoolBwd) skip_px = p.gskip + at;
+            }
+            const size_t pairs = (size_t)(cstep >> 3) * hws * 8;
+            if constexpr (MODE == kRowMask) {
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+#pragma unroll
+                    for (int k = 0; k < kMaskChunks; ++k)
+                        if (x_in && y0 + r < p.H && cfirst + k * cstep < Nc && n0 + cfirst + k * cstep < p.cout_valid)
+                            load_mask(mask_px + (size_t)k * pair + (size_t)r * p.W * 8, mk[r][k]);
+            }
             const bool ok = mbar_wait(smem_u32(&accf_bar[b]), (uint32_t)(i >> 1) & 1u);
             __syncwarp();
             if (!__all_sync(0xffffffffu, ok)) {
@@ -672,66 +840,101 @@ __global__ void __launch_bounds__(kRowThreads, 2) conv_tc_rows_kernel(const __gr
                 break;
             }
             tc_fence_after();
-            const float dq = dequant_factor(p);
-            constexpr int kRowUnroll = MP || EV != 0 ? 1 : R;  // prefetch / pool registers leave no room to unroll
+            const float dq = FP8 ? dequant_factor(p) : 1.0f;
+            uint32_t ha[8], hb[8];  // kRowPool: the even row's stored values of the two chunks
+            constexpr int kRowUnroll = MODE == kRowPoolBwd ? 1 : R;  // (unrolled it spills)
 #pragma unroll kRowUnroll
             for (int r = 0; r < R; ++r) {
-                const int y = y0 + r;
-                const bool valid = x < p.W && y < p.H;
-                const uint32_t tr = tmem + (uint32_t)(b * R + r) * rp.acc_stride + ((uint32_t)(q * 32) << 16);
-                const uint4 ca0 = na0, ca1 = na1, cb0 = nb0, cb1 = nb1;
-                if (pref && r + 1 < R) load_row(img, x, y + 1);
-                for (int c0 = cfirst; c0 < Nc; c0 += 2 * cstep) {
-                    uint32_t v[32];
+                const bool valid = x_in && y0 + r < p.H;
+                const uint32_t tr = tmem + (uint32_t)((b * R + R - 1 - r) * Nc) + ((uint32_t)(q * 32) << 16);
+                constexpr int kPer = MODE == kRowPoolBwd || MODE == kRowMask ? 1 : 2;  // chunks per TMEM-load wait
+                for (int c0 = cfirst, k = 0; c0 < Nc; c0 += kPer * cstep, k += kPer) {
+                    uint32_t v[16 * kPer];
                     const int c1 = c0 + cstep;
-                    const bool two = c1 < Nc;
+                    const bool two = kPer == 2 && c1 < Nc;
                     tmem_ld16_async(tr + (uint32_t)c0, v);
-                    if (two) tmem_ld16_async(tr + (uint32_t)c1, v + 16);
+                    if constexpr (kPer == 2) {
+                        if (two) tmem_ld16_async(tr + (uint32_t)c1, v + 16);
+                    }
                     tmem_wait_ld();
-                    uint32_t ka[8], kb[8];
                     const bool va = valid && n0 + c0 < p.cout_valid, vb = two && valid && n0 + c1 < p.cout_valid;
-                    if (va) epilogue16<EV == 2>(p, v, n0 + c0, img, x, y, s_bias + c0, dq, &amax, pref, ca0, ca1, ka);
-                    if (vb)
-                        epilogue16<EV == 2>(p, v + 16, n0 + c1, img, x, y, s_bias + c1, dq, &amax, pref, cb0, cb1, kb);
-                    if (pool) {
+                    uint32_t ka[8], kb[8];
+                    auto chunk = [&](const uint32_t* acc, int c, int kk, uint32_t* w) {
+                        if constexpr (MODE == kRowF32) {
+                            float f[3];
+#pragma unroll
+                            for (int j = 0; j < 3; ++j) {
+                                f[j] = __fadd_rn(__fmul_rn(__uint_as_float(acc[j]), dq), s_bias[c + j]);
+                                if (p.relu) f[j] = fmaxf(f[j], 0.0f);
+                            }
+                            p.out_f32[((size_t)img * p.H + y0 + r) * p.W + x] = make_float4(f[0], f[1], f[2], 0.0f);
+                        } else if constexpr (MODE == kRowPoolBwd) {
+                            scale_pack16<FP8>(acc, dq, w);
+                            const size_t at = (size_t)kk * pairs + (size_t)(2 * r) * Ws * 8;
+                            pool_bwd16<FP8>(w, mask_px + at, skip_px + at, out_px + at, Ws, hws, amax);
+                        } else {
+                            if constexpr (MODE == kRowMask || MODE == kRowPlain) {
+                                scale_pack16<FP8>(acc, dq, w);
+                            } else {
+                                bias_pack16<FP8>(acc, dq, s_bias + c, w);
+                                if (p.relu) {
+#pragma unroll
+                                    for (int j = 0; j < 8; ++j) w[j] = max_bf16(w[j], 0u);
+                                }
+                            }
+                            if constexpr (MODE == kRowMask) {
+                                if (kk == 0) {
+                                    apply_mask(w, mk[r][0][0], mk[r][0][1]);
+                                } else if (kMaskChunks == 2 && kk == 1) {
+                                    apply_mask(w, mk[r][kMaskChunks - 1][0], mk[r][kMaskChunks - 1][1]);
+                                } else {
+                                    uint4 mw[2];
+                                    load_mask(mask_px + (size_t)kk * pair + (size_t)r * p.W * 8, mw);
+                                    apply_mask(w, mw[0], mw[1]);
+                                }
+                            }
+                            if constexpr (FP8) fold_amax(amax, w, 8);
+                            __nv_bfloat16* o = out_px + (size_t)kk * pairs + (size_t)(r * up) * Ws * 8;
+                            if constexpr (MODE == kRowUp2) {
+#pragma unroll
+                                for (int gg = 0; gg < 2; ++gg) {
+                                    const uint32_t* u = w + 4 * gg;
+                                    const Words8 two_px = {{u[0], u[1], u[2], u[3], u[0], u[1], u[2], u[3]}};
+                                    store32(o + gg * hws * 8, two_px);
+                                    store32(o + gg * hws * 8 + (size_t)Ws * 8, two_px);
+                                }
+                            } else {
+                                store16(o, hws, w);
+                            }
+                        }
+                    };
+                    if (va) chunk(v, c0, k, ka);
+                    if constexpr (kPer == 2) {
+                        if (vb) chunk(v + 16, c1, k + 1, kb);
+                    }
+                    if constexpr (MODE == kRowPool && R % 2 == 0) {
+                        // 2x2 max-pool of the stored values: a window's two pixels are neighbouring lanes, its two
+                        // rows consecutive rows of this thread (R even, tiles start on even rows and columns)
                         if ((r & 1) == 0) {
 #pragma unroll
-                            for (int k = 0; k < 8; ++k) {
-                                ha[k] = ka[k];
-                                hb[k] = kb[k];
-                            }
+                            for (int j = 0; j < 8; ++j) ha[j] = ka[j], hb[j] = kb[j];
                         } else {
                             const int Hp = p.H >> 1, Wp = p.W >> 1;
-                            auto pool_store = [&](const uint32_t* h, const uint32_t* k, int c, bool ok) {
+                            auto pool_store = [&](const uint32_t* e, const uint32_t* o, int c, bool in) {
                                 uint32_t w[8];
 #pragma unroll
                                 for (int j = 0; j < 8; ++j) {
-                                    __nv_bfloat162 a = *reinterpret_cast<const __nv_bfloat162*>(&h[j]);
-                                    __nv_bfloat162 b = *reinterpret_cast<const __nv_bfloat162*>(&k[j]);
-                                    a = __hmax2(a, b);
-                                    uint32_t u = *reinterpret_cast<uint32_t*>(&a);
-                                    const uint32_t o = __shfl_xor_sync(0xffffffffu, u, 1);
-                                    a = __hmax2(a, *reinterpret_cast<const __nv_bfloat162*>(&o));
-                                    w[j] = *reinterpret_cast<uint32_t*>(&a);
+                                    const uint32_t u = max_bf16(e[j], o[j]);
+                                    w[j] = max_bf16(u, __shfl_xor_sync(0xffffffffu, u, 1));
                                 }
-                                if ((lane & 1) == 0 && ok) {
-                                    __nv_bfloat16* dst = p.pool_out + plane_off(img, p.pool_ctotal >> 3, c >> 3, Hp, Wp,
-                                                                                y >> 1, x >> 1);
-                                    *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
-                                    *reinterpret_cast<uint4*>(dst + (size_t)Hp * Wp * 8) =
-                                        make_uint4(w[4], w[5], w[6], w[7]);
-                                    if (p.pool_amax) {
-#pragma unroll
-                                        for (int j = 0; j < 8; ++j) {
-                                            const float2 f2 = __bfloat1622float2(
-                                                *reinterpret_cast<const __nv_bfloat162*>(&w[j]));
-                                            pool_amax = fmaxf(pool_amax, fmaxf(fabsf(f2.x), fabsf(f2.y)));
-                                        }
-                                    }
+                                if ((lane & 1) == 0 && in) {
+                                    store16(p.pool_out + plane_off(img, p.pool_ctotal >> 3, c >> 3, Hp, Wp, (y0 + r) >> 1, x >> 1),
+                                            (size_t)Hp * Wp, w);
+                                    if constexpr (FP8) fold_amax(pool_amax, w, 8);
                                 }
                             };
                             pool_store(ha, ka, n0 + c0, va);
-                            pool_store(hb, kb, n0 + c1, vb);
+                            if (two) pool_store(hb, kb, n0 + c1, vb);
                         }
                     }
                     __syncwarp();
@@ -741,8 +944,10 @@ __global__ void __launch_bounds__(kRowThreads, 2) conv_tc_rows_kernel(const __gr
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&acce_bar[b]));
         }
-        publish_amax(p.out_amax, amax, 0xffffffffu);
-        if (pool) publish_amax(p.pool_amax, pool_amax, 0xffffffffu);
+        if constexpr (FP8) {
+            publish_amax2(p.out_amax, amax);
+            if (MODE == kRowPool) publish_amax2(p.pool_amax, pool_amax);
+        }
     }
 
     tc_fence_before();
@@ -795,7 +1000,7 @@ const DeviceLimits& device_limits() {
             cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
             cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess ||
             cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev) != cudaSuccess ||
-            cudaFuncGetAttributes(&fa, conv_tc_rows_kernel<4, false, false, 0>) != cudaSuccess ||
+            cudaFuncGetAttributes(&fa, conv_tc_rows_kernel<4, false, kRowStore>) != cudaSuccess ||
             optin <= (int)fa.sharedSizeBytes) {
             L.sms = 0;
             return;
@@ -827,14 +1032,13 @@ bool plan_rows(const ConvParams& p, RowPlan* out) {
     for (int n_slices = 1; 16 * n_slices <= p.cout_pad; ++n_slices) {
         if (p.cout_pad % (16 * n_slices) != 0) continue;
         const int nc = p.cout_pad / n_slices;
-        const uint32_t acc_stride = pow2_at_least((uint32_t)nc);
         const uint32_t w_bytes = (uint32_t)n_chunks * 9u * (uint32_t)nc * 32u;
         // the largest R that fits, except that a plan of two CTAs per SM is
         // preferred to one of a single CTA with a larger R
         RowPlan single{};
         bool have_single = false;
         for (int R = kMaxRows; R >= 1; R >>= 1) {
-            const uint32_t tmem_cols = pow2_at_least(2u * (uint32_t)R * acc_stride);
+            const uint32_t tmem_cols = pow2_at_least(2u * (uint32_t)(R * nc));
             if (tmem_cols > 512u) continue;
             RowPlan rp{};
             rp.rows = R;
@@ -842,7 +1046,6 @@ bool plan_rows(const ConvParams& p, RowPlan* out) {
             rp.n_slices = n_slices;
             rp.plane_bytes = ((uint32_t)(R + 2) * kHaloW * 16u + 127u) & ~127u;
             rp.stage_bytes = (2u * rp.plane_bytes + 1023u) & ~1023u;
-            rp.acc_stride = acc_stride;
             rp.tmem_cols = tmem_cols;
             if (w_bytes + 2u * rp.stage_bytes + kAlign > kSmemMax) continue;
             rp.n_tiles = p.n_img * ((p.H + R - 1) / R) * p.tiles_x;
@@ -943,12 +1146,14 @@ bool conv_make_desc(ConvDesc* d, const void* x, const void* w, const char** why)
         const RowPlan& rp = d->rp;
         d->p.tiles_y = (p.H + rp.rows - 1) / rp.rows;
         // The same K-major weights [cout][tap][cin] viewed as (32 bytes of
-        // channels, cout, tap, chunk): one box lands in shared memory as
-        // [tap][nc][32 B].
-        const cuuint64_t hdims[4] = {32, (cuuint64_t)p.cout_pad, 9, (cuuint64_t)(p.cin_bytes / 32)};
-        const cuuint64_t hstr[3] = {(cuuint64_t)9 * p.cin_bytes, (cuuint64_t)p.cin_bytes, 32};
-        const cuuint32_t hwbox[4] = {32, (cuuint32_t)rp.nc, 9, 1};
-        r = enc(&d->tmap_wh, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, const_cast<void*>(w), hdims, hstr, hwbox, ones,
+        // channels, cout, tap row dy, tap column dx, chunk): one box lands in
+        // shared memory as [dx][dy][nc][32 B].
+        const cuuint64_t tap = (cuuint64_t)p.cin_bytes;
+        const cuuint64_t hdims[5] = {32, (cuuint64_t)p.cout_pad, 3, 3, (cuuint64_t)(p.cin_bytes / 32)};
+        const cuuint64_t hstr[4] = {9 * tap, 3 * tap, tap, 32};
+        const cuuint32_t hwbox[5] = {32, (cuuint32_t)rp.nc, 3, 3, 1};
+        const cuuint32_t ones5[5] = {1, 1, 1, 1, 1};
+        r = enc(&d->tmap_wh, CU_TENSOR_MAP_DATA_TYPE_UINT8, 5, const_cast<void*>(w), hdims, hstr, hwbox, ones5,
                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (r != CUDA_SUCCESS) {
@@ -959,25 +1164,23 @@ bool conv_make_desc(ConvDesc* d, const void* x, const void* w, const char** why)
     return true;
 }
 
-template <bool FP8, bool MP, int EV>
-static void set_rows_smem(int bytes, cudaError_t* err) {
-    const void* fs[3] = {(const void*)conv_tc_rows_kernel<1, FP8, MP, EV>,
-                         (const void*)conv_tc_rows_kernel<2, FP8, MP, EV>,
-                         (const void*)conv_tc_rows_kernel<4, FP8, MP, EV>};
-    for (const void* f : fs)
-        if (*err == cudaSuccess && bytes > 0)
-            *err = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+template <int R, bool FP8>
+static const void* rows_kernel(int mode) {
+    switch (mode) {
+        case kRowUp2: return (const void*)conv_tc_rows_kernel<R, FP8, kRowUp2>;
+        case kRowF32: return (const void*)conv_tc_rows_kernel<R, FP8, kRowF32>;
+        case kRowMask: return (const void*)conv_tc_rows_kernel<R, FP8, kRowMask>;
+        case kRowPlain: return (const void*)conv_tc_rows_kernel<R, FP8, kRowPlain>;
+        case kRowPoolBwd: return (const void*)conv_tc_rows_kernel<R, FP8, kRowPoolBwd>;
+        case kRowPool: return (const void*)conv_tc_rows_kernel<(R > 1 ? R : 2), FP8, kRowPool>;  // planned for even R only
+        default: return (const void*)conv_tc_rows_kernel<R, FP8, kRowStore>;
+    }
 }
 
-template <bool FP8, bool MP, int EV>
-static void launch_rows(const ConvDesc& d, cudaStream_t stream) {
-    const dim3 g(d.rp.grid), t(kRowThreads);
-    const size_t sm = d.rp.smem_bytes;
-    if (d.rp.rows == 4)
-        launch_k_dependent(conv_tc_rows_kernel<4, FP8, MP, EV>, g, t, sm, stream, d.tmap_wh, d.p, d.rp);
-    else if (d.rp.rows == 2)
-        launch_k_dependent(conv_tc_rows_kernel<2, FP8, MP, EV>, g, t, sm, stream, d.tmap_wh, d.p, d.rp);
-    else launch_k_dependent(conv_tc_rows_kernel<1, FP8, MP, EV>, g, t, sm, stream, d.tmap_wh, d.p, d.rp);
+static const void* rows_kernel(int rows, bool fp8, int mode) {
+    if (rows == 4) return fp8 ? rows_kernel<4, true>(mode) : rows_kernel<4, false>(mode);
+    if (rows == 2) return fp8 ? rows_kernel<2, true>(mode) : rows_kernel<2, false>(mode);
+    return fp8 ? rows_kernel<1, true>(mode) : rows_kernel<1, false>(mode);
 }
 
 bool conv_mask_prefetch(const ConvDesc& d) { return d.rows_form && d.p.mode == kDgradMask && d.rp.nc <= 64; }
@@ -993,32 +1196,19 @@ cudaError_t conv_launch(const ConvDesc& d, cudaStream_t stream) {
         for (const void* f : generic)
             if (attr_err == cudaSuccess)
                 attr_err = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, tile);
-        set_rows_smem<false, false, 0>(lim, &attr_err);
-        set_rows_smem<true, false, 0>(lim, &attr_err);
-        set_rows_smem<false, true, 0>(lim, &attr_err);
-        set_rows_smem<true, true, 0>(lim, &attr_err);
-        set_rows_smem<false, false, 1>(lim, &attr_err);
-        set_rows_smem<true, false, 1>(lim, &attr_err);
-        set_rows_smem<false, false, 2>(lim, &attr_err);
-        set_rows_smem<true, false, 2>(lim, &attr_err);
+        for (int rows : {1, 2, 4})
+            for (int mode = 0; mode <= kRowPool; ++mode)
+                for (bool fp8 : {false, true})
+                    if (attr_err == cudaSuccess)
+                        attr_err = cudaFuncSetAttribute(rows_kernel(rows, fp8, mode),
+                                                        cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     });
     if (attr_err != cudaSuccess) return attr_err;
     if (d.rows_form) {
-        // masked input gradients whose mask words fit the prefetch registers take the prefetching variant
-        const bool mp = conv_mask_prefetch(d);
-        const bool pl = d.p.pool_out != nullptr;  // conv_make_desc keeps it only where the plan can pool
-        const bool pb = d.p.mode == kDgradPoolBwd;
-        if (d.p.fp8) {
-            if (mp) launch_rows<true, true, 0>(d, stream);
-            else if (pl) launch_rows<true, false, 1>(d, stream);
-            else if (pb) launch_rows<true, false, 2>(d, stream);
-            else launch_rows<true, false, 0>(d, stream);
-        } else {
-            if (mp) launch_rows<false, true, 0>(d, stream);
-            else if (pl) launch_rows<false, false, 1>(d, stream);
-            else if (pb) launch_rows<false, false, 2>(d, stream);
-            else launch_rows<false, false, 0>(d, stream);
-        }
+        const int mode = d.p.pool_out != nullptr ? (int)kRowPool : d.p.mode;  // run_conv pools only where the plan can
+        using Kernel = void(const CUtensorMap, const ConvParams, const RowPlan);
+        auto* kernel = reinterpret_cast<Kernel*>(const_cast<void*>(rows_kernel(d.rp.rows, d.p.fp8 != 0, mode)));
+        launch_k_dependent(kernel, dim3(d.rp.grid), dim3(kRowThreads), d.rp.smem_bytes, stream, d.tmap_wh, d.p, d.rp);
         return cudaGetLastError();
     }
     const int n_tiles = d.p.n_img * d.p.tiles_y * d.p.tiles_x;

@@ -67,7 +67,6 @@ struct RowPlan {
     int grid;                // CTAs (a multiple of n_slices)
     uint32_t plane_bytes;    // halo plane stride in shared memory: (R + 2) rows x 130 pixels x 16 bytes, 128-aligned
     uint32_t stage_bytes;    // two planes, 1024-byte aligned
-    uint32_t acc_stride;     // TMEM columns between the accumulators of two rows
     uint32_t tmem_cols;      // TMEM columns allocated (two buffers of R accumulators)
     uint32_t smem_bytes;     // dynamic shared memory
 };
@@ -76,7 +75,7 @@ struct RowPlan {
 struct ConvDesc {
     CUtensorMap tmap_x;
     CUtensorMap tmap_w;
-    CUtensorMap tmap_wh;  // row-tile form: one 16-channel chunk of all 9 taps' weights, [tap][nc][16]
+    CUtensorMap tmap_wh;  // row-tile form: one 16-channel chunk of all 9 taps' weights, [dx][dy][nc][16]
     bool rows_form;
     RowPlan rp;
     ConvParams p;
@@ -93,8 +92,8 @@ bool conv_make_desc(ConvDesc* d, const void* x, const void* w, const char** why)
 // Runs the persistent row-tile kernel when planned, else one CTA per tile.
 cudaError_t conv_launch(const ConvDesc& d, cudaStream_t stream);
 
-// Whether conv_launch runs the row-tile variant that prefetches the ReLU-mask
-// words of the next row (masked input gradients whose mask words fit its registers).
+// Whether conv_launch runs the row-tile form with ReLU-mask words loaded ahead of the
+// accumulators (masked input gradients with at most 64 channels per CTA).
 bool conv_mask_prefetch(const ConvDesc& d);
 
 // Tensor map over BF16 8-channel planes [plane][H][W][16 B] (n_planes =

@@ -48,6 +48,17 @@ static __device__ bool mbar_wait(uint32_t bar, uint32_t parity) {
     }
 }
 
+// One lane of the (converged) warp, the same one every time.  MMAs are issued
+// under it from code that the whole warp runs: their descriptors then stay in
+// uniform registers.  Issued by a thread picked by its index they are moved
+// there one by one, 45 cycles per instruction, more than the instruction's own
+// 40 at M = 128, N = 32.
+static __device__ __forceinline__ bool elect_one() {
+    uint32_t ok;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(ok));
+    return ok != 0;
+}
+
 static __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 
 static __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }

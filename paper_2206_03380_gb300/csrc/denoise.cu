@@ -491,7 +491,7 @@ static cudaError_t run_conv(Unet& u, int level, const bf16* x, int x_slot, int c
         d.p.w_amax = reinterpret_cast<const float*>(u.wbase + u.L.amax) + w.i;
     }
     if (!conv_make_desc(&d, xin, win, why)) return cudaErrorInvalidValue;
-    if (pool.out && d.rows_form && d.rp.rows % 2 == 0 && d.rp.nc <= 64 && mode == kStore) {
+    if (pool.out && mode == kStore && (d.halo_form || (d.rows_form && d.rp.rows % 2 == 0 && d.rp.nc <= 64))) {
         d.p.pool_out = pool.out;
         d.p.pool_ctotal = pool.ctotal;
         d.p.pool_amax = u.out(pool.slot);

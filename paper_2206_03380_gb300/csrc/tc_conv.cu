@@ -1,6 +1,8 @@
-// tcgen05 implicit-GEMM 3x3 convolution (see tc_conv.cuh).
+// tcgen05 implicit-GEMM 3x3 convolution (see tc_conv.cuh): the row-tile form for
+// images at least 48 pixels wide, the halo-tile form for narrower ones, and for
+// layers neither can hold in shared memory the general form below.
 //
-// One CTA computes a tile of 128 output pixels (tw x th) for all output
+// General form: one CTA computes a tile of 128 output pixels (tw x th) for all output
 // channels: D[128 x cout_pad] (FP32, in tensor memory) = sum over the 9 taps
 // and over input-channel chunks of 16 of
 //   A[128 pixels x 16 ch] (the input shifted by the tap, zero outside the
@@ -50,6 +52,16 @@ __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* map
         : "memory");
 }
 
+// coordinates (2 x, y, plane) of a plane-row map (8-byte elements, two per pixel)
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2,
+                                            uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
+        "[%5];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(bar)
+        : "memory");
+}
+
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t bar) {
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
@@ -80,6 +92,16 @@ __device__ __forceinline__ uint64_t noswz_desc(uint32_t saddr, uint32_t lbo) {
     d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
     d |= (uint64_t)(128u >> 4) << 32;
     d |= (uint64_t)1 << 46;  // descriptor version; swizzle mode 0 (none)
+    return d;
+}
+
+// The same with 8-row groups `sbo` bytes apart.
+__device__ __forceinline__ uint64_t rows_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
+    uint64_t d = 0;
+    d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
+    d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
+    d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
+    d |= (uint64_t)1 << 46;
     return d;
 }
 
@@ -267,7 +289,7 @@ template <bool FP8, bool PB>
 __global__ void __launch_bounds__(kConvThreads) conv_tc_kernel(const __grid_constant__ CUtensorMap tmap_x,
                                                                const __grid_constant__ CUtensorMap tmap_w,
                                                                const ConvParams p) {
-    pdl_prologue();
+    pdl_wait();
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[kStages], empty_bar[kStages], acc_bar;
     __shared__ uint32_t tmem_slot;
@@ -309,6 +331,7 @@ __global__ void __launch_bounds__(kConvThreads) conv_tc_kernel(const __grid_cons
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
+    pdl_allow_dependents();  // every CTA holds its tensor memory by then
 
     int issued = 0;
     if (warp == 0 && lane == 0) {
@@ -572,6 +595,57 @@ __device__ __forceinline__ void pool_bwd16(const uint32_t* gp, const __nv_bfloat
     }
 }
 
+// The rest of 16 accumulator columns of one pixel, except for kRowF32: packed (left in w), activated or masked
+// (m0, m1: the mask words), folded into amax and stored at `out` (this pixel in the first of the two planes;
+// kRowUp2, kRowPoolBwd: its 2x2 block at twice the size; Ws, hws: row and plane of the output).
+template <int MODE, bool FP8>
+__device__ __forceinline__ void finish16(const ConvParams& p, const uint32_t* acc, float dq, const float* bias16,
+                                         uint4 m0, uint4 m1, const __nv_bfloat16* pooled, const __nv_bfloat16* skip,
+                                         __nv_bfloat16* out, int Ws, size_t hws, uint32_t* w, uint32_t& amax) {
+    if constexpr (MODE == kRowPoolBwd) {
+        scale_pack16<FP8>(acc, dq, w);
+        pool_bwd16<FP8>(w, pooled, skip, out, Ws, hws, amax);
+    } else {
+        if constexpr (MODE == kRowMask || MODE == kRowPlain) {
+            scale_pack16<FP8>(acc, dq, w);
+        } else {
+            bias_pack16<FP8>(acc, dq, bias16, w);
+            if (p.relu) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) w[j] = max_bf16(w[j], 0u);
+            }
+        }
+        if constexpr (MODE == kRowMask) apply_mask(w, m0, m1);
+        if constexpr (FP8) fold_amax(amax, w, 8);
+        if constexpr (MODE == kRowUp2) {
+#pragma unroll
+            for (int gg = 0; gg < 2; ++gg) {
+                const uint32_t* u = w + 4 * gg;
+                const Words8 two_px = {{u[0], u[1], u[2], u[3], u[0], u[1], u[2], u[3]}};
+                store32(out + gg * hws * 8, two_px);
+                store32(out + gg * hws * 8 + (size_t)Ws * 8, two_px);
+            }
+        } else {
+            store16(out, hws, w);
+        }
+    }
+}
+// kRowF32: channels 0..2 of one pixel
+__device__ __forceinline__ void finish_f32(const ConvParams& p, const uint32_t* acc, float dq, const float* bias,
+                                           size_t px) {
+    float f[3];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        f[j] = __fadd_rn(__fmul_rn(__uint_as_float(acc[j]), dq), bias[j]);
+        if (p.relu) f[j] = fmaxf(f[j], 0.0f);
+    }
+    p.out_f32[px] = make_float4(f[0], f[1], f[2], 0.0f);
+}
+__device__ __forceinline__ void load_mask_words(const __nv_bfloat16* at, size_t hw, uint4* w) {
+    w[0] = __ldg(reinterpret_cast<const uint4*>(at));
+    w[1] = __ldg(reinterpret_cast<const uint4*>(at + hw * 8));
+}
+
 // The MMAs of one 16-channel chunk (32-byte K-step) of a tile.  Halo row hr at
 // column shift dx is the A window of output rows r = hr - dy for every tap row
 // dy with 0 <= r < R.  Their accumulators lie in descending row order, so those
@@ -620,8 +694,9 @@ __global__ void __launch_bounds__(kRowThreads, 2) conv_tc_rows_kernel(const __gr
                                                                    const ConvParams p, const RowPlan rp) {
     // The setup that reads nothing the preceding kernel writes (barriers, bias, tensor memory and the
     // weight load: the weights and biases are packed once) runs before the wait on that kernel, so it
-    // overlaps the preceding kernel's tail when the launch is programmatically dependent.
-    pdl_allow_dependents();
+    // overlaps the preceding kernel's tail when the launch is programmatically dependent.  The next kernel may
+    // launch once every CTA holds its tensor memory: its CTAs' allocations then wait for this kernel's and never
+    // the other way round.
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(16) float s_bias[256];
     __shared__ __align__(8) uint64_t full_bar[kRowMaxStages], empty_bar[kRowMaxStages], accf_bar[2], acce_bar[2],
@@ -664,6 +739,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) conv_tc_rows_kernel(const __gr
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
+    pdl_allow_dependents();  // every CTA holds its tensor memory by then
 
     auto tile_origin = [&](int t, int* img, int* x0, int* y0) {
         const int tx = t % p.tiles_x;
@@ -798,10 +874,6 @@ __global__ void __launch_bounds__(kRowThreads, 2) conv_tc_rows_kernel(const __gr
         constexpr int kMaskChunks = R <= 2 ? 2 : 1;
         uint4 mk[MODE == kRowMask ? R : 1][MODE == kRowMask ? kMaskChunks : 1][2];
         const __nv_bfloat16* mask_px = nullptr;
-        auto load_mask = [&](const __nv_bfloat16* at, uint4* w) {
-            w[0] = __ldg(reinterpret_cast<const uint4*>(at));
-            w[1] = __ldg(reinterpret_cast<const uint4*>(at + hw * 8));
-        };
         int i = 0;
         for (int t = first; t < rp.n_tiles; t += step, ++i) {
             const int b = i & 1;
@@ -811,7 +883,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) conv_tc_rows_kernel(const __gr
             const bool x_in = x < p.W;
             // this pixel of the tile's first row in the output's, mask's and skip gradient's first plane
             // (kRowUp2, kRowPoolBwd: at twice the size)
-            const int up = MODE == kRowUp2 ? 2 : 1, dn = MODE == kRowPoolBwd ? 2 : 1, sc = up * dn;
+            constexpr int sc = MODE == kRowUp2 || MODE == kRowPoolBwd ? 2 : 1;
             const int Ws = p.W * sc;
             const size_t hws = hw * (sc * sc);
             auto first_px = [&](int ctotal, int coff) {
@@ -831,7 +903,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) conv_tc_rows_kernel(const __gr
 #pragma unroll
                     for (int k = 0; k < kMaskChunks; ++k)
                         if (x_in && y0 + r < p.H && cfirst + k * cstep < Nc && n0 + cfirst + k * cstep < p.cout_valid)
-                            load_mask(mask_px + (size_t)k * pair + (size_t)r * p.W * 8, mk[r][k]);
+                            load_mask_words(mask_px + (size_t)k * pair + (size_t)r * p.W * 8, hw, mk[r][k]);
             }
             const bool ok = mbar_wait(smem_u32(&accf_bar[b]), (uint32_t)(i >> 1) & 1u);
             __syncwarp();
@@ -861,51 +933,18 @@ __global__ void __launch_bounds__(kRowThreads, 2) conv_tc_rows_kernel(const __gr
                     uint32_t ka[8], kb[8];
                     auto chunk = [&](const uint32_t* acc, int c, int kk, uint32_t* w) {
                         if constexpr (MODE == kRowF32) {
-                            float f[3];
-#pragma unroll
-                            for (int j = 0; j < 3; ++j) {
-                                f[j] = __fadd_rn(__fmul_rn(__uint_as_float(acc[j]), dq), s_bias[c + j]);
-                                if (p.relu) f[j] = fmaxf(f[j], 0.0f);
-                            }
-                            p.out_f32[((size_t)img * p.H + y0 + r) * p.W + x] = make_float4(f[0], f[1], f[2], 0.0f);
-                        } else if constexpr (MODE == kRowPoolBwd) {
-                            scale_pack16<FP8>(acc, dq, w);
-                            const size_t at = (size_t)kk * pairs + (size_t)(2 * r) * Ws * 8;
-                            pool_bwd16<FP8>(w, mask_px + at, skip_px + at, out_px + at, Ws, hws, amax);
+                            finish_f32(p, acc, dq, s_bias + c, ((size_t)img * p.H + y0 + r) * p.W + x);
                         } else {
-                            if constexpr (MODE == kRowMask || MODE == kRowPlain) {
-                                scale_pack16<FP8>(acc, dq, w);
-                            } else {
-                                bias_pack16<FP8>(acc, dq, s_bias + c, w);
-                                if (p.relu) {
-#pragma unroll
-                                    for (int j = 0; j < 8; ++j) w[j] = max_bf16(w[j], 0u);
-                                }
-                            }
+                            uint4 mw[2] = {};
                             if constexpr (MODE == kRowMask) {
-                                if (kk == 0) {
-                                    apply_mask(w, mk[r][0][0], mk[r][0][1]);
-                                } else if (kMaskChunks == 2 && kk == 1) {
-                                    apply_mask(w, mk[r][kMaskChunks - 1][0], mk[r][kMaskChunks - 1][1]);
-                                } else {
-                                    uint4 mw[2];
-                                    load_mask(mask_px + (size_t)kk * pair + (size_t)r * p.W * 8, mw);
-                                    apply_mask(w, mw[0], mw[1]);
-                                }
+                                if (kk == 0) mw[0] = mk[r][0][0], mw[1] = mk[r][0][1];
+                                else if (kMaskChunks == 2 && kk == 1)
+                                    mw[0] = mk[r][kMaskChunks - 1][0], mw[1] = mk[r][kMaskChunks - 1][1];
+                                else load_mask_words(mask_px + (size_t)kk * pair + (size_t)r * p.W * 8, hw, mw);
                             }
-                            if constexpr (FP8) fold_amax(amax, w, 8);
-                            __nv_bfloat16* o = out_px + (size_t)kk * pairs + (size_t)(r * up) * Ws * 8;
-                            if constexpr (MODE == kRowUp2) {
-#pragma unroll
-                                for (int gg = 0; gg < 2; ++gg) {
-                                    const uint32_t* u = w + 4 * gg;
-                                    const Words8 two_px = {{u[0], u[1], u[2], u[3], u[0], u[1], u[2], u[3]}};
-                                    store32(o + gg * hws * 8, two_px);
-                                    store32(o + gg * hws * 8 + (size_t)Ws * 8, two_px);
-                                }
-                            } else {
-                                store16(o, hws, w);
-                            }
+                            const size_t at = (size_t)kk * pairs + (size_t)(r * sc) * Ws * 8;
+                            finish16<MODE, FP8>(p, acc, dq, s_bias + c, mw[0], mw[1], mask_px + at, skip_px + at,
+                                                out_px + at, Ws, hws, w, amax);
                         }
                     };
                     if (va) chunk(v, c0, k, ka);
@@ -965,6 +1004,187 @@ __global__ void __launch_bounds__(kRowThreads, 2) conv_tc_rows_kernel(const __gr
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(rp.tmem_cols)
                      : "memory");
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Halo-tile form, for narrower images: a CTA computes 8 x 16 output pixels of a
+// slice of Nc output channels with its whole working set in shared memory at
+// once.  One TMA box brings the halo, 18 rows x 10 pixels of every input plane
+// (planes as rows of 8-byte elements, zeros outside the image), and one box per
+// tap its weights of all channel chunks ([tap][chunk][Nc][16 ch], 32-byte
+// swizzle), so the MMAs start when the halo and the first tap's weights are
+// there and wait for nothing but the next tap's.  The A operand of a tap is the
+// halo from pixel (dy, dx) on: a tile row's 8 pixels are one core matrix, tile
+// rows 160 bytes apart.  Accumulators add their products in the order tap,
+// chunk.  What bounds it is the latency of this chain (launch, halo, MMAs at
+// 32 + Nc / 4 cycles, epilogue), so the output channels are spread over as many
+// CTAs as there are SMs.  Measured, the network's forward at 2 x 128 x 128 (six
+// of its layers are this narrow) in a graph: 184 -> 92 us (before: one TMA round
+// trip per tap and chunk, 14 to 33 us a layer).
+constexpr int kHaloThreads = 128;
+constexpr int kHaloTw = 8, kHaloTh = 16;                         // output pixels
+constexpr int kHaloPx = kHaloTw + 2, kHaloRows = kHaloTh + 2;    // input pixels
+constexpr uint32_t kHaloPlane = kHaloPx * kHaloRows * 16;        // bytes of one input plane
+
+template <bool FP8, int MODE>
+__global__ void __launch_bounds__(kHaloThreads) conv_tc_halo_kernel(const __grid_constant__ CUtensorMap tmap_x8,
+                                                                    const __grid_constant__ CUtensorMap tmap_wt,
+                                                                    const ConvParams p, const HaloPlan hp) {
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(16) float s_bias[256];
+    __shared__ __align__(8) uint64_t a_bar, w_bar[9], acc_bar;
+    __shared__ uint32_t tmem_slot;
+    __shared__ volatile int failed;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    const uint32_t wbase = base + hp.a_bytes;
+    const int Nc = hp.nc, n_chunks = p.cin_bytes >> 5;
+    const uint32_t w_tap = (uint32_t)(n_chunks * Nc) * 32u;
+    int tile = blockIdx.x;
+    const int n0 = (tile % hp.n_slices) * Nc;
+    tile /= hp.n_slices;
+    const int x0 = (tile % hp.tiles_x) * kHaloTw;
+    tile /= hp.tiles_x;
+    const int y0 = (tile % hp.tiles_y) * kHaloTh, img = tile / hp.tiles_y;
+
+    if (threadIdx.x == 0) {
+        mbar_init(smem_u32(&a_bar), 1);
+        for (int t = 0; t < 9; ++t) mbar_init(smem_u32(&w_bar[t]), 1);
+        mbar_init(smem_u32(&acc_bar), 1);
+        failed = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    for (int c = threadIdx.x; c < Nc; c += blockDim.x) s_bias[c] = p.bias ? p.bias[n0 + c] : 0.0f;
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
+                     "r"(hp.tmem_cols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_slot;
+    pdl_allow_dependents();  // every CTA holds its tensor memory by then
+    if (warp == 0 && lane == 0) {  // the weights were packed once: they need not wait for the preceding kernel
+        for (int t = 0; t < 9; ++t) {
+            mbar_expect_tx(smem_u32(&w_bar[t]), w_tap);
+            tma_load_4d(wbase + (uint32_t)t * w_tap, &tmap_wt, 0, n0, 0, t, smem_u32(&w_bar[t]));
+        }
+    }
+    pdl_wait();  // activations, masks and outputs: after the preceding kernel has completed
+    if (warp == 0) {
+        if (lane == 0) {
+            const int planes = 2 * n_chunks;
+            mbar_expect_tx(smem_u32(&a_bar), (uint32_t)planes * kHaloPlane);
+            tma_load_3d(base, &tmap_x8, 2 * (x0 - 1), y0 - 1, img * planes, smem_u32(&a_bar));
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+        const uint32_t idesc = FP8 ? e4m3_idesc(128, Nc) : bf16_idesc(128, Nc);
+        const bool leader = elect_one();
+        bool ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&a_bar), 0u));
+        for (int t = 0; ok && t < 9; ++t) {
+            ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&w_bar[t]), 0u));
+            if (!ok) break;
+            tc_fence_after();
+            const uint64_t a0 = rows_desc(base + (uint32_t)((t / 3) * kHaloPx + t % 3) * 16u, kHaloPlane, kHaloPx * 16u);
+            const uint64_t b0 = sw32_desc(wbase + (uint32_t)t * w_tap);
+            for (int c = 0; c < n_chunks; ++c) {
+                const uint64_t ad = a0 + (uint64_t)((uint32_t)c * (2u * kHaloPlane >> 4));
+                const uint64_t bd = b0 + (uint64_t)((uint32_t)(c * Nc) * 2u);
+                const uint32_t acc = t > 0 || c > 0 ? 1u : 0u;
+                if (leader) mma_issue<FP8>(tm, ad, bd, idesc, acc);
+                __syncwarp();
+            }
+        }
+        if (ok && leader)
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                             smem_u32(&acc_bar))
+                         : "memory");
+        __syncwarp();
+        if (!ok) failed = 1;
+    }
+    __syncwarp();
+
+    // ---- epilogue: every thread owns one accumulator row (one pixel)
+    const int m = warp * 32 + lane;
+    const int x = x0 + m % kHaloTw, y = y0 + m / kHaloTw;
+    const bool in = x < p.W && y < p.H;
+    constexpr int sc = MODE == kRowUp2 || MODE == kRowPoolBwd ? 2 : 1;
+    const int Ws = p.W * sc;
+    const size_t hw = (size_t)p.H * p.W, hws = hw * (sc * sc);
+    auto first_px = [&](int ctotal, int coff) {
+        return ((((size_t)img * (ctotal >> 3) + ((coff + n0) >> 3)) * (p.H * sc) + y * sc) * Ws + x * sc) * 8;
+    };
+    __nv_bfloat16* out_px = MODE == kRowF32 ? nullptr : p.out + first_px(p.out_ctotal, p.out_coff);
+    const __nv_bfloat16 *mask_px = nullptr, *skip_px = nullptr;
+    if (MODE == kRowMask || MODE == kRowPoolBwd) {
+        mask_px = p.mask + first_px(p.mask_ctotal, p.mask_coff);
+        if (MODE == kRowPoolBwd) skip_px = p.gskip + first_px(p.mask_ctotal, p.mask_coff);
+    }
+    uint4 first_mask[2] = {};
+    if (MODE == kRowMask && in && n0 < p.cout_valid) load_mask_words(mask_px, hw, first_mask);
+    const float dq = FP8 ? dequant_factor(p) : 1.0f;
+    const bool acc_ok = mbar_wait(smem_u32(&acc_bar), 0u);
+    if (!acc_ok) failed = 1;
+    __syncwarp();
+    tc_fence_after();
+    uint32_t amax = 0, pool_amax = 0;
+    for (int c0 = 0, k = 0; c0 < Nc; c0 += 16, ++k) {
+        uint32_t v[16], w[8];
+        tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
+        const bool valid = acc_ok && in && n0 + c0 < p.cout_valid;
+        if (valid) {
+            if constexpr (MODE == kRowF32) {
+                finish_f32(p, v, dq, s_bias + c0, ((size_t)img * p.H + y) * p.W + x);
+            } else {
+                uint4 mw[2] = {first_mask[0], first_mask[1]};
+                if (MODE == kRowMask && k > 0) load_mask_words(mask_px + (size_t)(2 * k) * hw * 8, hw, mw);
+                const size_t at = (size_t)(2 * k) * hws * 8;
+                finish16<MODE, FP8>(p, v, dq, s_bias + c0, mw[0], mw[1], mask_px + at, skip_px + at, out_px + at, Ws, hws,
+                                    w, amax);
+            }
+        }
+        if constexpr (MODE == kRowPool) {  // a window is four lanes of the warp: x in bit 0, y in bit 3
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                w[j] = max_bf16(w[j], __shfl_xor_sync(0xffffffffu, w[j], 1));
+                w[j] = max_bf16(w[j], __shfl_xor_sync(0xffffffffu, w[j], 8));
+            }
+            if (valid && (lane & 9) == 0) {
+                const int Hp = p.H >> 1, Wp = p.W >> 1;
+                store16(p.pool_out + plane_off(img, p.pool_ctotal >> 3, (n0 + c0) >> 3, Hp, Wp, y >> 1, x >> 1),
+                        (size_t)Hp * Wp, w);
+                if constexpr (FP8) fold_amax(pool_amax, w, 8);
+            }
+        }
+        __syncwarp();
+    }
+    if constexpr (FP8) {
+        publish_amax2(p.out_amax, amax);
+        if (MODE == kRowPool) publish_amax2(p.pool_amax, pool_amax);
+    }
+
+    // ---- teardown
+    tc_fence_before();
+    __syncthreads();
+    if (failed) {
+        if (threadIdx.x == 0) {
+            atomicExch(p.err, 1u);
+            // wait (bounded) for this CTA's own TMA copies still in flight
+            for (int t = 0; t < 9; ++t)
+                if (!mbar_wait(smem_u32(&w_bar[t]), 0u)) break;
+            mbar_wait(smem_u32(&a_bar), 0u);
+        }
+        __syncthreads();
+    }
+    if (warp == 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(hp.tmem_cols) : "memory");
     }
 }
 
@@ -1112,10 +1332,61 @@ int conv_pick_tile_w(int W) {
     return tw;
 }
 
+// Halo-tile plan: the tile's halo of every plane and a slice's weights fit in
+// shared memory at once; the fewest channels per slice that still leave no SM
+// with a second CTA, so that the chain of one is as short as it gets.
+static bool plan_halo(const ConvParams& p, HaloPlan* out) {
+    const DeviceLimits& lim = device_limits();
+    if (lim.sms <= 0 || p.W >= kHaloMaxW) return false;
+    const int n_chunks = p.cin_bytes / 32;
+    HaloPlan hp{};
+    hp.tiles_x = (p.W + kHaloTw - 1) / kHaloTw;
+    hp.tiles_y = (p.H + kHaloTh - 1) / kHaloTh;
+    const long long tiles = (long long)p.n_img * hp.tiles_x * hp.tiles_y;
+    const size_t a_bytes = ((size_t)(2 * n_chunks) * kHaloPlane + 1023) & ~(size_t)1023;
+    if (2 * n_chunks > 256 || a_bytes > lim.rows_smem_max) return false;
+    hp.a_bytes = (uint32_t)a_bytes;
+    bool found = false;
+    for (int n = 1; 16 * n <= p.cout_pad; ++n) {
+        if (p.cout_pad % (16 * n) != 0) continue;
+        const int nc = p.cout_pad / n;
+        const size_t smem = a_bytes + (size_t)9 * n_chunks * nc * 32 + 1024;
+        if (smem > lim.rows_smem_max) continue;
+        if (found && tiles * n > lim.sms) break;
+        hp.nc = nc;
+        hp.n_slices = n;
+        hp.tmem_cols = pow2_at_least((uint32_t)nc);
+        hp.smem_bytes = (uint32_t)smem;
+        hp.grid = (int)(tiles * n);
+        found = true;
+    }
+    if (!found || tiles * hp.n_slices > 0x7fffffffll) return false;
+    *out = hp;
+    return true;
+}
+
 bool conv_make_desc(ConvDesc* d, const void* x, const void* w, const char** why) {
     auto enc = encode_fn(why);
     if (!enc) return false;
     const ConvParams& p = d->p;
+    d->p.x = x;
+    d->halo_form = plan_halo(p, &d->hp);
+    if (d->halo_form) {
+        if (!encode_plane_rows_map(&d->tmap_x, x, p.W, p.H, (long long)p.n_img * (p.cin_bytes / 16), kHaloPx, kHaloRows,
+                                   2 * (p.cin_bytes / 32), why))
+            return false;
+        const cuuint64_t tdims[4] = {32, (cuuint64_t)p.cout_pad, (cuuint64_t)(p.cin_bytes / 32), 9};
+        const cuuint64_t tstr[3] = {(cuuint64_t)9 * p.cin_bytes, 32, (cuuint64_t)p.cin_bytes};
+        const cuuint32_t tbox[4] = {32, (cuuint32_t)d->hp.nc, (cuuint32_t)(p.cin_bytes / 32), 1};
+        const cuuint32_t ones4[4] = {1, 1, 1, 1};
+        if (enc(&d->tmap_w, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, const_cast<void*>(w), tdims, tstr, tbox, ones4,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) {
+            *why = "tap weight tensor map rejected by the driver";
+            return false;
+        }
+        return true;
+    }
     // The maps move bytes: activations are planes of 16-byte pixel rows
     // ([img * cin_bytes / 16 + plane][H][W][16 B]), weights are K-major rows
     // of 9 * cin_bytes bytes, BF16 or E4M3 alike.
@@ -1140,7 +1411,6 @@ bool conv_make_desc(ConvDesc* d, const void* x, const void* w, const char** why)
         *why = "weight tensor map rejected by the driver";
         return false;
     }
-    d->p.x = x;
     d->rows_form = plan_rows(d->p, &d->rp);
     if (d->rows_form) {
         const RowPlan& rp = d->rp;
@@ -1163,6 +1433,20 @@ bool conv_make_desc(ConvDesc* d, const void* x, const void* w, const char** why)
     }
     return true;
 }
+
+template <bool FP8>
+static const void* halo_kernel(int mode) {
+    switch (mode) {
+        case kRowUp2: return (const void*)conv_tc_halo_kernel<FP8, kRowUp2>;
+        case kRowF32: return (const void*)conv_tc_halo_kernel<FP8, kRowF32>;
+        case kRowMask: return (const void*)conv_tc_halo_kernel<FP8, kRowMask>;
+        case kRowPlain: return (const void*)conv_tc_halo_kernel<FP8, kRowPlain>;
+        case kRowPoolBwd: return (const void*)conv_tc_halo_kernel<FP8, kRowPoolBwd>;
+        case kRowPool: return (const void*)conv_tc_halo_kernel<FP8, kRowPool>;
+        default: return (const void*)conv_tc_halo_kernel<FP8, kRowStore>;
+    }
+}
+static const void* halo_kernel(bool fp8, int mode) { return fp8 ? halo_kernel<true>(mode) : halo_kernel<false>(mode); }
 
 template <int R, bool FP8>
 static const void* rows_kernel(int mode) {
@@ -1196,6 +1480,10 @@ cudaError_t conv_launch(const ConvDesc& d, cudaStream_t stream) {
         for (const void* f : generic)
             if (attr_err == cudaSuccess)
                 attr_err = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, tile);
+        for (int mode = 0; mode <= kRowPool; ++mode)
+            for (bool fp8 : {false, true})
+                if (attr_err == cudaSuccess)
+                    attr_err = cudaFuncSetAttribute(halo_kernel(fp8, mode), cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         for (int rows : {1, 2, 4})
             for (int mode = 0; mode <= kRowPool; ++mode)
                 for (bool fp8 : {false, true})
@@ -1204,6 +1492,13 @@ cudaError_t conv_launch(const ConvDesc& d, cudaStream_t stream) {
                                                         cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     });
     if (attr_err != cudaSuccess) return attr_err;
+    if (d.halo_form) {
+        const int mode = d.p.pool_out != nullptr ? (int)kRowPool : d.p.mode;
+        using Kernel = void(const CUtensorMap, const CUtensorMap, const ConvParams, const HaloPlan);
+        auto* kernel = reinterpret_cast<Kernel*>(const_cast<void*>(halo_kernel(d.p.fp8 != 0, mode)));
+        launch_k_dependent(kernel, dim3(d.hp.grid), dim3(kHaloThreads), d.hp.smem_bytes, stream, d.tmap_x, d.tmap_w, d.p, d.hp);
+        return cudaGetLastError();
+    }
     if (d.rows_form) {
         const int mode = d.p.pool_out != nullptr ? (int)kRowPool : d.p.mode;  // run_conv pools only where the plan can
         using Kernel = void(const CUtensorMap, const ConvParams, const RowPlan);

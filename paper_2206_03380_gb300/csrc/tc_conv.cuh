@@ -71,10 +71,23 @@ struct RowPlan {
     uint32_t smem_bytes;     // dynamic shared memory
 };
 
+// Launch plan of the halo-tile form (tiles of 8 x 16 pixels, everything a tile needs resident at once).
+constexpr int kHaloMaxW = 48;  // images narrower than this
+struct HaloPlan {
+    int nc;                  // output channels per CTA (MMA N); n_slices * nc = cout_pad
+    int n_slices;
+    int tiles_x, tiles_y, grid;
+    uint32_t a_bytes;        // the halo of all planes in shared memory, 1024-byte aligned
+    uint32_t tmem_cols;
+    uint32_t smem_bytes;     // dynamic shared memory
+};
+
 // Host helpers (tc_conv.cu).
 struct ConvDesc {
-    CUtensorMap tmap_x;
-    CUtensorMap tmap_w;
+    CUtensorMap tmap_x;      // (halo-tile form: plane rows of 8-byte elements)
+    CUtensorMap tmap_w;      // (halo-tile form: (32 bytes of channels, cout, chunk, tap))
+    bool halo_form;
+    HaloPlan hp;
     CUtensorMap tmap_wh;  // row-tile form: one 16-channel chunk of all 9 taps' weights, [dx][dy][nc][16]
     bool rows_form;
     RowPlan rp;

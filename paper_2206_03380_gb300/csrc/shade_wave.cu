@@ -165,7 +165,8 @@ struct ListRays {
 
     __device__ __forceinline__ unsigned count() const { return n; }
     __device__ __forceinline__ unsigned take(unsigned k) { return atomicAdd(B.counter + 1, k); }
-    __device__ __forceinline__ int start(unsigned i, int id, f3& o, f3& d) {
+    __device__ __forceinline__ int start(unsigned i, int id, f3& o, f3& d, int& node) {
+        node = 0;
         const float4 v = __ldg(B.ray + i);
         const int slot = __float_as_int(v.w);
         d = xyz(v);

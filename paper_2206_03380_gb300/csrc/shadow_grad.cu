@@ -24,6 +24,7 @@
 #include "common.cuh"
 #include "internal.h"
 #include "shading.cuh"
+#include "trace.cuh"
 
 namespace mcdi {
 namespace {
@@ -195,8 +196,16 @@ __global__ void __launch_bounds__(kEdgeThreads) edge_write_kernel(const int* __r
     }
 }
 
-__device__ __forceinline__ f3 load_vert(const float* __restrict__ v, int i) {
-    return mk(__ldg(v + 3 * (size_t)i), __ldg(v + 3 * (size_t)i + 1), __ldg(v + 3 * (size_t)i + 2));
+// vertex i: an 8-byte load of its aligned pair and one of the third component
+// (the edge samples' random gathers cost one L1 wavefront per lane and load);
+// `pairs`: whether the array is 8-byte aligned, the same for the whole grid
+__device__ __forceinline__ f3 load_vert(const float* __restrict__ v, int i, bool pairs) {
+    const float* p = v + 3 * (size_t)i;
+    if (!pairs) return mk(__ldg(p), __ldg(p + 1), __ldg(p + 2));
+    const int odd = i & 1;
+    const float2 q = __ldg(reinterpret_cast<const float2*>(p + odd));
+    const float t = __ldg(p + (odd ? 0 : 2));
+    return odd ? mk(t, q.x, q.y) : mk(q.x, q.y, t);
 }
 
 __device__ __forceinline__ void scatter3(float* g, int i, f3 d) {
@@ -205,136 +214,244 @@ __device__ __forceinline__ void scatter3(float* g, int i, f3 d) {
     atomicAdd(g + 3 * (size_t)i + 2, d.z);
 }
 
-// Any hit for one ray with the whole warp: lane k walks the k-th of 32 equal
-// segments of the depth-first node array along the escape links.  A lane that
-// starts inside a subtree skips the box tests of its ancestors outside the
-// segment, which only adds box tests: a triangle the ray hits has every
-// ancestor box hit (boxes are conservative), so some lane reaches its leaf,
-// and the result equals the one-lane traversal's.  All lanes call this with
-// the same ray; the loop runs uniformly and ends when a lane finds a hit or
-// every lane has left its segment (each step moves strictly forward).
-__device__ __forceinline__ bool warp_any_hit(const void* nodes, const TriRecord* __restrict__ tris, int n_tris,
-                                             const RayInv& r, int lane) {
-    if (n_tris <= 0) return false;
-    const ThreadedNode* tn = threaded_nodes(nodes, n_tris);
-    const int m = 2 * n_tris - 1, seg = (m + 31) / 32;
-    int i = lane * seg;
-    const int hi = min(m, i + seg);
-    bool found = false;
-    for (;;) {
-        const bool active = i < hi;
-        if (!__any_sync(0xffffffffu, active)) return false;
-        if (active) {
-            i = threaded_step(tn, tris, r, i);
-            if (i < 0) {
-                found = true;
-                i = hi;
+// The outer rays of a CTA's candidate samples, in shared memory, traced by
+// trace_rays.  They graze surfaces and visit many nodes, so a list too short to
+// keep the CTA's 128 lanes busy is traced in up to 16 parts per ray, by as many
+// lanes, that start at the nodes two levels below the root (a node with a leaf
+// or empty child stands for itself).  Parts find a hit twice and visit what a
+// ray's end would have spared: lists of up to 32 rays are split.  Measured
+// (grad kernel, no lists split / up to 32 / all): 171 / 160 / 166 us with 4
+// candidates per 2048 samples, 339 / 319 / 431 us with 100.
+struct OuterRays {
+    static constexpr int kParts = 16;
+    static constexpr unsigned kSplit = 32;  // the longest list whose rays are traced in parts
+    static constexpr int kCap = 256;
+    float4 dir[kCap];     // w: the sample (offset in the CTA's run, int bits)
+    float4 origin[kCap];
+    unsigned hit[kCap / 32];
+    int part[kParts];  // start nodes, kWideDone beyond the last
+    unsigned n, head;
+    TraceStacks stacks;
+
+    __device__ __forceinline__ void find_parts(const void* nodes, int n_tris) {  // one thread
+        int list[kParts];
+        int k = 1;
+        list[0] = 0;
+        if (n_tris > 0) {
+            const WideNode* wn = wide_nodes(nodes, n_tris);
+            for (int level = 0; level < 2; ++level) {
+                int next[kParts], m = 0;
+                for (int i = 0; i < k; ++i) {
+                    const int4 d = __ldg(&wn[list[i]].d);
+                    if (d.x < 0 || d.y < 0 || d.z < 0 || d.w < 0) {
+                        next[m++] = list[i];
+                    } else {
+                        next[m] = d.x, next[m + 1] = d.y, next[m + 2] = d.z, next[m + 3] = d.w;
+                        m += 4;
+                    }
+                }
+                k = m;
+                for (int i = 0; i < k; ++i) list[i] = next[i];
             }
         }
-        if (__any_sync(0xffffffffu, found)) return true;
+        for (int i = 0; i < kParts; ++i) part[i] = i < k ? list[i] : kWideDone;
     }
+    __device__ __forceinline__ unsigned pending() const { return *(volatile const unsigned*)&n; }
+    // parts a ray is traced in: while a round's rays in parts would be few per lane
+    __device__ __forceinline__ int parts() const { return pending() <= kSplit ? kParts : 1; }
+    __device__ __forceinline__ unsigned count() const { return pending() * parts(); }
+    __device__ __forceinline__ unsigned take(unsigned k) { return atomicAdd(&head, k); }
+    __device__ __forceinline__ void load(int id, f3& o, f3& d) const {
+        o = xyz(origin[id]);
+        d = xyz(dir[id]);
+    }
+    __device__ __forceinline__ int start(unsigned i, int, f3& o, f3& d, int& node) const {
+        const bool split = pending() <= kSplit;
+        const int id = (int)(split ? i / kParts : i);
+        load(id, o, d);
+        const unsigned done = ((volatile const unsigned*)hit)[id >> 5] >> (id & 31);  // by another part
+        node = done & 1u ? kWideDone : split ? part[i % kParts] : 0;
+        return id;
+    }
+    __device__ __forceinline__ void blocked(int id) { atomicOr(&hit[id >> 5], 1u << (id & 31)); }
+};
+
+// What an edge sample is up to its outer ray.
+struct EdgeSample {
+    int4 ed;
+    f3 o, w, nout, ab;
+    float s, r2, ci;
+};
+
+// Sample j of a pixel (position and normal only; the shading setup waits for
+// the few samples whose outer ray is open): false unless its edge is a
+// silhouette seen from the pixel, above the horizon.
+__device__ __forceinline__ bool draw_edge_sample(const ShadeArgs& a, const float* __restrict__ verts, int n_verts,
+                                                 const int4* __restrict__ edges, int E, long long idx, int view,
+                                                 uint32_t pix, int j, EdgeSample* S) {
+    const float4 pos = a.gb_pos[idx];
+    const f3 N = xyz(a.gb_nrm[idx]);
+    const float l2 = dot(N, N);
+    if (!(pos.w > 0.0f) || !(l2 > 0.0f) || E <= 0) return false;
+    const f3 nrm = N * (1.0f / sqrtf(l2));  // as load_pixel forms it
+    const uint4 x = philox4x32_10(make_uint4(pix, (uint32_t)view, (uint32_t)j, a.stream_word),
+                                  make_uint2((uint32_t)(a.seed & 0xffffffffull), (uint32_t)(a.seed >> 32)));
+    const int e = (int)(((unsigned long long)(x.x >> 8) * (unsigned)E) >> 24);
+    S->s = (float)(x.y >> 8) * 5.9604644775390625e-8f;
+    const int4 ed = __ldg(edges + e);
+    S->ed = ed;
+    if ((unsigned)ed.x >= (unsigned)n_verts || (unsigned)ed.y >= (unsigned)n_verts ||
+        (unsigned)ed.z >= (unsigned)n_verts || ed.w >= n_verts)
+        return false;
+    const f3 o = xyz(pos) + nrm * a.ray_eps;
+    const bool pairs = ((size_t)verts & 7) == 0;
+    const f3 va = load_vert(verts, ed.x, pairs), vb = load_vert(verts, ed.y, pairs);
+    // the horizon first: it needs two of the four vertices
+    S->ab = vb - va;
+    const f3 d = va + S->ab * S->s - o;
+    S->r2 = dot(d, d);
+    S->w = d * (1.0f / sqrtf(S->r2));
+    S->ci = dot(nrm, S->w);
+    if (!(S->ci > 0.0f)) return false;
+    const f3 m = cross(va - o, vb - o);
+    const float lm = sqrtf(dot(m, m));
+    if (!(lm > 0.0f)) return false;
+    const f3 vc = load_vert(verts, ed.z, pairs);
+    const float s1 = dot(m, vc - o);
+    const float s2 = ed.w >= 0 ? dot(m, load_vert(verts, ed.w, pairs) - o) : s1;
+    if (!(s1 * s2 > 0.0f)) return false;  // both faces on one side of the plane (o, a, b): silhouette
+    S->nout = m * ((s1 > 0.0f ? -1.0f : 1.0f) / lm);
+    S->o = o;
+    return true;
 }
 
-// One thread per (pixel, edge sample).  The rare samples that reach the outer
-// ray (silhouette, above the horizon) are traced one after another by the
-// whole warp, so that each grazing ray's long chain of dependent node fetches
-// is split 32 ways.
+// A CTA owns a run of kRounds * kGradThreads (pixel, edge sample) pairs.  Its
+// threads draw them, a round of one each at a time; the few that are candidates
+// (silhouette, above the horizon: 0.2% of the samples of the mesh below) append
+// their outer ray in shared memory, and when a round might overflow the list,
+// or after the last, all lanes trace the list (trace_rays) and the samples whose
+// ray is open are drawn again and scattered.  What bounds it is the latency of
+// the samples' gathers (60%), then of the grazing outer rays' node chains; a
+// run of 4096 keeps the ends of runs few and still gives each SM its 7 CTAs.
+// Measured, 4.2M samples (512 x 512, 16 each) of 297k edges: 160 us (the whole
+// warp walking one outer ray at a time over the depth-first nodes: 243).
+constexpr int kRounds = 32;
+
 __global__ void __launch_bounds__(kGradThreads) shadow_edge_grad_kernel(
     ShadeArgs a, const float* __restrict__ verts, int n_verts, const int4* __restrict__ edges,
     const int* __restrict__ n_edges_dev, int max_edges, int M, float eta, const float4* __restrict__ g_cd,
     const float4* __restrict__ g_cs, float* g_verts, float* sample_w) {
     pdl_prologue();
-    const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long P = (long long)a.N * a.H * a.W;
-    const bool in_range = tid < P * M;
-    const long long idx = in_range ? tid / M : 0;
-    const int j = (int)(tid - idx * M);
+    __shared__ OuterRays rays;
+    const long long P = (long long)a.N * a.H * a.W, total = P * M;
+    const long long run0 = (long long)blockIdx.x * (kRounds * kGradThreads);
     const int lane = threadIdx.x & 31;
     const int E = min(max(*n_edges_dev, 0), max_edges);
-    const int view = (int)(idx / ((long long)a.H * a.W));
-    const uint32_t pix = (uint32_t)(idx - (long long)view * a.H * a.W);
-    // position and normal only (the shading setup waits for the few samples that reach the outer ray);
-    // n is formed exactly as load_pixel forms it
-    const float4 pos = in_range ? a.gb_pos[idx] : make_float4(0.f, 0.f, 0.f, 0.f);
-    const f3 N = in_range ? xyz(a.gb_nrm[idx]) : mk(0.f, 0.f, 0.f);
-    const float l2 = dot(N, N);
-    bool cand = false;
-    f3 o{}, w{}, nout{}, ab{};
-    float s = 0.f, r2 = 1.f, ci = 0.f;
-    int4 ed{};
-    do {
-        if (!(pos.w > 0.0f) || !(l2 > 0.0f) || E <= 0) break;
-        const f3 nrm = N * (1.0f / sqrtf(l2));
-        const uint4 x = philox4x32_10(make_uint4(pix, (uint32_t)view, (uint32_t)j, a.stream_word),
-                                      make_uint2((uint32_t)(a.seed & 0xffffffffull), (uint32_t)(a.seed >> 32)));
-        const int e = (int)(((unsigned long long)(x.x >> 8) * (unsigned)E) >> 24);
-        s = (float)(x.y >> 8) * 5.9604644775390625e-8f;
-        ed = __ldg(edges + e);
-        if ((unsigned)ed.x >= (unsigned)n_verts || (unsigned)ed.y >= (unsigned)n_verts ||
-            (unsigned)ed.z >= (unsigned)n_verts || ed.w >= n_verts)
-            break;
-        o = xyz(pos) + nrm * a.ray_eps;
-        const f3 va = load_vert(verts, ed.x), vb = load_vert(verts, ed.y);
-        const f3 m = cross(va - o, vb - o);
-        const float lm = sqrtf(dot(m, m));
-        if (!(lm > 0.0f)) break;
-        const float s1 = dot(m, load_vert(verts, ed.z) - o);
-        const float s2 = ed.w >= 0 ? dot(m, load_vert(verts, ed.w) - o) : s1;
-        if (!(s1 * s2 > 0.0f)) break;  // both faces on one side of the plane (o, a, b): silhouette
-        ab = vb - va;
-        const f3 d = va + ab * s - o;
-        r2 = dot(d, d);
-        w = d * (1.0f / sqrtf(r2));
-        ci = dot(nrm, w);
-        if (!(ci > 0.0f)) break;
-        nout = m * ((s1 > 0.0f ? -1.0f : 1.0f) / lm);
-        cand = true;
-    } while (false);
-    // the outer rays of this warp's candidates, each traced by all 32 lanes
-    bool open = false;
-    const f3 dir = normalize(w + nout * eta);
-    for (unsigned todo = __ballot_sync(0xffffffffu, cand); todo; todo &= todo - 1u) {
-        const int src = __ffs(todo) - 1;
-        const f3 ro = mk(__shfl_sync(0xffffffffu, o.x, src), __shfl_sync(0xffffffffu, o.y, src),
-                         __shfl_sync(0xffffffffu, o.z, src));
-        const f3 rd = mk(__shfl_sync(0xffffffffu, dir.x, src), __shfl_sync(0xffffffffu, dir.y, src),
-                         __shfl_sync(0xffffffffu, dir.z, src));
-        const bool hit = warp_any_hit(a.nodes, static_cast<const TriRecord*>(a.tris), a.n_tris, make_ray(ro, rd), lane);
-        if (lane == src) open = !hit;
-    }
-    float wt = 0.0f;
-    if (open) {
-        Pixel px{};
-        load_pixel(pos, a.gb_nrm[idx], a.gb_kd[idx], a.gb_korm[idx],
-                   mk(a.cams[view].origin[0], a.cams[view].origin[1], a.cams[view].origin[2]), &px);
-        Probe Pr;
-        Pr.W = a.Wp;
-        Pr.H = a.Hp;
-        float st;
-        const int t = texel_of_dir(Pr, w, &st);
-        const f3 L = xyz(__ldg(a.env + t));
-        const f3 gd = xyz(g_cd[idx]);
-        float gw = (L.x * gd.x + L.y * gd.y + L.z * gd.z) * ci * MCDI_INV_PI;
-        if (px.spec_on) {
-            const f3 gs = xyz(g_cs[idx]);
-            const f3 h = normalize(w + px.wo);
-            const float nh = dot(px.n, h), vh = dot(px.wo, h);
-            const float D = ggx_D(nh, sin2_between(px.n, h), px.a2);
-            const float G2 = 1.0f / (1.0f + ggx_lambda(ci, px.a2) + ggx_lambda(px.co, px.a2));
-            const float q = schlick_weight(vh);
-            const f3 F = mk(px.F0.x + (1.f - px.F0.x) * q, px.F0.y + (1.f - px.F0.y) * q,
-                            px.F0.z + (1.f - px.F0.z) * q);
-            gw += (L.x * gs.x * F.x + L.y * gs.y * F.y + L.z * gs.z * F.z) * D * G2 / (4.0f * px.co);
+    // pixel, view and sample of the run's pair k, by 32-bit divisions from the run's first
+    __shared__ long long s_idx;
+    __shared__ unsigned s_first[3];  // sample, pixel, view
+    const unsigned HW = (unsigned)a.H * (unsigned)a.W;
+    auto locate = [&](unsigned k, long long* idx, int* view, uint32_t* pix, int* j) {
+        const unsigned t = s_first[0] + k, q = t / (unsigned)M, p = s_first[1] + q, v = p / HW;
+        *j = (int)(t - q * (unsigned)M);
+        *idx = s_idx + q;
+        *view = (int)(s_first[2] + v);
+        *pix = p - v * HW;
+    };
+    auto flush = [&]() {  // whole CTA, after a barrier
+        trace_rays(a.nodes, static_cast<const TriRecord*>(a.tris), a.n_tris, rays.stacks, rays);
+        __syncthreads();
+        const unsigned n = rays.n;
+        for (unsigned i = threadIdx.x; i < n; i += kGradThreads) {
+            if ((rays.hit[i >> 5] >> (i & 31)) & 1u) continue;
+            const int k = __float_as_int(rays.dir[i].w);
+            long long idx;
+            int view, j;
+            uint32_t pix;
+            locate(k, &idx, &view, &pix, &j);
+            EdgeSample S;
+            if (!draw_edge_sample(a, verts, n_verts, edges, E, idx, view, pix, j, &S)) continue;  // (it was one)
+            Pixel px{};
+            load_pixel(a.gb_pos[idx], a.gb_nrm[idx], a.gb_kd[idx], a.gb_korm[idx],
+                       mk(a.cams[view].origin[0], a.cams[view].origin[1], a.cams[view].origin[2]), &px);
+            Probe Pr;
+            Pr.W = a.Wp;
+            Pr.H = a.Hp;
+            float st;
+            const int t = texel_of_dir(Pr, S.w, &st);
+            const f3 L = xyz(__ldg(a.env + t));
+            const f3 gd = xyz(g_cd[idx]);
+            float gw = (L.x * gd.x + L.y * gd.y + L.z * gd.z) * S.ci * MCDI_INV_PI;
+            if (px.spec_on) {
+                const f3 gs = xyz(g_cs[idx]);
+                const f3 h = normalize(S.w + px.wo);
+                const float nh = dot(px.n, h), vh = dot(px.wo, h);
+                const float D = ggx_D(nh, sin2_between(px.n, h), px.a2);
+                const float G2 = 1.0f / (1.0f + ggx_lambda(S.ci, px.a2) + ggx_lambda(px.co, px.a2));
+                const float q = schlick_weight(vh);
+                const f3 F = mk(px.F0.x + (1.f - px.F0.x) * q, px.F0.y + (1.f - px.F0.y) * q,
+                                px.F0.z + (1.f - px.F0.z) * q);
+                gw += (L.x * gs.x * F.x + L.y * gs.y * F.y + L.z * gs.z * F.z) * D * G2 / (4.0f * px.co);
+            }
+            const f3 c = cross(S.w, S.ab);
+            const float J = sqrtf(dot(c, c)) / S.r2;
+            const float wt = -a.tau * gw * J * ((float)E / (float)M);
+            if (wt != 0.0f) {
+                scatter3(g_verts, S.ed.x, S.nout * (wt * (1.0f - S.s)));
+                scatter3(g_verts, S.ed.y, S.nout * (wt * S.s));
+            }
+            if (sample_w) sample_w[run0 + k] = wt;
         }
-        const f3 c = cross(w, ab);
-        const float J = sqrtf(dot(c, c)) / r2;
-        wt = -a.tau * gw * J * ((float)E / (float)M);
-        if (wt != 0.0f) {
-            scatter3(g_verts, ed.x, nout * (wt * (1.0f - s)));
-            scatter3(g_verts, ed.y, nout * (wt * s));
-        }
+    };
+    auto clear = [&]() {  // whole CTA, between barriers
+        if (threadIdx.x == 0) rays.n = rays.head = 0u;
+        if (threadIdx.x < OuterRays::kCap / 32) rays.hit[threadIdx.x] = 0u;
+    };
+    clear();
+    if (threadIdx.x == 0) rays.find_parts(a.nodes, a.n_tris);
+    if (threadIdx.x == 32) {
+        s_idx = run0 / M;
+        const long long view = s_idx / HW;
+        s_first[0] = (unsigned)(run0 - s_idx * M);
+        s_first[1] = (unsigned)(s_idx - view * HW);
+        s_first[2] = (unsigned)view;
     }
-    if (sample_w && in_range) sample_w[tid] = wt;
+    __syncthreads();
+    for (int r = 0; r < kRounds; ++r) {
+        const int k = r * kGradThreads + threadIdx.x;
+        const long long tid = run0 + k;
+        EdgeSample S;
+        bool cand = false;
+        if (tid < total) {
+            long long idx;
+            int view, j;
+            uint32_t pix;
+            locate(k, &idx, &view, &pix, &j);
+            cand = draw_edge_sample(a, verts, n_verts, edges, E, idx, view, pix, j, &S);
+            if (sample_w) sample_w[tid] = 0.0f;
+        }
+        const unsigned mask = __ballot_sync(0xffffffffu, cand);
+        if (mask) {
+            unsigned base = 0;
+            if (lane == 0) base = atomicAdd(&rays.n, (unsigned)__popc(mask));
+            base = __shfl_sync(0xffffffffu, base, 0);
+            if (cand) {
+                const unsigned i = base + __popc(mask & ((1u << lane) - 1u));
+                const f3 dir = normalize(S.w + S.nout * eta);
+                rays.dir[i] = make_float4(dir.x, dir.y, dir.z, __int_as_float(k));
+                rays.origin[i] = make_float4(S.o.x, S.o.y, S.o.z, 0.f);
+            }
+        }
+        __syncthreads();
+        const bool full = rays.pending() > OuterRays::kCap - kGradThreads;
+        if (full || r == kRounds - 1) {
+            flush();
+            __syncthreads();
+            if (r == kRounds - 1) break;
+            clear();
+        }
+        __syncthreads();  // every thread has read the count before the next round adds to it
+    }
 }
 
 inline size_t edge_table_cap(int n_tris) {
@@ -396,7 +513,8 @@ cudaError_t launch_shadow_edge_grad(const ShadeArgs& a, const float* verts, int 
                                     const float4* g_cs, float* g_verts, float* sample_w, cudaStream_t stream) {
     const long long n = (long long)a.N * a.H * a.W * n_samples;
     if (n <= 0) return cudaGetLastError();
-    launch_k(shadow_edge_grad_kernel, (int)((n + kGradThreads - 1) / kGradThreads), kGradThreads, 0, stream, a, verts,
+    const long long run = kRounds * kGradThreads;
+    launch_k(shadow_edge_grad_kernel, (int)((n + run - 1) / run), kGradThreads, 0, stream, a, verts,
              n_verts, edges, n_edges, max_edges, n_samples, eta, g_cd, g_cs, g_verts, sample_w);
     return cudaGetLastError();
 }

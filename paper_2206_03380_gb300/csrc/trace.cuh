@@ -37,8 +37,9 @@ struct TraceStacks {  // a CTA's columns: one thread's entries in one bank
 // of the depth-first copy instead.
 //
 // R supplies the rays: R.count() of them, the same for all warps; R.take(n)
-// (lane 0) reserves the next n and returns the first; R.start(i, id, o, d)
-// loads ray i and returns the lane's handle for it (id: the handle of its ray
+// (lane 0) reserves the next n and returns the first; R.start(i, id, o, d,
+// node) loads ray i, sets the node it starts at (0, the root, or kWideDone for
+// none) and returns the lane's handle for it (id: the handle of its ray
 // before); R.load(id, o, d) gives a ray again by handle (the current ray's or
 // the one before); R.blocked(id) records a hit.
 template <class R>
@@ -71,10 +72,9 @@ __device__ __forceinline__ void trace_rays(const void* __restrict__ nodes, const
             if (free_lane && my < n_rays) {
                 f3 o, d;
                 last = cur;
-                cur = rays.start(my, cur, o, d);
+                cur = rays.start(my, cur, o, d, node);
                 inv = make_ray(o, d).inv;
                 oi = mk(-o.x * inv.x, -o.y * inv.y, -o.z * inv.z);
-                node = 0;
                 lmark = la;
             }
             more = base + (unsigned)__popc(idle) < n_rays;
@@ -161,8 +161,9 @@ struct BlockRays {
         d = xyz(v);
         o = xyz(origin[__float_as_int(v.w) & 31]);
     }
-    __device__ __forceinline__ int start(unsigned i, int, f3& o, f3& d) const {
+    __device__ __forceinline__ int start(unsigned i, int, f3& o, f3& d, int& node) const {
         load((int)i, o, d);
+        node = 0;
         return (int)i;
     }
     __device__ __forceinline__ void blocked(int id) {

@@ -135,4 +135,31 @@ __host__ __device__ inline const WideNode* wide_nodes(const void* nodes, int n_t
 
 constexpr int kTraversalStack = 64;  // >= depth of a tree over 62-bit unique keys
 
+// two fused multiply-adds in one instruction: (x.x a + b, x.y a + b)
+__device__ __forceinline__ float2 fma2(float2 x, float2 a, float2 b) {
+    float2 r;
+    asm("{\n\t.reg .b64 rx, ra, rb, rd;\n\t"
+        "mov.b64 rx, {%2, %3};\n\tmov.b64 ra, {%4, %5};\n\tmov.b64 rb, {%6, %7};\n\t"
+        "fma.rn.f32x2 rd, rx, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(x.x), "f"(x.y), "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+    float2 r;
+    asm("{\n\t.reg .b64 ra, rb, rd;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
+        "mul.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+    float2 r;
+    asm("{\n\t.reg .b64 ra, rb, rd;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
+        "add.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+
 }  // namespace mcdi

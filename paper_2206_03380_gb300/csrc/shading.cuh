@@ -300,17 +300,6 @@ __device__ __forceinline__ void sts64(uint32_t a, float x, float y) {
     asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(x), "f"(y) : "memory");
 }
 
-// two fused multiply-adds in one instruction: (x.x a + b, x.y a + b)
-__device__ __forceinline__ float2 fma2(float2 x, float2 a, float2 b) {
-    float2 r;
-    asm("{\n\t.reg .b64 rx, ra, rb, rd;\n\t"
-        "mov.b64 rx, {%2, %3};\n\tmov.b64 ra, {%4, %5};\n\tmov.b64 rb, {%6, %7};\n\t"
-        "fma.rn.f32x2 rd, rx, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
-        : "=f"(r.x), "=f"(r.y)
-        : "f"(x.x), "f"(x.y), "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-    return r;
-}
-
 // The node part of wide_step for a traversal that postpones its triangle
 // tests: hit inner children are appended to the lane's node stack (entries at
 // shared address na, kStep bytes apart), hit leaf children to its leaf queue

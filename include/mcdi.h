@@ -422,8 +422,10 @@ MCDI_API mcdi_status mcdi_read_sweep(const void* buf, size_t bytes, int passes, 
  *
  * Weight gradient (the live-trained denoiser of App. B; the main results of
  * Sec. 4.2 lock the weights and need none):
- * mcdi_denoise_wgrad_bytes (host): scratch bytes mcdi_denoise_wgrad needs for
- * n_img images of H x W.
+ * mcdi_denoise_wgrad_bytes (host): scratch bytes for mcdi_denoise_wgrad with
+ * n_img images of H x W: room for the partial sums of several convolutions,
+ * which then share a launch (the largest one's are the least it accepts; the
+ * results do not depend on it).
  * mcdi_denoise_wgrad: after mcdi_denoise_fwd (acts) and mcdi_denoise_bwd
  * (grad_ws) of the same images, precision and sizes, writes gw (device FP32,
  * n_params values in the order of mcdi_denoise_pack_weights' params:

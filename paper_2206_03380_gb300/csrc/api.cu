@@ -624,13 +624,13 @@ mcdi_status mcdi_denoise_wgrad(int precision, int n_img, int H, int W, const voi
     REQUIRE(grad_ws != nullptr && ((uintptr_t)grad_ws & 255u) == 0 && grad_bytes >= need_g,
             "grad_ws must be 256-byte aligned and hold %zu bytes", need_g);
     REQUIRE(gw != nullptr && ((uintptr_t)gw & 3u) == 0, "gw must be a non-NULL device float pointer");
-    const size_t need_s = mcdi::unet_wgrad_bytes(n_img, H, W);
+    const size_t need_s = mcdi::unet_wgrad_bytes_min(n_img, H, W);
     REQUIRE(scratch != nullptr && ((uintptr_t)scratch & 255u) == 0, "scratch must be 256-byte aligned");
     REQUIRE(scratch_bytes >= need_s, "scratch too small: %zu < %zu bytes", scratch_bytes, need_s);
     REQUIRE(err != nullptr && ((uintptr_t)err & 3u) == 0, "err must be a device uint32");
     const char* why = "";
-    const cudaError_t e =
-        mcdi::launch_unet_wgrad(acts, grad_ws, n_img, H, W, gw, scratch, err, static_cast<cudaStream_t>(stream), &why);
+    const cudaError_t e = mcdi::launch_unet_wgrad(acts, grad_ws, n_img, H, W, gw, scratch, scratch_bytes, err,
+                                                  static_cast<cudaStream_t>(stream), &why);
     if (e == cudaErrorInvalidValue && why[0]) return fail(MCDI_DEVICE_ERROR, "denoise_wgrad: %s", why);
     return launched(e, "denoise_wgrad");
 }
@@ -767,8 +767,8 @@ mcdi_status mcdi_conv3x3_wgrad(const void* x, const void* g, int n_img, int H, i
     REQUIRE(scratch_bytes >= need, "scratch too small: %zu < %zu bytes", scratch_bytes, need);
     REQUIRE(err != nullptr && ((uintptr_t)err & 3u) == 0, "err must be a device uint32");
     const char* why = "";
-    const cudaError_t e = mcdi::launch_wgrad(x, cin_pad, g, cout_pad, n_img, H, W, cin, cout, scratch, gw, err,
-                                             static_cast<cudaStream_t>(stream), &why);
+    const mcdi::WgradConv conv{x, g, cin_pad, cout_pad, n_img, H, W, cin, cout, gw};
+    const cudaError_t e = mcdi::launch_wgrad(&conv, 1, scratch, err, static_cast<cudaStream_t>(stream), &why);
     if (e == cudaErrorInvalidValue && why[0]) return fail(MCDI_DEVICE_ERROR, "conv3x3_wgrad: %s", why);
     return launched(e, "conv3x3_wgrad");
 }

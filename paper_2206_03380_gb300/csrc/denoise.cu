@@ -679,31 +679,54 @@ cudaError_t launch_unet_bwd(const void* weights, int precision, int n, int H, in
 static const int kWgX[kUnetConvs] = {X0, A1, P1, A2, P2, A3, P3, B1, CAT3, D3A, CAT2, D2A, CAT1, D1A, D1B};
 static const int kWgG[kUnetConvs] = {GA1, GE1, GA2, GE2, GA3, GE3, GB1, GB2, GD3A, GD3B, GD2A, GD2B, GD1A, GD1B, GY};
 
-size_t unet_wgrad_bytes(int n, int H, int W) {
+static size_t conv_wgrad_bytes(int k, int n, int H, int W) {
+    const int l = kPlan[k].level;
+    return wgrad_scratch_bytes(kActC[kWgX[k]], kGradC[kWgG[k]], n, H >> l, W >> l);
+}
+
+size_t unet_wgrad_bytes_min(int n, int H, int W) {
     size_t m = 0;
-    for (int k = 0; k < kUnetConvs; ++k) {
-        const int l = kPlan[k].level;
-        m = std::max(m, wgrad_scratch_bytes(kActC[kWgX[k]], kGradC[kWgG[k]], n, H >> l, W >> l));
-    }
+    for (int k = 0; k < kUnetConvs; ++k) m = std::max(m, conv_wgrad_bytes(k, n, H, W));
     return m;
 }
 
+// Room for the partial sums of all convolutions, up to half the L2: beyond, the
+// sums would go to memory and back between the two kernels, and the
+// convolutions fill the GPU by themselves.  Measured, launched kernel by kernel,
+// scratch of 64 / 256 MB: 2 x 256 x 256 126 / 123 us, 2 x 512 x 512 285 / 266,
+// 8 x 800 x 800 1599 / 1551 (of the largest convolution: 219, 348, 1636).
+size_t unet_wgrad_bytes(int n, int H, int W) {
+    size_t sum = 0;
+    for (int k = 0; k < kUnetConvs; ++k) sum += conv_wgrad_bytes(k, n, H, W);
+    return std::max(unet_wgrad_bytes_min(n, H, W), std::min(sum, (size_t)64 << 20));
+}
+
 cudaError_t launch_unet_wgrad(const void* acts, const void* grad_ws, int n, int H, int W, float* gw, void* scratch,
-                              unsigned* err, cudaStream_t s, const char** why) {
+                              size_t scratch_bytes, unsigned* err, cudaStream_t s, const char** why) {
     size_t aoff[kActs], goff[kGrads], t;
     layout_of<kActs>(kActC, kActLvl, n, H, W, aoff, &t);
     layout_of<kGrads>(kGradC, kGradLvl, n, H, W, goff, &t);
-    size_t o = 0;  // parameter order: W[co][ci][3][3], then b[co], per convolution
+    static_assert(kUnetConvs <= kWgradMaxLayers, "a group may hold every convolution");
+    WgradConv group[kUnetConvs];
+    int m = 0;
+    size_t o = 0, used = 0;  // parameter order: W[co][ci][3][3], then b[co], per convolution
     for (int k = 0; k < kUnetConvs; ++k) {
         const int l = kPlan[k].level;
-        const cudaError_t e =
-            launch_wgrad(static_cast<const char*>(acts) + aoff[kWgX[k]], kActC[kWgX[k]],
-                         static_cast<const char*>(grad_ws) + goff[kWgG[k]], kGradC[kWgG[k]], n, H >> l, W >> l,
-                         kPlan[k].ci, kPlan[k].co, scratch, gw + o, err, s, why);
-        if (e != cudaSuccess) return e;
+        const size_t need = conv_wgrad_bytes(k, n, H, W);
+        if (m > 0 && used + need > scratch_bytes) {  // a group ends where the scratch is full
+            const cudaError_t e = launch_wgrad(group, m, scratch, err, s, why);
+            if (e != cudaSuccess) return e;
+            m = 0;
+            used = 0;
+        }
+        group[m++] = WgradConv{static_cast<const char*>(acts) + aoff[kWgX[k]],
+                               static_cast<const char*>(grad_ws) + goff[kWgG[k]], kActC[kWgX[k]], kGradC[kWgG[k]], n,
+                               H >> l, W >> l, kPlan[k].ci, kPlan[k].co, gw + o};
+        used += need;
         o += (size_t)kPlan[k].co * kPlan[k].ci * 9 + kPlan[k].co;
     }
-    return cudaGetLastError();
+    const cudaError_t e = launch_wgrad(group, m, scratch, err, s, why);
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t launch_conv3x3(const void* x, int n, int H, int W, int cin_pad, const void* w, const float* bias,

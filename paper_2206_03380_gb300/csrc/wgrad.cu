@@ -31,7 +31,15 @@
 // four warps read the accumulators back and store this CTA's partial sums
 // ([dx][co][row], one 128-byte line per warp store), and a second kernel adds
 // the partials of each weight in a fixed order, so results are bitwise
-// repeatable.  Every wait is bounded (2 s of %globaltimer): on a timeout the
+// repeatable.  A launch takes several convolutions (the U-Net's 15 as far as
+// their partial sums fit the scratch), the ones with the longest CTAs first: one
+// by one, each launch is some 8 us of latency (set-up, the first loads, the
+// partials' stores) around a few microseconds of loads, and most leave SMs idle.
+// Measured, the U-Net's weight gradient in a graph, launches one by one / grouped:
+// 2 x 256 x 256: 200 / 111 us; 1 x 64 x 72: 152 / 23; 2 x 512 x 512: 327 / 269;
+// 8 x 800 x 800: 1599 / 1577, the same sums in the same order.  There it is the
+// loads through L2 that bound it (every input row three times, every gradient row
+// at three shifts).  Every wait is bounded (2 s of %globaltimer): on a timeout the
 // kernel sets *err, drains its own copies and frees its tensor memory.
 #include <cuda_bf16.h>
 
@@ -64,6 +72,28 @@ struct WgradArgs {
     unsigned* err;
 };
 
+// One convolution of a launch: its CTAs are blocks first .. of the kernel, its
+// elements' blocks first_red .. of the reduction.
+struct WgradLayer {
+    CUtensorMap xf, xl, g;  // input boxes of 5 planes (all groups but the last) and of the last group's planes;
+                            // gradient boxes of all gp planes, one row
+    WgradArgs a;
+    int ci, co, n_rb;
+    int split;              // how its reduction adds (wgrad_reduce_kernel)
+    int first, first_red;
+    float* gw;
+};
+struct WgradBatch {
+    WgradLayer layer[kWgradMaxLayers];
+    int n;
+};
+
+__device__ __forceinline__ const WgradLayer& layer_of(const WgradBatch& b, int WgradLayer::*first) {
+    int k = 0;
+    while (k + 1 < b.n && (int)blockIdx.x >= b.layer[k + 1].*first) ++k;
+    return b.layer[k];
+}
+
 __device__ __forceinline__ int group_planes(const WgradArgs& a, int g) {
     return g == a.n_groups - 1 ? a.xp - kGroupPlanes * (a.n_groups - 1) : kGroupPlanes;
 }
@@ -86,22 +116,19 @@ __device__ __forceinline__ void mma_mn(uint32_t d, uint64_t ad, uint64_t bd, uin
         : "memory");
 }
 
-// tmap_xf / tmap_xl: input boxes of 5 planes (all groups but the last) and of the last group's planes;
-// tmap_g: gradient boxes of all gp planes, one row.
-__global__ void __launch_bounds__(kWgThreads, 2) wgrad_kernel(const __grid_constant__ CUtensorMap tmap_xf,
-                                                              const __grid_constant__ CUtensorMap tmap_xl,
-                                                              const __grid_constant__ CUtensorMap tmap_g,
-                                                              const WgradArgs a) {
+__global__ void __launch_bounds__(kWgThreads, 2) wgrad_kernel(const __grid_constant__ WgradBatch batch) {
     pdl_prologue();
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[kWgMaxStages], empty_bar[kWgMaxStages], acc_bar;
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int failed;
 
+    const WgradLayer& L = layer_of(batch, &WgradLayer::first);
+    const WgradArgs& a = L.a;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* const base_ptr = smem_raw + (base - smem_u32(smem_raw));
-    const int bid = blockIdx.x;
+    const int bid = (int)blockIdx.x - L.first;
     const int grp = bid % a.n_groups, rb = bid / a.n_groups;
     const int P = group_planes(a, grp);
     const int x_slots = 3 * P;  // slots (plane, dy) filled by TMA
@@ -121,17 +148,14 @@ __global__ void __launch_bounds__(kWgThreads, 2) wgrad_kernel(const __grid_const
         failed = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // slots past the TMA box are never loaded: set them once per stage, to zero, except channel 0 of the
-    // ones slot in the first group
-    {
+    // The ones slot of the first group: 1 in channel 0, set once per stage.  The other slots past the TMA box
+    // are left as they are: they feed only accumulator rows that are never stored.
+    if (grp == 0) {
         const int px = (int)(a.slot_bytes / 16);
-        const int n_pad = (kGroupSlots - x_slots) * px;
-        for (int s = 0; s < a.stages; ++s) {
-            uint4* pad = reinterpret_cast<uint4*>(base_ptr + (size_t)s * a.stage_bytes + (size_t)x_slots * a.slot_bytes);
-            for (int i = threadIdx.x; i < n_pad; i += blockDim.x) {
-                const bool one = grp == 0 && x_slots + i / px == kOnesSlot;
-                pad[i] = make_uint4(one ? 0x3F80u : 0u, 0u, 0u, 0u);  // BF16 1.0 in channel 0
-            }
+        for (int i = threadIdx.x; i < a.stages * px; i += blockDim.x) {
+            const int st = i / px;
+            reinterpret_cast<uint4*>(base_ptr + (size_t)st * a.stage_bytes + (size_t)kOnesSlot * a.slot_bytes)[i - st * px] =
+                make_uint4(0x3F80u, 0u, 0u, 0u);  // BF16 1.0 in channel 0
         }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -150,7 +174,7 @@ __global__ void __launch_bounds__(kWgThreads, 2) wgrad_kernel(const __grid_const
     if (warp == 0) {
         if (lane == 0) {
             // ---- loader: per item one input box (3 rows of this group's planes) and three G boxes (dx = 0, 1, 2)
-            const CUtensorMap* xmap = grp == a.n_groups - 1 ? &tmap_xl : &tmap_xf;
+            const CUtensorMap* xmap = grp == a.n_groups - 1 ? &L.xl : &L.xf;
             const uint32_t tx = (grp == a.n_groups - 1 ? a.x_bytes_last : a.x_bytes_full) + 3u * a.g_bytes;
             const uint32_t g_copy = (uint32_t)a.gp * a.slot_bytes;  // bytes of one shifted G copy in shared memory
             int img = r0 / a.H, y = r0 - img * a.H, q0 = 0, s = 0;
@@ -165,7 +189,7 @@ __global__ void __launch_bounds__(kWgThreads, 2) wgrad_kernel(const __grid_const
                 tma_load_3d(st, xmap, 2 * q0, y - 1, img * a.xp + grp * kGroupPlanes, fb);
 #pragma unroll
                 for (int dx = 0; dx < 3; ++dx)
-                    tma_load_3d(st + x_region + (uint32_t)dx * g_copy, &tmap_g, 2 * (q0 + 1 - dx), y, img * a.gp, fb);
+                    tma_load_3d(st + x_region + (uint32_t)dx * g_copy, &L.g, 2 * (q0 + 1 - dx), y, img * a.gp, fb);
                 issued = it + 1;
                 q0 += a.seg;  // next item: segment, then row, then image
                 if (q0 >= a.W) {
@@ -236,13 +260,18 @@ __global__ void __launch_bounds__(kWgThreads, 2) wgrad_kernel(const __grid_const
         const int m = warp * 32 + lane;
         const bool row_ok = m / 8 < x_slots || (grp == 0 && m / 8 == kOnesSlot && (m & 7) == 0);
         float* out = a.partial + (size_t)bid * 3 * N * 128 + m;
-        for (int c0 = 0; c0 < 3 * N; c0 += 16) {
-            uint32_t v[16];
-            tmem_ld16_async(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
+        const uint32_t acc = tmem + ((uint32_t)(warp * 32) << 16);
+        for (int c0 = 0; c0 < 3 * N; c0 += 48) {  // N is a multiple of 16
+            uint32_t v[3][16];
+#pragma unroll
+            for (int q = 0; q < 3; ++q) tmem_ld16_async(acc + (uint32_t)(c0 + 16 * q), v[q]);
             tmem_wait_ld();
             if (!row_ok) continue;
 #pragma unroll
-            for (int k = 0; k < 16; ++k) out[(size_t)(c0 + k) * 128] = n_items > 0 ? __uint_as_float(v[k]) : 0.0f;
+            for (int q = 0; q < 3; ++q)
+#pragma unroll
+                for (int k = 0; k < 16; ++k)
+                    out[(size_t)(c0 + 16 * q + k) * 128] = n_items > 0 ? __uint_as_float(v[q][k]) : 0.0f;
         }
     }
     tc_fence_before();
@@ -263,28 +292,32 @@ __global__ void __launch_bounds__(kWgThreads, 2) wgrad_kernel(const __grid_const
 // The sum over row blocks of the CTAs' partials, in a fixed order, stored at each element's weight
 // gw[co][ci][dy][dx] (n = co; slot m / 8 = 3 plane + dy within the group) or, for the ones row (first
 // group, slot 15, channel 0) at dx = 1, at the bias gradient db[co].  Elements r = (dx, n, m) of a group run
-// with m fastest (coalesced).  kSplit: a block of 8 warps owns 32 consecutive elements, warp w adds the
+// with m fastest (coalesced).  split: a block of 8 warps owns 32 consecutive elements, warp w adds the
 // partials of row blocks w, w + 8, ... and warp 0 adds the 8 warp sums in order (many row blocks); else one
 // thread per element adds all row blocks in order (few row blocks).
 constexpr int kReduceWarps = 8;
-template <bool kSplit>
-__global__ void __launch_bounds__(32 * kReduceWarps) wgrad_reduce_kernel(const WgradArgs a, int ci, int co, int n_rb,
-                                                                        float* __restrict__ gw) {
+__global__ void __launch_bounds__(32 * kReduceWarps) wgrad_reduce_kernel(const __grid_constant__ WgradBatch batch) {
     pdl_prologue();
+    const WgradLayer& L = layer_of(batch, &WgradLayer::first_red);
+    const WgradArgs& a = L.a;
+    const bool split = L.split != 0;
+    const int ci = L.ci, co = L.co, n_rb = L.n_rb;
+    float* __restrict__ gw = L.gw;
     __shared__ float red[kReduceWarps][32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int N = 8 * a.gp;
     const int per_group = 3 * N * 128;
-    const int elems_per_block = kSplit ? 32 : 32 * kReduceWarps;
+    const int elems_per_block = split ? 32 : 32 * kReduceWarps;
     const int blocks_per_group = per_group / elems_per_block;
-    const int grp = blockIdx.x / blocks_per_group;
-    const int r = (blockIdx.x - grp * blocks_per_group) * elems_per_block + (kSplit ? lane : (int)threadIdx.x);
+    const int block = (int)blockIdx.x - L.first_red;
+    const int grp = block / blocks_per_group;
+    const int r = (block - grp * blocks_per_group) * elems_per_block + (split ? lane : (int)threadIdx.x);
     const int m = r & 127, n = (r >> 7) % N, dx = (r >> 7) / N;
     const int slot = m / 8, pl = slot / 3, dy = slot - 3 * pl;
     const int c_in = (grp * kGroupPlanes + pl) * 8 + (m & 7);
     const bool bias = grp == 0 && slot == kOnesSlot && (m & 7) == 0 && dx == 1;
     const bool valid = n < co && ((slot < 3 * group_planes(a, grp) && c_in < ci) || bias);
-    const int b0 = kSplit ? warp : 0, db = kSplit ? kReduceWarps : 1;
+    const int b0 = split ? warp : 0, db = split ? kReduceWarps : 1;
     float s = 0.0f;
     if (valid) {
         const float* p = a.partial + (size_t)grp * per_group + r;
@@ -300,7 +333,7 @@ __global__ void __launch_bounds__(32 * kReduceWarps) wgrad_reduce_kernel(const W
         }
         for (; b < n_rb; b += db) s += p[(size_t)b * stride];
     }
-    if (kSplit) {
+    if (split) {
         red[warp][lane] = s;
         __syncthreads();
         if (warp != 0) return;
@@ -374,34 +407,66 @@ size_t wgrad_scratch_bytes(int x_ctot, int g_ctot, int n_img, int H, int W) {
     return align256(P.partial_bytes);
 }
 
-cudaError_t launch_wgrad(const void* x, int x_ctot, const void* g, int g_ctot, int n_img, int H, int W, int ci,
-                         int co, void* scratch, float* gw, unsigned* err, cudaStream_t s, const char** why) {
-    WgradPlan P = wgrad_plan(x_ctot / 8, g_ctot / 8, n_img, H, W, device_sms());
-    if (P.smem > kWgSmemMax || x_ctot % 8 || g_ctot % 16 || ci > x_ctot || co > g_ctot ||
-        g_ctot / 8 > kMaxGPlanes) {
-        *why = "weight-gradient shape outside the supported range";
+cudaError_t launch_wgrad(const WgradConv* conv, int n, void* scratch, unsigned* err, cudaStream_t s,
+                         const char** why) {
+    WgradBatch B{};
+    if (n < 1 || n > kWgradMaxLayers) {
+        *why = "too many convolutions in a weight-gradient launch";
         return cudaErrorInvalidValue;
     }
-    const int xp = x_ctot / 8, p_full = xp < kGroupPlanes ? xp : kGroupPlanes;
-    const int p_last = xp - kGroupPlanes * (P.a.n_groups - 1);
-    CUtensorMap mxf, mxl, mg;
-    if (!encode_plane_rows_map(&mxf, x, W, H, (long long)n_img * xp, P.a.seg, 3, p_full, why) ||
-        !encode_plane_rows_map(&mxl, x, W, H, (long long)n_img * xp, P.a.seg, 3, p_last, why) ||
-        !encode_plane_rows_map(&mg, g, W, H, (long long)n_img * (g_ctot / 8), P.a.seg, 1, g_ctot / 8, why))
-        return cudaErrorInvalidValue;
-    P.a.partial = static_cast<float*>(scratch);
-    P.a.err = err;
-    cudaError_t e = cudaFuncSetAttribute(wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P.smem);
+    const int sms = device_sms();
+    // the convolutions whose CTAs take longest go first (K-steps of their rows times the width of a step)
+    int order[kWgradMaxLayers];
+    long long work[kWgradMaxLayers];
+    WgradPlan plan[kWgradMaxLayers];
+    for (int k = 0; k < n; ++k) {
+        const WgradConv& c = conv[k];
+        plan[k] = wgrad_plan(c.x_ctot / 8, c.g_ctot / 8, c.n_img, c.H, c.W, sms);
+        const WgradArgs& a = plan[k].a;
+        if (plan[k].smem > kWgSmemMax || c.x_ctot % 8 || c.g_ctot % 16 || c.ci > c.x_ctot || c.co > c.g_ctot ||
+            c.g_ctot / 8 > kMaxGPlanes) {
+            *why = "weight-gradient shape outside the supported range";
+            return cudaErrorInvalidValue;
+        }
+        work[k] = (long long)a.rows_per_cta * ((c.W + a.seg - 1) / a.seg) * a.seg * c.g_ctot;
+        int i = k;
+        for (; i > 0 && work[order[i - 1]] < work[k]; --i) order[i] = order[i - 1];
+        order[i] = k;
+    }
+    size_t smem = 0, off = 0;
+    int blocks = 0, red_blocks = 0;
+    B.n = n;
+    for (int i = 0; i < n; ++i) {
+        const WgradConv& c = conv[order[i]];
+        const WgradPlan& P = plan[order[i]];
+        WgradLayer& L = B.layer[i];
+        L.a = P.a;
+        const int xp = c.x_ctot / 8, p_full = xp < kGroupPlanes ? xp : kGroupPlanes;
+        const int p_last = xp - kGroupPlanes * (L.a.n_groups - 1);
+        const long long xs = (long long)c.n_img * xp, gs = (long long)c.n_img * (c.g_ctot / 8);
+        if (!encode_plane_rows_map(&L.xf, c.x, c.W, c.H, xs, L.a.seg, 3, p_full, why) ||
+            !encode_plane_rows_map(&L.xl, c.x, c.W, c.H, xs, L.a.seg, 3, p_last, why) ||
+            !encode_plane_rows_map(&L.g, c.g, c.W, c.H, gs, L.a.seg, 1, c.g_ctot / 8, why))
+            return cudaErrorInvalidValue;
+        L.a.partial = reinterpret_cast<float*>(static_cast<char*>(scratch) + off);
+        L.a.err = err;
+        L.ci = c.ci;
+        L.co = c.co;
+        L.gw = c.gw;
+        L.n_rb = P.n_rb;
+        L.split = P.n_rb > 24;  // one thread per element while the row blocks are few; else 8 warps per 32 elements
+        L.first = blocks;
+        L.first_red = red_blocks;
+        blocks += P.grid;
+        red_blocks += 3 * c.g_ctot * 128 / (L.split ? 32 : 32 * kReduceWarps) * L.a.n_groups;
+        off += align256(P.partial_bytes);
+        if (P.smem > smem) smem = P.smem;
+    }
+    cudaError_t e = cudaFuncSetAttribute(wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    e = launch_k(wgrad_kernel, P.grid, kWgThreads, P.smem, s, mxf, mxl, mg, P.a);
+    e = launch_k(wgrad_kernel, blocks, kWgThreads, smem, s, B);
     if (e != cudaSuccess) return e;
-    // one thread per element while the row blocks are few; else 8 warps per 32 elements
-    const int per_group = 3 * g_ctot * 128;
-    if (P.n_rb <= 24)
-        return launch_k(wgrad_reduce_kernel<false>, per_group / (32 * kReduceWarps) * P.a.n_groups, 32 * kReduceWarps, 0,
-                        s, P.a, ci, co, P.n_rb, gw);
-    return launch_k(wgrad_reduce_kernel<true>, per_group / 32 * P.a.n_groups, 32 * kReduceWarps, 0, s, P.a, ci, co,
-                    P.n_rb, gw);
+    return launch_k(wgrad_reduce_kernel, red_blocks, 32 * kReduceWarps, 0, s, B);
 }
 
 }  // namespace mcdi

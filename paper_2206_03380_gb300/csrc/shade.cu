@@ -28,32 +28,73 @@ __device__ __forceinline__ f3 cam_origin(const mcdi_camera* cams, int view) {
 }
 
 // ---------------------------------------------------------------- G-buffer
+// A warp casts 4 x 4 pixels (or 16 x 1, 8 x 2, .. 1 x 16 where a narrow image
+// would leave lanes out), so that its rays visit the same nodes; a CTA's four
+// warps lie 2 x 2 (or in a row or a column).
+struct CastTiles {
+    int log_w, log_wx;  // log2 of the warp tile's width and of the warps side by side
+    int nx, ny;         // CTAs per view
+};
+CastTiles cast_tiles(int H, int W) {
+    CastTiles T{2, 1, 0, 0};
+    while (T.log_w < 4 && (8 >> T.log_w) >= H) ++T.log_w;
+    while (T.log_w > 0 && (1 << (T.log_w - 1)) >= W) --T.log_w;
+    if ((1 << T.log_w) >= W) T.log_wx = 0;
+    else if ((16 >> T.log_w) >= H) T.log_wx = 2;
+    T.nx = ((W - 1) >> (T.log_w + T.log_wx)) + 1;
+    T.ny = ((H - 1) >> (6 - T.log_w - T.log_wx)) + 1;
+    return T;
+}
+
+// Whether a ray from o may use the four-wide nodes: a plane's distance is off by
+// up to 3 u |plane - o| and half a quantisation step, and the child boxes are a
+// whole step (at least 2^-17 of the largest coordinate m of the root box) wider
+// on each side, so |o| may be 2^-18 m / 3 u - m = 20 m; 16 m is taken.
+__device__ __forceinline__ bool wide_cast_ok(const BvhNode* __restrict__ nodes, f3 o) {
+    const float4 a = __ldg(&nodes->a), b = __ldg(&nodes->b), c = __ldg(&nodes->c);
+    const float mx = fmaxf(fmaxf(fabsf(a.x), fabsf(a.y)), fmaxf(fabsf(b.x), fabsf(b.y)));
+    const float my = fmaxf(fmaxf(fabsf(a.z), fabsf(a.w)), fmaxf(fabsf(b.z), fabsf(b.w)));
+    const float mz = fmaxf(fmaxf(fabsf(c.x), fabsf(c.y)), fmaxf(fabsf(c.z), fabsf(c.w)));
+    return fmaxf(fabsf(o.x), fmaxf(fabsf(o.y), fabsf(o.z))) <= 16.0f * fmaxf(mx, fmaxf(my, mz));
+}
+
 __global__ void __launch_bounds__(kShadeThreads) primary_cast_kernel(
     const BvhNode* __restrict__ nodes, const TriRecord* __restrict__ tris, int n_tris, const float* __restrict__ verts,
     const float* __restrict__ vnrm, const int* __restrict__ tri_idx, int n_verts, const mcdi_camera* __restrict__ cams,
-    int N, int H, int W, const float4* __restrict__ tex_kd, const float4* __restrict__ tex_korm, int S, float uv_ox,
-    float uv_oz, float uv_s, float4* __restrict__ gb_pos, float4* __restrict__ gb_nrm, float4* __restrict__ gb_kd,
-    float4* __restrict__ gb_korm) {
+    int N, int H, int W, const CastTiles T, const float4* __restrict__ tex_kd, const float4* __restrict__ tex_korm, int S,
+    float uv_ox, float uv_oz, float uv_s, float4* __restrict__ gb_pos, float4* __restrict__ gb_nrm,
+    float4* __restrict__ gb_kd, float4* __restrict__ gb_korm) {
     pdl_prologue();
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (long long)N * H * W) return;
-    const int view = (int)(idx / ((long long)H * W));
-    const int pix = (int)(idx - (long long)view * H * W);
-    const int x = pix % W, y = pix / W;
+    __shared__ float2 stack[(kCastStack + 1) * kShadeThreads / 2];
+    const int per_view = T.nx * T.ny;
+    const int view = blockIdx.x / per_view, tile = blockIdx.x - view * per_view;
+    const int warp = threadIdx.x >> 5, ray_of_warp = (threadIdx.x & 31) >> 1;
+    const int ty = tile / T.nx, tx = tile - ty * T.nx;
+    const int wx = warp & ((1 << T.log_wx) - 1), wy = warp >> T.log_wx;
+    const int x = (((tx << T.log_wx) + wx) << T.log_w) + (ray_of_warp & ((1 << T.log_w) - 1));
+    const int y = (((ty << (2 - T.log_wx)) + wy) << (4 - T.log_w)) + (ray_of_warp >> T.log_w);
+    const bool inside = x < W && y < H;
+    const long long idx = ((long long)view * H + y) * W + x;
     const mcdi_camera& C = cams[view];
     const f3 o = mk(C.origin[0], C.origin[1], C.origin[2]);
     const f3 d = camera_dir(C, x, y, W, H);
+    const RayInv ray = make_ray(o, d);
     float t, u = 0.f, v = 0.f;
-    const int leaf = closest_hit(nodes, tris, n_tris, make_ray(o, d), &t, &u, &v);
+    int leaf = kWideOverflow;
+    if (n_tris > 0 && wide_cast_ok(nodes, o))  // the same for the whole CTA: one view
+        leaf = closest_hit_wide(wide_nodes(nodes, n_tris), tris, ray, inside ? 0 : -1,
+                                stack + (threadIdx.x >> 1) * (kCastStack + 1), &t, &u, &v);
+    if (!inside) return;
+    if (leaf == kWideOverflow) leaf = closest_hit(nodes, tris, n_tris, ray, &t, &u, &v);
     float4 P = make_float4(0.f, 0.f, 0.f, 0.f), Nn = P, KD = P, KORM = P;
     if (leaf >= 0)
         gbuffer_hit(__float_as_int(__ldg(&tris[leaf].v0.w)), u, v, verts, vnrm, tri_idx, n_verts,
                     reinterpret_cast<const float*>(tex_kd), reinterpret_cast<const float*>(tex_korm), S, uv_ox, uv_oz,
                     uv_s, &P, &Nn, &KD, &KORM);
-    gb_pos[idx] = P;
-    gb_nrm[idx] = Nn;
-    gb_kd[idx] = KD;
-    gb_korm[idx] = KORM;
+    // the pair's lanes computed the same; each writes two of the four
+    const bool odd = threadIdx.x & 1;
+    (odd ? gb_nrm : gb_pos)[idx] = odd ? Nn : P;
+    (odd ? gb_korm : gb_kd)[idx] = odd ? KORM : KD;
 }
 
 // ---------------------------------------------------------------- forward
@@ -349,10 +390,10 @@ cudaError_t launch_primary_cast(const void* nodes, const void* tris, int n_tris,
                                 int H, int W, const float* tex_kd, const float* tex_korm, int tex_size, float uv_ox,
                                 float uv_oz, float uv_s, float* gb_pos, float* gb_nrm, float* gb_kd, float* gb_korm,
                                 cudaStream_t stream) {
-    const long long P = (long long)N * H * W;
-    launch_k(primary_cast_kernel, grid_for(P, kShadeThreads), kShadeThreads, 0, stream,
+    const CastTiles T = cast_tiles(H, W);
+    launch_k(primary_cast_kernel, (unsigned)T.nx * (unsigned)T.ny * (unsigned)N, kShadeThreads, 0, stream,
              static_cast<const BvhNode*>(nodes), static_cast<const TriRecord*>(tris), n_tris, verts, vnrm, tri_idx,
-             n_verts, cams, N, H, W, reinterpret_cast<const float4*>(tex_kd), reinterpret_cast<const float4*>(tex_korm),
+             n_verts, cams, N, H, W, T, reinterpret_cast<const float4*>(tex_kd), reinterpret_cast<const float4*>(tex_korm),
              tex_size, uv_ox, uv_oz, uv_s, reinterpret_cast<float4*>(gb_pos), reinterpret_cast<float4*>(gb_nrm),
              reinterpret_cast<float4*>(gb_kd), reinterpret_cast<float4*>(gb_korm));
     return cudaGetLastError();

@@ -409,6 +409,145 @@ __device__ __forceinline__ int closest_hit(const BvhNode* __restrict__ nodes, co
     return best;
 }
 
+// tri_hit with every rounding written out (the products as closest_hit's are contracted)
+__device__ __forceinline__ float tri_hit_rn(f3 o, f3 d, const TriRecord* __restrict__ tris, int k, float* bu, float* bv) {
+    f3 v0, e1, e2;
+    load_record(tris, k, v0, e1, e2);
+    const f3 p = cross_rn(d, e2);
+    const float det = dot_rn(e1, p);
+    if (det == 0.0f) return FLT_MAX;
+    const float inv = 1.0f / det;
+    const f3 s = {__fsub_rn(o.x, v0.x), __fsub_rn(o.y, v0.y), __fsub_rn(o.z, v0.z)};
+    const float u = __fmul_rn(dot_rn(s, p), inv);
+    if (u < 0.0f || u > 1.0f) return FLT_MAX;
+    const f3 q = cross_rn(s, e1);
+    const float v = __fmul_rn(dot_rn(d, q), inv);
+    if (v < 0.0f || __fadd_rn(u, v) > 1.0f) return FLT_MAX;
+    const float t = __fmul_rn(dot_rn(e2, q), inv);
+    if (!(t > 0.0f)) return FLT_MAX;
+    *bu = u;
+    *bv = v;
+    return t;
+}
+
+// closest_hit over the four-wide nodes by pairs of lanes, one ray a pair and two
+// children of its node a lane.  What bounds it is the rays' chains of dependent
+// loads (node, then a leaf's triangle, some 700 cycles each from L2; 15 nodes a
+// ray, 60 for one in a hundred, up to 180) and, with a million triangles, the
+// instructions of warps most of whose rays are done: a pair halves both against a
+// ray per lane (four lanes a ray add more instructions than they hide), and the
+// next node (the nearest inner child, or the nearest pending one) is loaded before
+// the triangles are tested.  Measured, primary_cast of 512 x 512 pixels, 1.18M
+// triangles: 166 us (176 with four lanes, 205 with one; a ray per lane over the
+// two-child nodes 175), 190k triangles, 133 x 77: 86 (71; 127; 115), 157k
+// triangles, 64 x 64: 79 (63; 119; 108).  A persistent tracer that refills lanes
+// leaves too few in flight: 208 to 340.
+// The whole warp calls it and stays together (node: 0, or -1 for a pair without a
+// ray).  Pending nodes and their entry distances are a row of shared memory per
+// ray.  Returns the leaf, the same in both lanes, or kWideOverflow: more pending
+// nodes than the row holds.
+constexpr int kCastStack = 24;
+constexpr int kWideOverflow = -2;
+__device__ __forceinline__ int closest_hit_wide(const WideNode* __restrict__ wn, const TriRecord* __restrict__ tris,
+                                                const RayInv& r, int node, float2* stack, float* t_out, float* bu,
+                                                float* bv) {
+    const unsigned full = 0xffffffffu, none = 0xffffffffu;
+    const int q = threadIdx.x & 1;
+    int best = -1, sp = 0;
+    float tbest = FLT_MAX, tmine = FLT_MAX;  // of the pair, of this lane's children (best, *bu, *bv)
+    const f3 oi = mk(-r.o.x * r.inv.x, -r.o.y * r.inv.y, -r.o.z * r.inv.z);
+    const bool px = r.inv.x >= 0.0f, py = r.inv.y >= 0.0f, pz = r.inv.z >= 0.0f;
+    float4 a, b, c;
+    int2 l = make_int2(0, 0);  // the node, and the links of this lane's children
+    auto load = [&](int k) {
+        asm volatile("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
+                     : "l"(wn + k));
+        c = __ldg(&wn[k].c);
+        l = __ldg(reinterpret_cast<const int2*>(&wn[k].d) + q);
+    };
+    bool overflow = false;
+    if (node >= 0) load(node);
+    while (__any_sync(full, node >= 0)) {  // ends: every four-wide node is visited at most once per ray
+        const uint32_t lox = __float_as_uint(b.z), loy = __float_as_uint(b.w), loz = __float_as_uint(c.x);
+        const uint32_t hix = __float_as_uint(c.y), hiy = __float_as_uint(c.z), hiz = __float_as_uint(c.w);
+        const uint32_t nx = (px ? lox : hix) >> (16 * q), fx = (px ? hix : lox) >> (16 * q);
+        const uint32_t ny = (py ? loy : hiy) >> (16 * q), fy = (py ? hiy : loy) >> (16 * q);
+        const uint32_t nz = (pz ? loz : hiz) >> (16 * q), fz = (pz ? hiz : loz) >> (16 * q);
+        const float ax = a.w * r.inv.x, ay = b.x * r.inv.y, az = b.y * r.inv.z;
+        const float bx = fmaf(-8388608.0f, ax, fmaf(a.x, r.inv.x, oi.x));
+        const float by = fmaf(-8388608.0f, ay, fmaf(a.y, r.inv.y, oi.y));
+        const float bz = fmaf(-8388608.0f, az, fmaf(a.z, r.inv.z, oi.z));
+        const float2 ax2 = {ax, ax}, bx2 = {bx, bx}, ay2 = {ay, ay}, by2 = {by, by}, az2 = {az, az}, bz2 = {bz, bz};
+        const float2 x0 = fma2({qbyte(nx, 0), qbyte(nx, 1)}, ax2, bx2), x1 = fma2({qbyte(fx, 0), qbyte(fx, 1)}, ax2, bx2);
+        const float2 y0 = fma2({qbyte(ny, 0), qbyte(ny, 1)}, ay2, by2), y1 = fma2({qbyte(fy, 0), qbyte(fy, 1)}, ay2, by2);
+        const float2 z0 = fma2({qbyte(nz, 0), qbyte(nz, 1)}, az2, bz2), z1 = fma2({qbyte(fz, 0), qbyte(fz, 1)}, az2, bz2);
+        const float ta = fmax3(x0.x, y0.x, fmaxf(z0.x, 0.0f)), tb = fmax3(x0.y, y0.y, fmaxf(z0.y, 0.0f));
+        const bool hita = node >= 0 && ta <= fmin3(x1.x, y1.x, fminf(z1.x, tbest));
+        const bool hitb = node >= 0 && tb <= fmin3(x1.y, y1.y, fminf(z1.y, tbest));
+        // inner children by entry distance, ties by child
+        const uint32_t ka = hita && l.x >= 0 ? (__float_as_uint(ta) & ~3u) | (uint32_t)(2 * q) : none;
+        const uint32_t kb = hitb && l.y >= 0 ? (__float_as_uint(tb) & ~3u) | (uint32_t)(2 * q + 1) : none;
+        const uint32_t kc = __shfl_xor_sync(full, ka, 1), kd = __shfl_xor_sync(full, kb, 1);
+        const uint32_t first = min(min(ka, kb), min(kc, kd));
+        const int n_in = (ka != none) + (kb != none) + (kc != none) + (kd != none);
+        int leafa = hita && l.x < 0 ? ~l.x : -1, leafb = hitb && l.y < 0 ? ~l.y : -1;
+        int next = __shfl_sync(full, first & 1u ? l.y : l.x, (threadIdx.x & 30) | (int)(first >> 1 & 1u));
+        float tnext = __uint_as_float(first);
+        if (sp + 3 > kCastStack) overflow = true;
+        if (n_in > 1 && !overflow) {
+            const int top = sp + n_in - 1;
+            const int ra = (kb < ka) + (kc < ka) + (kd < ka), rb = (ka < kb) + (kc < kb) + (kd < kb);
+            if (ka != none && ra > 0) stack[top - ra] = make_float2(__uint_as_float(ka), __int_as_float(l.x));
+            if (kb != none && rb > 0) stack[top - rb] = make_float2(__uint_as_float(kb), __int_as_float(l.y));
+            sp = top;
+        }
+        __syncwarp();
+        if (n_in == 0) {
+            next = -1;
+            while (sp > 0 && next < 0) {  // the nearest pending node not behind the hit
+                const float2 e = stack[--sp];
+                if (e.x <= tbest) next = __float_as_int(e.y), tnext = e.x;
+            }
+        }
+        if (overflow || node < 0) next = -1, sp = 0;
+        node = next;
+        if (node >= 0) load(node);
+        if (__any_sync(full, leafa >= 0 || leafb >= 0)) {
+            float t = FLT_MAX;
+            do {
+                const int k = leafa >= 0 ? leafa : leafb;
+                if (leafa >= 0) leafa = -1;
+                else leafb = -1;
+                if (k >= 0) {
+                    float u, v;
+                    t = fminf(t, tri_hit_rn(r.o, r.d, tris, k, &u, &v));
+                    if (t < tmine) tmine = t, best = k, *bu = u, *bv = v;
+                }
+                __syncwarp();
+            } while (__any_sync(full, leafb >= 0));
+            tbest = fminf(tbest, fminf(t, __shfl_xor_sync(full, t, 1)));
+            if (node >= 0 && tnext > tbest) {  // behind the new hit: and so may be the pending ones
+                node = -1;
+                while (sp > 0 && node < 0) {
+                    const float2 e = stack[--sp];
+                    if (e.x <= tbest) node = __float_as_int(e.y);
+                }
+                if (node >= 0) load(node);
+            }
+            __syncwarp();
+        }
+    }
+    // the pair's nearest hit: its lane's leaf and barycentrics
+    const unsigned who = __ballot_sync(full, best >= 0 && tmine == tbest) >> (threadIdx.x & 30) & 3u;
+    const int src = (threadIdx.x & 30) | (who == 2u ? 1 : 0);
+    best = __shfl_sync(full, best, src);
+    *bu = __shfl_sync(full, *bu, src);
+    *bv = __shfl_sync(full, *bv, src);
+    *t_out = tbest;
+    return overflow ? kWideOverflow : best;
+}
+
 // ---------------------------------------------------------------- probe
 // largest k in [0, n-1] with cdf[k] <= u
 __device__ __forceinline__ int upper_index(const float* __restrict__ cdf, int n, float u) {

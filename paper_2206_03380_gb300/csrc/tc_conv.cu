@@ -270,7 +270,7 @@ __device__ __forceinline__ void epilogue16(const ConvParams& p, const uint32_t* 
 
 // Publish a thread's running max |value| of the stored output: rounded to BF16
 // like the stored values (rounding is monotonic, so this is the max over the
-// stored tensor), reduced over the warp, one atomic per warp.
+// stored tensor), reduced over the warp, one atomic per warp while the maximum grows.
 __device__ __forceinline__ void publish_amax(unsigned* out_amax, float m, unsigned mask) {
     if (out_amax == nullptr) return;
     const unsigned b = __float_as_uint(__bfloat162float(__float2bfloat16_rn(m)));
@@ -518,7 +518,7 @@ __device__ __forceinline__ void publish_amax2(unsigned* out_amax, uint32_t am) {
     if (out_amax == nullptr) return;
     const unsigned hi = am & 0xffff0000u, lo = am << 16;  // the two halves as floats' bits (non-negative)
     const unsigned w = __reduce_max_sync(0xffffffffu, hi > lo ? hi : lo);
-    if ((threadIdx.x & 31) == 0 && w) atomicMax(out_amax, w);
+    if ((threadIdx.x & 31) == 0 && w > *(volatile const unsigned*)out_amax) atomicMax(out_amax, w);
 }
 // 32 bytes (two neighbouring pixels of an 8-channel plane) in one access: whole sectors, half the instructions
 struct Words8 {

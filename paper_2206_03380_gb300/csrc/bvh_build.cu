@@ -915,7 +915,7 @@ cudaError_t launch_build_bvh(const float* verts, int n_verts, const int* tris, i
     uint32_t* dtot = reinterpret_cast<uint32_t*>(s + L.digit_tot);
     int* parent_int = reinterpret_cast<int*>(s + L.parent_int);
     int* parent_leaf = reinterpret_cast<int*>(s + L.parent_leaf);
-    uint32_t* room = reinterpret_cast<uint32_t*>(s + L.flags);
+    uint32_t* room = reinterpret_cast<uint32_t*>(s + L.run_boxes);
     float4* box_int = reinterpret_cast<float4*>(s + L.box_int);
     float4* box_leaf = reinterpret_cast<float4*>(s + L.box_leaf);
     BvhNode* nodes = static_cast<BvhNode*>(nodes_v);
@@ -969,7 +969,7 @@ cudaError_t launch_refit_bvh(const float* verts, int n_verts, const int* tris, i
     const uint32_t* order = reinterpret_cast<const uint32_t*>(s + (kSortPasses % 2 ? L.vals1 : L.vals0));
     int* parent_int = reinterpret_cast<int*>(s + L.parent_int);
     int* parent_leaf = reinterpret_cast<int*>(s + L.parent_leaf);
-    uint32_t* room = reinterpret_cast<uint32_t*>(s + L.flags);
+    uint32_t* room = reinterpret_cast<uint32_t*>(s + L.run_boxes);
     float4* box_int = reinterpret_cast<float4*>(s + L.box_int);
     float4* box_leaf = reinterpret_cast<float4*>(s + L.box_leaf);
     BvhNode* nodes = static_cast<BvhNode*>(nodes_v);

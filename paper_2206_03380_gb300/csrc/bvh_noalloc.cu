@@ -13,7 +13,7 @@
 // is being captured (the first call in a context must come before any
 // capture).  All calls in a context share the array and it keeps the previous
 // call's contents; the build writes every scratch word it later reads
-// (bounds, histograms, parents, arrival counters, boxes), so nothing needs
+// (bounds, histograms, parents, boxes), so nothing needs
 // clearing between calls.  Calls whose work overlaps on the GPU (two streams,
 // or two host threads) race on the array and must be serialised by the
 // caller.

@@ -12,7 +12,7 @@ namespace mcdi {
 
 // ---- BVH build scratch layout (offsets in bytes, 256-byte aligned) ----
 struct BvhScratch {
-    size_t bounds, keys0, keys1, vals0, vals1, hist, digit_tot, parent_int, parent_leaf, flags, box_int, box_leaf;
+    size_t bounds, keys0, keys1, vals0, vals1, hist, digit_tot, parent_int, parent_leaf, run_boxes, box_int, box_leaf;
     size_t total;
     int nblocks;  // radix-sort tiles
 };
@@ -50,7 +50,7 @@ constexpr BvhScratch bvh_scratch_layout(int n) {
     s.digit_tot = o; o = align256(o + ((size_t)1 << kSortDigitBits) * sizeof(uint32_t));
     s.parent_int = o; o = align256(o + ni * sizeof(int));
     s.parent_leaf = o; o = align256(o + un * sizeof(int));
-    s.flags = o; o = align256(o + ni * sizeof(uint32_t));
+    s.run_boxes = o; o = align256(o + ni * sizeof(uint32_t));  // boxes of 32 leaves and of runs, 34 bytes per 32 leaves
     s.box_int = o; o = align256(o + ni * 2 * sizeof(float4));
     s.box_leaf = o; o = align256(o + un * 2 * sizeof(float4));
     s.total = o;

@@ -21,6 +21,8 @@
 // of each key by atomicMin), then an ordered compaction.
 #include <limits.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "internal.h"
 #include "shading.cuh"
@@ -325,26 +327,29 @@ __device__ __forceinline__ bool draw_edge_sample(const ShadeArgs& a, const float
     return true;
 }
 
-// A CTA owns a run of kRounds * kGradThreads (pixel, edge sample) pairs.  Its
+// A CTA owns a run of rounds * kGradThreads (pixel, edge sample) pairs.  Its
 // threads draw them, a round of one each at a time; the few that are candidates
 // (silhouette, above the horizon: 0.2% of the samples of the mesh below) append
 // their outer ray in shared memory, and when a round might overflow the list,
 // or after the last, all lanes trace the list (trace_rays) and the samples whose
 // ray is open are drawn again and scattered.  What bounds it is the latency of
-// the samples' gathers (60%), then of the grazing outer rays' node chains; a
-// run of 4096 keeps the ends of runs few and still gives each SM its 7 CTAs.
-// Measured, 4.2M samples (512 x 512, 16 each) of 297k edges: 160 us (the whole
-// warp walking one outer ray at a time over the depth-first nodes: 243).
-constexpr int kRounds = 32;
+// the samples' gathers (60%), then of the grazing outer rays' node chains.  Runs
+// are as long as 32 rounds where that still gives each SM its 7 CTAs (their ends
+// are then few), down to one round where the samples are few: of 300 x 400 x 9
+// samples in 8 rounds 82 us, of 200 x 150 x 2 in one 61 (the whole warp walking
+// one outer ray at a time over the depth-first nodes, a sample per thread: 153
+// and 91).  Measured, 4.2M samples (512 x 512, 16 each) of 297k edges: 157 us
+// (243).
+constexpr int kMaxRounds = 32, kGradBlocksPerSM = 7;
 
 __global__ void __launch_bounds__(kGradThreads) shadow_edge_grad_kernel(
     ShadeArgs a, const float* __restrict__ verts, int n_verts, const int4* __restrict__ edges,
     const int* __restrict__ n_edges_dev, int max_edges, int M, float eta, const float4* __restrict__ g_cd,
-    const float4* __restrict__ g_cs, float* g_verts, float* sample_w) {
+    const float4* __restrict__ g_cs, float* g_verts, float* sample_w, int rounds) {
     pdl_prologue();
     __shared__ OuterRays rays;
     const long long P = (long long)a.N * a.H * a.W, total = P * M;
-    const long long run0 = (long long)blockIdx.x * (kRounds * kGradThreads);
+    const long long run0 = (long long)blockIdx.x * (rounds * kGradThreads);
     const int lane = threadIdx.x & 31;
     const int E = min(max(*n_edges_dev, 0), max_edges);
     // pixel, view and sample of the run's pair k, by 32-bit divisions from the run's first
@@ -359,6 +364,11 @@ __global__ void __launch_bounds__(kGradThreads) shadow_edge_grad_kernel(
         *pix = p - v * HW;
     };
     auto flush = [&]() {  // whole CTA, after a barrier
+        if (rays.pending() == 0u) return;
+        if (rays.pending() <= OuterRays::kSplit) {
+            if (threadIdx.x == 0) rays.find_parts(a.nodes, a.n_tris);
+            __syncthreads();
+        }
         trace_rays(a.nodes, static_cast<const TriRecord*>(a.tris), a.n_tris, rays.stacks, rays);
         __syncthreads();
         const unsigned n = rays.n;
@@ -408,8 +418,7 @@ __global__ void __launch_bounds__(kGradThreads) shadow_edge_grad_kernel(
         if (threadIdx.x < OuterRays::kCap / 32) rays.hit[threadIdx.x] = 0u;
     };
     clear();
-    if (threadIdx.x == 0) rays.find_parts(a.nodes, a.n_tris);
-    if (threadIdx.x == 32) {
+    if (threadIdx.x == 0) {
         s_idx = run0 / M;
         const long long view = s_idx / HW;
         s_first[0] = (unsigned)(run0 - s_idx * M);
@@ -417,7 +426,7 @@ __global__ void __launch_bounds__(kGradThreads) shadow_edge_grad_kernel(
         s_first[2] = (unsigned)view;
     }
     __syncthreads();
-    for (int r = 0; r < kRounds; ++r) {
+    for (int r = 0; r < rounds; ++r) {
         const int k = r * kGradThreads + threadIdx.x;
         const long long tid = run0 + k;
         EdgeSample S;
@@ -444,10 +453,10 @@ __global__ void __launch_bounds__(kGradThreads) shadow_edge_grad_kernel(
         }
         __syncthreads();
         const bool full = rays.pending() > OuterRays::kCap - kGradThreads;
-        if (full || r == kRounds - 1) {
+        if (full || r == rounds - 1) {
             flush();
             __syncthreads();
-            if (r == kRounds - 1) break;
+            if (r == rounds - 1) break;
             clear();
         }
         __syncthreads();  // every thread has read the count before the next round adds to it
@@ -513,9 +522,16 @@ cudaError_t launch_shadow_edge_grad(const ShadeArgs& a, const float* verts, int 
                                     const float4* g_cs, float* g_verts, float* sample_w, cudaStream_t stream) {
     const long long n = (long long)a.N * a.H * a.W * n_samples;
     if (n <= 0) return cudaGetLastError();
-    const long long run = kRounds * kGradThreads;
+    // the longest runs that still give every SM its CTAs
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const long long resident = (long long)sms * kGradBlocksPerSM * kGradThreads;
+    const int rounds = (int)std::min<long long>(std::max<long long>(n / resident, 1), kMaxRounds);
+    const long long run = (long long)rounds * kGradThreads;
     launch_k(shadow_edge_grad_kernel, (int)((n + run - 1) / run), kGradThreads, 0, stream, a, verts,
-             n_verts, edges, n_edges, max_edges, n_samples, eta, g_cd, g_cs, g_verts, sample_w);
+             n_verts, edges, n_edges, max_edges, n_samples, eta, g_cd, g_cs, g_verts, sample_w, rounds);
     return cudaGetLastError();
 }
 

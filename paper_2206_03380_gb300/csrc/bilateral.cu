@@ -22,7 +22,7 @@
 // exponentials are one (base 2), slopes are
 // staged in the backward instead of formed per weight, and uncovered neighbours
 // (zero normal and colours) take no branch.  Measured, two images: 512 x 512,
-// sigma 2: forward 44 us, backward 49; 3 x 700 x 611, sigma 3.9: 313 and 397
+// sigma 2: forward 45 us, backward 50; 3 x 700 x 611, sigma 3.9: 324 and 410
 // (a pixel per thread, two exponentials and a division per weight, a branch per
 // neighbour: 63 and 81, 630 and 816).  Four pixels per thread halve the loads
 // but leave too few warps: 56 and 57, 377 and 480.

@@ -25,7 +25,11 @@ namespace mcdi {
 namespace {
 
 constexpr int kGenThreads = 128;
-constexpr int kGenBlocksPerSM = 9;  // 56 registers, no spills; 7 and 8: 4% slower, 10 spills: 2% slower
+// CTAs of sample generation per SM: 9 (56 registers) for grids of at least four
+// waves, 8 (64 registers) below, where fewer and shorter waves count more.
+// Measured (8 / 9): 160,000 CTAs of 32 samples 3047 / 2985 us, 8,192 of 16 101 /
+// 100, 3,088 of 27 55 / 58, 2,233 of 38 67 / 74; 7 and 10 are slower than either.
+constexpr int kGenBlocks = 9, kGenBlocksSmall = 8;
 constexpr int kTraceBlocksPerSM = 8;  // 7: the same; 9 and 10 spill: 5% and 15% slower
 
 struct WaveBuffers {
@@ -89,7 +93,8 @@ __global__ void wave_reset_kernel(void* ws, long long P, long long slots) {
 // depend on which warp drew it.
 constexpr int kGenQuarters = kGenThreads / 32;
 
-__global__ void __launch_bounds__(kGenThreads, kGenBlocksPerSM) wave_gen_kernel(ShadeArgs a, void* ws,
+template <int kBlocks>
+__global__ void __launch_bounds__(kGenThreads, kBlocks) wave_gen_kernel(ShadeArgs a, void* ws,
                                                                   float4* __restrict__ kd_out) {
     pdl_prologue();
     extern __shared__ float s_marg[];
@@ -334,15 +339,16 @@ cudaError_t launch_shade_fwd_wave(const ShadeArgs& a, float4* c_d, float4* kd_ou
     const long long P = (long long)a.N * a.H * a.W;
     const int spp = a.n_light + a.n_cos + a.n_ggx;
     const int gblocks = (int)((P + kGenThreads - 1) / kGenThreads);
-    if (parts & 1) {
-        launch_k(wave_reset_kernel, 1, 1, 0, stream, ws, P, P * spp);
-        launch_k(wave_gen_kernel, (int)((P + 31) / 32), kGenThreads, (size_t)(a.Hp + 1) * sizeof(float), stream, a,
-                 ws, kd_out);
-    }
-    if (!(parts & 2)) return cudaGetLastError();
     int dev = 0, sms = 152, per_sm = 8;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (parts & 1) {
+        launch_k(wave_reset_kernel, 1, 1, 0, stream, ws, P, P * spp);
+        const int blocks = (int)((P + 31) / 32);
+        launch_k(blocks < 4 * kGenBlocks * sms ? wave_gen_kernel<kGenBlocksSmall> : wave_gen_kernel<kGenBlocks>, blocks,
+                 kGenThreads, (size_t)(a.Hp + 1) * sizeof(float), stream, a, ws, kd_out);
+    }
+    if (!(parts & 2)) return cudaGetLastError();
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, wave_trace_kernel, kTraceThreads, 0);
     if (per_sm < 1) per_sm = 1;
     launch_k(wave_trace_kernel, sms * per_sm, kTraceThreads, 0, stream, a.nodes, static_cast<const TriRecord*>(a.tris),

@@ -661,11 +661,27 @@ def time_denoiser_e4m3(pipe, den_params, conv_flops, flush, stream, steps):
     return out
 
 
+def wgrad_groups(den):
+    """How many groups the 15 convolutions share launches in: as many in a row as the scratch holds partial sums of
+    (channels of the input and of the gradient, level)."""
+    from paper_2206_03380_gb300 import mcdi
+
+    convs = [(16, 32, 0), (32, 32, 0), (32, 48, 1), (48, 48, 1), (48, 64, 2), (64, 64, 2), (64, 96, 3), (96, 96, 3),
+             (160, 64, 2), (64, 64, 2), (112, 48, 1), (48, 48, 1), (80, 32, 0), (32, 32, 0), (32, 16, 0)]
+    room, groups, used = mcdi.denoise_wgrad_bytes(den.n_img, den.H, den.W), 1, 0
+    for ci, co, lv in convs:
+        need = mcdi.conv3x3_wgrad_bytes(den.n_img, den.H >> lv, den.W >> lv, ci, co)
+        if used and used + need > room:
+            groups, used = groups + 1, 0
+        used += need
+    return groups
+
+
 def time_denoiser_wgrad(den, conv_flops, flush, stream, steps):
     """The denoiser's weight gradient (the live-trained variant, App. B; not part of the timed
-    step, whose denoiser weights are locked) after the step's forward and input gradient: 15
-    tcgen05 weight-gradient launches and 15 deterministic reductions, CUDA events, L2 flushed
-    before each pass.  FLOPs: the forward's (2 * 9 * c_in * c_out per pixel and convolution)."""
+    step, whose denoiser weights are locked) after the step's forward and input gradient: a
+    tcgen05 weight-gradient launch and a deterministic reduction per group of convolutions, CUDA
+    events, L2 flushed before each pass.  FLOPs: the forward's (2 * 9 * c_in * c_out per pixel and convolution)."""
     import torch
 
     gw = den.weight_grad(stream=stream)
@@ -685,7 +701,7 @@ def time_denoiser_wgrad(den, conv_flops, flush, stream, steps):
     tpeak, tkind = tensor_peak()
     tf = conv_flops / (t * 1e-3) / 1e12
     return {"ms": round(t, 4), "tflops": round(tf, 2), "peak": tpeak, "frac": round(tf / tpeak, 4),
-            "peak_source": tkind, "launches": 30, "finite": bool(torch.isfinite(gw).all().item()),
+            "peak_source": tkind, "launches": 2 * wgrad_groups(den), "finite": bool(torch.isfinite(gw).all().item()),
             "note": "dW and db of the 15 convolutions for the step's loss; off the timed step (locked weights)"}
 
 

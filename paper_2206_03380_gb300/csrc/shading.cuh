@@ -100,8 +100,6 @@ __device__ __forceinline__ float tri_hit(const RayInv& r, const TriRecord* __res
     return tri_hit_v(r, xyz(v0), xyz(e1), xyz(e2), bu, bv);
 }
 
-// The same test of a shadow ray (hit or not) with every rounding written out
-// (the products of tri_hit_v as the compiler contracts them).
 // Triangle record k in two loads: records are 48 bytes apart on 16-byte
 // boundaries, so either their first 32 bytes or their last 32 start on a
 // 32-byte boundary.  (Each load of a lane is one L1 wavefront when lanes read
@@ -118,6 +116,9 @@ __device__ __forceinline__ void load_record(const TriRecord* __restrict__ tris, 
     e1 = odd ? xyz(x) : xyz(y);
     e2 = odd ? xyz(y) : xyz(z);
 }
+
+// The same test of a shadow ray (hit or not) with every rounding written out
+// (the products of tri_hit_v as the compiler contracts them).
 __device__ __forceinline__ bool tri_blocks(f3 o, f3 d, const TriRecord* __restrict__ tris, int k) {
     f3 v0, e1, e2;
     load_record(tris, k, v0, e1, e2);

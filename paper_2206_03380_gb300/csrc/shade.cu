@@ -78,14 +78,16 @@ __global__ void __launch_bounds__(kShadeThreads) primary_cast_kernel(
     const mcdi_camera& C = cams[view];
     const f3 o = mk(C.origin[0], C.origin[1], C.origin[2]);
     const f3 d = camera_dir(C, x, y, W, H);
+    // a degenerate camera's NaN passes every box test (minimum and maximum drop it) and no triangle's: a miss
+    const bool live = inside && finite_ray(o, d);
     const RayInv ray = make_ray(o, d);
     float t, u = 0.f, v = 0.f;
     int leaf = kWideOverflow;
     if (n_tris > 0 && wide_cast_ok(nodes, o))  // the same for the whole CTA: one view
-        leaf = closest_hit_wide(wide_nodes(nodes, n_tris), tris, ray, inside ? 0 : -1,
+        leaf = closest_hit_wide(wide_nodes(nodes, n_tris), tris, n_tris, ray, live ? 0 : -1,
                                 stack + (threadIdx.x >> 1) * (kCastStack + 1), &t, &u, &v);
     if (!inside) return;
-    if (leaf == kWideOverflow) leaf = closest_hit(nodes, tris, n_tris, ray, &t, &u, &v);
+    if (leaf == kWideOverflow) leaf = live ? closest_hit(nodes, tris, n_tris, ray, &t, &u, &v) : -1;
     float4 P = make_float4(0.f, 0.f, 0.f, 0.f), Nn = P, KD = P, KORM = P;
     if (leaf >= 0)
         gbuffer_hit(__float_as_int(__ldg(&tris[leaf].v0.w)), u, v, verts, vnrm, tri_idx, n_verts,

@@ -59,6 +59,13 @@ __device__ __forceinline__ RayInv make_ray(f3 o, f3 d) {
     return r;
 }
 
+// whether neither the ray's origin nor its direction has a NaN or an infinity
+__device__ __forceinline__ bool finite_ray(f3 o, f3 d) {
+    const float big = 3.402823466e38f;
+    return fabsf(o.x) <= big && fabsf(o.y) <= big && fabsf(o.z) <= big && fabsf(d.x) <= big && fabsf(d.y) <= big &&
+           fabsf(d.z) <= big;
+}
+
 // slab test of one box given as (lo.x, hi.x, lo.y, hi.y) + (lo.z, hi.z);
 // returns the entry distance or +inf on a miss.  The exit distance is scaled by
 // 1 + 2 gamma_3 so that rounding never drops a box the ray touches (Ize 2013).
@@ -444,14 +451,16 @@ __device__ __forceinline__ float tri_hit_rn(f3 o, f3 d, const TriRecord* __restr
 // triangles, 64 x 64: 79 (63; 119; 108).  A persistent tracer that refills lanes
 // leaves too few in flight: 208 to 340.
 // The whole warp calls it and stays together (node: 0, or -1 for a pair without a
-// ray).  Pending nodes and their entry distances are a row of shared memory per
+// ray).  An empty slot's box is inverted, which rejects every finite ray; its link
+// is checked all the same before it becomes a triangle's
+// index.  Pending nodes and their entry distances are a row of shared memory per
 // ray.  Returns the leaf, the same in both lanes, or kWideOverflow: more pending
 // nodes than the row holds.
 constexpr int kCastStack = 24;
 constexpr int kWideOverflow = -2;
 __device__ __forceinline__ int closest_hit_wide(const WideNode* __restrict__ wn, const TriRecord* __restrict__ tris,
-                                                const RayInv& r, int node, float2* stack, float* t_out, float* bu,
-                                                float* bv) {
+                                                int n_tris, const RayInv& r, int node, float2* stack, float* t_out,
+                                                float* bu, float* bv) {
     const unsigned full = 0xffffffffu, none = 0xffffffffu;
     const int q = threadIdx.x & 1;
     int best = -1, sp = 0;
@@ -492,7 +501,9 @@ __device__ __forceinline__ int closest_hit_wide(const WideNode* __restrict__ wn,
         const uint32_t kc = __shfl_xor_sync(full, ka, 1), kd = __shfl_xor_sync(full, kb, 1);
         const uint32_t first = min(min(ka, kb), min(kc, kd));
         const int n_in = (ka != none) + (kb != none) + (kc != none) + (kd != none);
-        int leafa = hita && l.x < 0 ? ~l.x : -1, leafb = hitb && l.y < 0 ? ~l.y : -1;
+        // (an inner link's complement is negative, an empty slot's beyond every triangle)
+        int leafa = hita && (unsigned)~l.x < (unsigned)n_tris ? ~l.x : -1;
+        int leafb = hitb && (unsigned)~l.y < (unsigned)n_tris ? ~l.y : -1;
         int next = __shfl_sync(full, first & 1u ? l.y : l.x, (threadIdx.x & 30) | (int)(first >> 1 & 1u));
         float tnext = __uint_as_float(first);
         if (sp + 3 > kCastStack) overflow = true;

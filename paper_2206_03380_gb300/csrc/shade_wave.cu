@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(kTraceThreads) wave_stats_kernel(const void* _
         int node = 0, sp = 0;
         for (int it = 0; it < 2 * n_tris && node >= 0; ++it) {
             ++c[1];
-            node = wide_step<1, true>(wn, tris, r, node, stack, sp, overflow, &tests);
+            node = wide_step<1, true>(wn, tris, n_tris, r, node, stack, sp, overflow, &tests);
         }
         blocked = node == kWideBlocked || (node >= 0 || overflow ? any_hit_threaded(nodes, tris, n_tris, r) : false);
         c[0] += 1;

@@ -249,10 +249,11 @@ __device__ __forceinline__ unsigned wide_child_hits(const RayInv& r, float4 a, f
 // or kWideDone.  Stack entry i lives at stack[i * kStride] (a thread's column
 // of a shared-memory array, or a local array); a push beyond kWideStack sets
 // *overflow instead (the caller then decides the ray by the stackless walk);
-// kCount adds the triangle tests made to *tri_tests.
+// kCount adds the triangle tests made to *tri_tests.  A ray with infinite
+// coordinates meets empty slots too: their links are no triangle's.
 template <int kStride = 1, bool kCount = false>
 __device__ __forceinline__ int wide_step(const WideNode* __restrict__ wn, const TriRecord* __restrict__ tris,
-                                         const RayInv& r, int node, int* stack, int& sp, bool& overflow,
+                                         int n_tris, const RayInv& r, int node, int* stack, int& sp, bool& overflow,
                                          unsigned* tri_tests = nullptr) {
     float4 a, b, c;
     int4 d;
@@ -283,6 +284,7 @@ __device__ __forceinline__ int wide_step(const WideNode* __restrict__ wn, const 
         const int k = __ffs(leaves) - 1;
         leaves &= leaves - 1;
         const int l = k == 0 ? d.x : k == 1 ? d.y : k == 2 ? d.z : d.w;
+        if ((unsigned)~l >= (unsigned)n_tris) continue;
         if (kCount) ++*tri_tests;
         if (tri_blocks(r.o, r.d, tris, ~l)) return kWideBlocked;
     }

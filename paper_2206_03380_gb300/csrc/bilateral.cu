@@ -13,6 +13,8 @@
 // same weights.  Backward: the transpose as a gather, g(q) = sum_p g(p) w(p, q)
 // / W(p) over the footprint of q, with W saved by the forward (no atomics, so
 // the gradient is deterministic).
+#include <type_traits>
+
 #include "internal.h"
 
 namespace mcdi {
@@ -61,11 +63,12 @@ struct Center {  // the pixel p of a weight w(p, q)
     float z, gx, gy, eps, nx, ny, nz;
 };
 
+// (the sums' roundings written out: weight_pair forms the same bits)
 __device__ __forceinline__ float bilateral_weight(const Center& p, const Guide& q, int dx, int dy, float inv2s2) {
     const float ws = expf(-(float)(dx * dx + dy * dy) * inv2s2);
-    const float pred = fabsf(p.gx * (float)dx + p.gy * (float)dy);
+    const float pred = fabsf(__fmaf_rn(p.gy, (float)dy, __fmul_rn(p.gx, (float)dx)));
     const float wz = expf(-fabsf(p.z - q.z) / (kSigmaZ * pred + p.eps));
-    const float wn = pow128(p.nx * q.nx + p.ny * q.ny + p.nz * q.nz);
+    const float wn = pow128(__fmaf_rn(p.nz, q.nz, __fmaf_rn(p.ny, q.ny, __fmul_rn(p.nx, q.nx))));
     return ws * wz * wn;
 }
 
@@ -156,45 +159,64 @@ __global__ void __launch_bounds__(kTile* kTile) bilateral_fwd_kernel(const float
 // column; guides and the upstream gradients divided by W(p) over the tile plus its
 // halo are staged in shared memory, and from the guides every staged pixel's
 // slopes.  What bounds it is three things at about the same level, per weight and
-// warp: some 30 issued instructions, 2 MUFU operations (16 cycles of a scheduler)
-// and shared-memory wavefronts (14 per neighbour for two images), then the
-// staging's latency.  So a neighbour loaded once meets two pixels, their
-// arithmetic goes in packed pairs, the two exponentials are one (base 2), and
-// uncovered neighbours (zero normal and gradients) take no branch.  Measured, two
-// images: 512 x 512, sigma 2: 50 us; 3 x 700 x 611, sigma 3.9: 410 (a pixel per
-// thread, slopes formed per weight, two exponentials, a division and a branch:
-// 81 and 816).  Four pixels per thread halve the loads but leave too few warps: 57
-// and 480.  The forward is not built this way: its images go through an absolute
-// difference next (image_loss), whose gradient is a sign, so a last bit of them is
-// a whole gradient, and with the factors rounded as they are above two pixels per
-// thread gain nothing (66 and 503 us against 63 and 631, 27 against 22 at 133 x 77).
+// warp: some 45 issued instructions, 3 MUFU operations and shared-memory
+// wavefronts (16 per neighbour for two images), then the staging's latency.  So a
+// neighbour loaded once meets two pixels, their arithmetic goes in packed pairs,
+// the spatial factors come from a table, the division takes no branch, and
+// uncovered neighbours (zero normal and gradients) take none either.  Every
+// operation is rounded as in bilateral_weight, so the weights are the forward's,
+// bit for bit.  Measured, two images: 512 x 512, sigma 2: 36 us; 3 x 700 x 611,
+// sigma 3.9: 408 (a pixel per thread, slopes formed per weight, two exponentials,
+// a division and a branch: 68 and 824; with an approximate quotient and one
+// approximate exponential 34 and 377, whose weights are off by up to twice as
+// much: not taken).  The gradient's error against 64 bits, with the loss before
+// it, is 0.5 to 12% below either of theirs over ten shapes.  The forward is not built this way: two pixels per thread gain
+// it nothing (66 and 503 us against 63 and 631, 27 against 22 at 133 x 77).
 constexpr int kTileW = 32;
 constexpr int kRows = 2;  // pixels of a thread, in one column
-constexpr int kUnroll = 3;
-// Warps of a CTA: 4, or 8 from radius 7, where the staged halo leaves an SM room
-// for 12 warps in CTAs of 4 and 16 in CTAs of 8.  Measured (4 / 8 warps): radius 8,
-// 3 x 700 x 611: 438 / 373 us; radius 4, 512 x 512: 47 / 53 us (fewer, larger CTAs
-// level the coverage less).
-constexpr int kMaxWarps = 8, kWideRadius = 6;
-constexpr float kLog2E = 1.44269504088896341f;
+constexpr int kUnroll = 4;  // 3: 3 to 8% slower, 5 and 6: 2 to 10%
+// Warps of a CTA: 8, whose tiles share more of their halo, or 4 where CTAs of 4 do
+// not outnumber the SMs and fewer would leave some idle.  Measured (4 / 8 warps), two
+// images: 133 x 77, radius 8: 34 / 41 us, radius 4: 15.7 / 17.4; 256 x 256: 18.9 /
+// 17.5; 512 x 512: 35.8 / 36.0; 3 x 700 x 611, radius 8: 469 / 405; 4 x 800 x 800,
+// radius 5: 366 / 320.
+constexpr int kMaxWarps = 8;
+// Depths for which weight_pair's divisors (from 1e-3 of one to 17 times the largest) stay in div_pair's range.
+constexpr float kPlainMin = 0x1p-40f, kPlainMax = 0x1p40f;
 
-__device__ __forceinline__ float exp2_approx(float x) {
-    float r;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
 __device__ __forceinline__ float2 both(float v) { return make_float2(v, v); }
 
-// Two weights: spatial part of the argument (base 2) `ws`, depth change that the
-// slope predicts over the offset `pred`, depth offset `eps`, depth difference
-// `dz`, cosine of the normals `nn`.
+__device__ __forceinline__ float rcp_approx(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// n / d of two pairs, rounded as the operator / rounds it, without its branch: a
+// reciprocal with one Newton step, and the quotient corrected by its exact
+// remainder (P. Markstein, "Computation of elementary functions on the IBM RISC
+// System/6000 processor", 1990).  For d in [2^-60, 2^60] and |n| up to 2^60: no
+// step leaves the normal range, or the quotient is too small to matter beside 1.
+__device__ __forceinline__ float2 div_pair(float2 n, float2 d) {
+    const float2 nd = make_float2(-d.x, -d.y);
+    float2 r = make_float2(rcp_approx(d.x), rcp_approx(d.y));
+    r = fma2(r, fma2(nd, r, both(1.0f)), r);
+    const float2 q = mul2(n, r);
+    return fma2(fma2(nd, q, n), r, q);
+}
+
+// Two of bilateral_weight's weights, rounded as there: spatial factors `ws`,
+// depth change that the slope predicts over the offset `pred`, depth offset
+// `eps`, depth difference `dz`, cosine of the normals `nn`.
+template <bool kPlain>
 __device__ __forceinline__ float2 weight_pair(float2 ws, float2 pred, float eps, float2 dz, float2 nn) {
-    const float ax = fmaf(-kLog2E * fabsf(dz.x), __fdividef(1.0f, fabsf(pred.x) + eps), ws.x);
-    const float ay = fmaf(-kLog2E * fabsf(dz.y), __fdividef(1.0f, fabsf(pred.y) + eps), ws.y);
+    const float2 n = make_float2(-fabsf(dz.x), -fabsf(dz.y));
+    const float2 d = make_float2(kSigmaZ * fabsf(pred.x) + eps, kSigmaZ * fabsf(pred.y) + eps);
+    const float2 a = kPlain ? div_pair(n, d) : make_float2(n.x / d.x, n.y / d.y);
     float2 v = make_float2(fmaxf(nn.x, 0.0f), fmaxf(nn.y, 0.0f));
 #pragma unroll
     for (int i = 0; i < 7; ++i) v = mul2(v, v);
-    return mul2(v, make_float2(exp2_approx(ax), exp2_approx(ay)));
+    return mul2(mul2(ws, make_float2(expf(a.x), expf(a.y))), v);
 }
 
 struct Tile {  // staged extents: the guides one ring wider (slopes) than the gradients
@@ -206,20 +228,18 @@ struct Tile {  // staged extents: the guides one ring wider (slopes) than the gr
 // The weights of staged row s (relative to the thread's first pixel) for its two
 // pixels, s and s - 1 rows away; kEdge: one of them is beyond the footprint, and
 // its gradients are left out (an infinity there must not meet a zero weight).
-template <int K, bool kEdge>
+template <int K, bool kPlain, bool kEdge>
 __device__ __forceinline__ void gather_row(const Guide* g, const float2* slope, const float4* c, int cplane, int R, int s,
-                                           float spatial, float2 z, float2 nx, float2 ny, float2 nz, float2 (&acc)[K][3]) {
+                                           const float2* ws, float2 z, float2 nx, float2 ny, float2 nz, float2 (&acc)[K][3]) {
     const float2 dy = make_float2((float)s, (float)(s - 1));
-    const float2 ws_row = mul2(mul2(dy, dy), both(spatial));
     const bool v0 = !kEdge || abs(s) <= R, v1 = !kEdge || abs(s - 1) <= R;
 #pragma unroll kUnroll
     for (int dx = -R; dx <= R; ++dx) {
         const Guide p = g[dx];  // the weight's centre; the offset's sign drops out
         const float2 sl = slope[dx];
-        const float fx = (float)dx;
-        const float2 pred = fma2(both(sl.x), both(fx), mul2(both(sl.y), dy));
-        const float2 nn = fma2(nx, both(p.nx), fma2(ny, both(p.ny), mul2(nz, both(p.nz))));
-        float2 w = weight_pair(add2(ws_row, both(spatial * (fx * fx))), pred, kEpsRel * fabsf(p.z),
+        const float2 pred = fma2(both(sl.y), dy, both(__fmul_rn(sl.x, (float)dx)));
+        const float2 nn = fma2(nz, both(p.nz), fma2(ny, both(p.ny), mul2(nx, both(p.nx))));
+        float2 w = weight_pair<kPlain>(ws[dx], pred, kEpsRel * fabsf(p.z),
                                make_float2(z.x - p.z, z.y - p.z), nn);
         if (kEdge) w = make_float2(v0 ? w.x : 0.0f, v1 ? w.y : 0.0f);
 #pragma unroll
@@ -252,12 +272,16 @@ __global__ void __launch_bounds__(32 * kMaxWarps) bilateral_bwd_kernel(const flo
     const int cplane = T.cw * T.ch;
     float4* sc = smem + T.gw * T.gh;                          // K planes of g / W
     float2* ss = reinterpret_cast<float2*>(sc + K * cplane);  // slopes
+    float2* s_ws = ss + cplane;                               // spatial factors of rows s and s - 1, [s + R][dx + R]
     const mcdi_camera C = cams[view];
     const size_t plane = (size_t)H * W, gbase = (size_t)view * plane;
+    bool plain = true;
 #pragma unroll 4
     for (int i = threadIdx.x; i < T.gw * T.gh; i += threads) {
         const int sy = i / T.gw, sx = i - sy * T.gw;
-        sg[i] = load_guide(pos, nrm, C, H, W, gbase, x0 + sx - (R + 1), y0 + sy - (R + 1));
+        const Guide g = load_guide(pos, nrm, C, H, W, gbase, x0 + sx - (R + 1), y0 + sy - (R + 1));
+        sg[i] = g;
+        plain &= g.z < 0.0f || (g.z >= kPlainMin && g.z <= kPlainMax);
     }
 #pragma unroll 4
     for (int i = threadIdx.x; i < cplane; i += threads) {
@@ -273,7 +297,12 @@ __global__ void __launch_bounds__(32 * kMaxWarps) bilateral_bwd_kernel(const flo
                 inside && w > 0.0f ? make_float4(v.x * iw, v.y * iw, v.z * iw, 0.0f) : make_float4(0, 0, 0, 0);
         }
     }
-    __syncthreads();
+    plain = __syncthreads_and(plain);
+    for (int i = threadIdx.x; i < (2 * R + 2) * (2 * R + 1); i += threads) {
+        const int row = i / (2 * R + 1), dx = i - row * (2 * R + 1) - R, s = row - R;
+        s_ws[i] = make_float2(expf(-(float)(dx * dx + s * s) * inv2s2),
+                              expf(-(float)(dx * dx + (s - 1) * (s - 1)) * inv2s2));
+    }
     for (int i = threadIdx.x; i < cplane; i += threads) {
         const int sy = i / T.cw, sx = i - sy * T.cw;
         const Guide* g = sg + (sy + 1) * T.gw + sx + 1;
@@ -299,13 +328,19 @@ __global__ void __launch_bounds__(32 * kMaxWarps) bilateral_bwd_kernel(const flo
     if (cov[0] || cov[1]) {
         const float2 z = make_float2(a.z, b.z), nx = make_float2(a.nx, b.nx), ny = make_float2(a.ny, b.ny),
                      nz = make_float2(a.nz, b.nz);
-        const float spatial = -inv2s2 * kLog2E;
-        for (int s = -R; s <= R + 1; ++s) {
-            const Guide* g = g0 + s * T.gw;
-            const int o = o0 + s * T.cw;
-            if (s > -R && s <= R) gather_row<K, false>(g, ss + o, sc + o, cplane, R, s, spatial, z, nx, ny, nz, acc);
-            else gather_row<K, true>(g, ss + o, sc + o, cplane, R, s, spatial, z, nx, ny, nz, acc);
-        }
+        auto gather = [&](auto plain_depths) {
+            constexpr bool kPlain = decltype(plain_depths)::value;
+            for (int s = -R; s <= R + 1; ++s) {
+                const Guide* g = g0 + s * T.gw;
+                const int o = o0 + s * T.cw;
+                const float2* ws = s_ws + (s + R) * (2 * R + 1) + R;
+                if (s > -R && s <= R)
+                    gather_row<K, kPlain, false>(g, ss + o, sc + o, cplane, R, s, ws, z, nx, ny, nz, acc);
+                else gather_row<K, kPlain, true>(g, ss + o, sc + o, cplane, R, s, ws, z, nx, ny, nz, acc);
+            }
+        };
+        if (plain) gather(std::true_type{});
+        else gather(std::false_type{});
     }
 #pragma unroll
     for (int i = 0; i < kRows; ++i) {
@@ -336,10 +371,17 @@ cudaError_t allow_smem(const void* kernel, size_t smem) {
 template <int K>
 cudaError_t launch_bwd(const float4* pos, const float4* nrm, const mcdi_camera* cams, int N, int H, int W,
                        const float* wsum, const float4* g_out, float inv2s2, int R, float4* g_in, cudaStream_t s) {
-    const int warps = R > kWideRadius ? kMaxWarps : kMaxWarps / 2;
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    constexpr int kFew = kMaxWarps / 2;
+    const long long few = (long long)((W + kTileW - 1) / kTileW) * ((H + kRows * kFew - 1) / (kRows * kFew)) * N;
+    const int warps = few <= sms ? kFew : kMaxWarps;
     const Tile T(R, warps);
-    const size_t smem = (size_t)T.gw * T.gh * sizeof(Guide) + (size_t)T.cw * T.ch * (K * sizeof(float4) + sizeof(float2));
-    const cudaError_t e = allow_smem((const void*)bilateral_bwd_kernel<K>, smem);
+    const size_t smem = (size_t)T.gw * T.gh * sizeof(Guide) + (size_t)T.cw * T.ch * (K * sizeof(float4) + sizeof(float2)) +
+                        (size_t)(2 * R + 2) * (2 * R + 1) * sizeof(float2);
+    e = allow_smem((const void*)bilateral_bwd_kernel<K>, smem);
     if (e != cudaSuccess) return e;
     const dim3 grid((W + kTileW - 1) / kTileW, (H + kRows * warps - 1) / (kRows * warps), N);
     launch_k(bilateral_bwd_kernel<K>, grid, 32 * warps, smem, s, pos, nrm, cams, N, H, W, wsum, g_out, inv2s2, R, g_in);

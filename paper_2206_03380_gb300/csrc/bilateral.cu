@@ -154,6 +154,89 @@ __global__ void __launch_bounds__(kTile* kTile) bilateral_fwd_kernel(const float
     wsum[gbase + pix] = wt;
 }
 
+// Backward for radii 0 and 1 on images up to about 600 x 600: a pixel per thread, in
+// the forward's tiles.  With at most nine weights a pixel the other form's table,
+// slopes and second barrier cost more than its pairs save, until loads and
+// arithmetic outweigh them.  Measured (this / the other), two images, radius 1: 100 x
+// 90: 7.2 / 9.7 us, 400 x 400: 11.0 / 13.1, 640 x 640: 21.5 / 21.7, 2 x 800 x 800: 70 /
+// 66; radius 2: 100 x 90: 11.4 / 11.1, 320 x 300: 19.5 / 13.9.
+constexpr int kNearRadius = 1, kNearTiles = 10;  // tiles of the other form per SM
+__global__ void __launch_bounds__(kTile* kTile) bilateral_bwd_near_kernel(
+    const float4* __restrict__ pos, const float4* __restrict__ nrm, const mcdi_camera* __restrict__ cams, int N, int H,
+    int W, int K, const float* __restrict__ wsum, const float4* __restrict__ g_out, float inv2s2, int R,
+    float4* __restrict__ g_in) {
+    pdl_prologue();
+    extern __shared__ float4 smem[];
+    const int view = blockIdx.z;
+    const int x0 = blockIdx.x * kTile, y0 = blockIdx.y * kTile;
+    const int gw = kTile + 2 * (R + 1), cw = kTile + 2 * R;
+    Guide* sg = reinterpret_cast<Guide*>(smem);
+    float4* sgw = smem + gw * gw;  // K planes of g / W over cw * cw
+    const mcdi_camera C = cams[view];
+    const size_t plane = (size_t)H * W;
+    const size_t gbase = (size_t)view * plane;
+    for (int i = threadIdx.x; i < gw * gw; i += blockDim.x) {
+        const int sx = i % gw, sy = i / gw;
+        sg[i] = load_guide(pos, nrm, C, H, W, gbase, x0 + sx - (R + 1), y0 + sy - (R + 1));
+    }
+    for (int k = 0; k < K; ++k) {
+        const size_t cbase = (size_t)(view + k * N) * plane;
+        for (int i = threadIdx.x; i < cw * cw; i += blockDim.x) {
+            const int x = x0 + i % cw - R, y = y0 + i / cw - R;
+            float4 v = make_float4(0, 0, 0, 0);
+            if (x >= 0 && y >= 0 && x < W && y < H) {
+                const float w = wsum[gbase + (size_t)y * W + x];
+                if (w > 0.0f) {
+                    const float4 g = g_out[cbase + (size_t)y * W + x];
+                    const float iw = 1.0f / w;
+                    v = make_float4(g.x * iw, g.y * iw, g.z * iw, 0.0f);
+                }
+            }
+            sgw[k * cw * cw + i] = v;
+        }
+    }
+    __syncthreads();
+    const int tx = threadIdx.x % kTile, ty = threadIdx.x / kTile;
+    const int x = x0 + tx, y = y0 + ty;
+    if (x >= W || y >= H) return;
+    const size_t pix = (size_t)y * W + x;
+    const Guide q = sg[(ty + R + 1) * gw + tx + R + 1];
+    if (q.z < 0.0f) {  // uncovered: pass through
+        for (int k = 0; k < K; ++k) {
+            const size_t i = (size_t)(view + k * N) * plane + pix;
+            const float4 g = g_out[i];
+            g_in[i] = make_float4(g.x, g.y, g.z, 0.0f);
+        }
+        return;
+    }
+    float acc[kMaxImgPerView][3] = {};
+    // p = q + (ox, oy); the offset of q seen from p is (-ox, -oy)
+    for (int oy = -R; oy <= R; ++oy) {
+        for (int ox = -R; ox <= R; ++ox) {
+            const int sx = tx + R + 1 + ox, sy = ty + R + 1 + oy;
+            if (sg[sy * gw + sx].z < 0.0f) continue;
+            const Center p = center_of(sg, gw, sx, sy);
+            const float w = bilateral_weight(p, q, -ox, -oy, inv2s2);
+            const int ci = (ty + R + oy) * cw + tx + R + ox;
+#pragma unroll
+            for (int k = 0; k < kMaxImgPerView; ++k) {
+                if (k >= K) break;
+                const float4 g = sgw[k * cw * cw + ci];
+                acc[k][0] += w * g.x;
+                acc[k][1] += w * g.y;
+                acc[k][2] += w * g.z;
+            }
+        }
+    }
+    for (int k = 0; k < K; ++k)
+        g_in[(size_t)(view + k * N) * plane + pix] = make_float4(acc[k][0], acc[k][1], acc[k][2], 0.0f);
+}
+
+size_t bilateral_smem(int R, int K) {
+    const int gw = kTile + 2 * (R + 1), cw = kTile + 2 * R;
+    return (size_t)gw * gw * sizeof(Guide) + (size_t)K * cw * cw * sizeof(float4);
+}
+
 // ---- backward
 // A CTA owns a tile of one view, 32 pixels wide, each thread two pixels of a
 // column; guides and the upstream gradients divided by W(p) over the tile plus its
@@ -170,17 +253,19 @@ __global__ void __launch_bounds__(kTile* kTile) bilateral_fwd_kernel(const float
 // a division and a branch: 68 and 824; with an approximate quotient and one
 // approximate exponential 34 and 377, whose weights are off by up to twice as
 // much: not taken).  The gradient's error against 64 bits, with the loss before
-// it, is 0.5 to 12% below either of theirs over ten shapes.  The forward is not built this way: two pixels per thread gain
-// it nothing (66 and 503 us against 63 and 631, 27 against 22 at 133 x 77).
+// it, is 0.5 to 12% below either of theirs over ten shapes.  The forward is not
+// built this way: two pixels per thread gain it nothing (66 and 503 us against 63
+// and 631, 27 against 22 at 133 x 77).
 constexpr int kTileW = 32;
 constexpr int kRows = 2;  // pixels of a thread, in one column
 constexpr int kUnroll = 4;  // 3: 3 to 8% slower, 5 and 6: 2 to 10%
-// Warps of a CTA: 8, whose tiles share more of their halo, or 4 where CTAs of 4 do
-// not outnumber the SMs and fewer would leave some idle.  Measured (4 / 8 warps), two
-// images: 133 x 77, radius 8: 34 / 41 us, radius 4: 15.7 / 17.4; 256 x 256: 18.9 /
-// 17.5; 512 x 512: 35.8 / 36.0; 3 x 700 x 611, radius 8: 469 / 405; 4 x 800 x 800,
-// radius 5: 366 / 320.
-constexpr int kMaxWarps = 8;
+// Warps of a CTA: 4, or from radius 4 on, where the halo is as large as the tile, 8,
+// unless CTAs of 4 do not outnumber the SMs and fewer would leave some idle.
+// Measured (4 / 8 warps), two images: 133 x 77, radius 8: 34 / 41 us, radius 4: 15.7 /
+// 17.4; 256 x 256: 18.9 / 17.5; 512 x 512: 35.8 / 36.0; 3 x 700 x 611, radius 8: 469 /
+// 408; 4 x 800 x 800, radius 5: 366 / 320; 320 x 300, radius 2: 13.9 / 15.1, radius 3:
+// 17.6 / 20.0; 512 x 512, radius 3: 27.5 / 27.7.
+constexpr int kMaxWarps = 8, kWideRadius = 4;
 // Depths for which weight_pair's divisors (from 1e-3 of one to 17 times the largest) stay in div_pair's range.
 constexpr float kPlainMin = 0x1p-40f, kPlainMax = 0x1p40f;
 
@@ -358,11 +443,6 @@ __global__ void __launch_bounds__(32 * kMaxWarps) bilateral_bwd_kernel(const flo
     }
 }
 
-size_t bilateral_smem(int R, int K) {
-    const int gw = kTile + 2 * (R + 1), cw = kTile + 2 * R;
-    return (size_t)gw * gw * sizeof(Guide) + (size_t)K * cw * cw * sizeof(float4);
-}
-
 cudaError_t allow_smem(const void* kernel, size_t smem) {
     return smem > 48 * 1024 ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
                             : cudaSuccess;
@@ -377,7 +457,13 @@ cudaError_t launch_bwd(const float4* pos, const float4* nrm, const mcdi_camera* 
     if (e != cudaSuccess) return e;
     constexpr int kFew = kMaxWarps / 2;
     const long long few = (long long)((W + kTileW - 1) / kTileW) * ((H + kRows * kFew - 1) / (kRows * kFew)) * N;
-    const int warps = few <= sms ? kFew : kMaxWarps;
+    if (R <= kNearRadius && few <= (long long)kNearTiles * sms) {
+        const dim3 grid((W + kTile - 1) / kTile, (H + kTile - 1) / kTile, N);
+        launch_k(bilateral_bwd_near_kernel, grid, kTile * kTile, bilateral_smem(R, K), s, pos, nrm, cams, N, H, W, K,
+                 wsum, g_out, inv2s2, R, g_in);
+        return cudaGetLastError();
+    }
+    const int warps = R < kWideRadius || few <= sms ? kFew : kMaxWarps;
     const Tile T(R, warps);
     const size_t smem = (size_t)T.gw * T.gh * sizeof(Guide) + (size_t)T.cw * T.ch * (K * sizeof(float4) + sizeof(float2)) +
                         (size_t)(2 * R + 2) * (2 * R + 1) * sizeof(float2);

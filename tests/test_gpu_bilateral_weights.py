@@ -48,3 +48,26 @@ def test_backward_has_the_forwards_weights(cuda_lib, guides, radius, K, sigma, s
             assert torch.equal(f[both], b[both]), (dx, dy, (f - b)[both].abs().max())
             pairs += int((both & (f > 0)).sum())
     assert pairs > int(cov.sum()) * (1 if radius == 0 else 3) * 0.9
+
+
+@pytest.mark.parametrize("radius,K", [(0, 1), (1, 2), (1, 4)])
+def test_small_radii_on_both_sides_of_the_size_line(cuda_lib, guides, radius, K):
+    """A large image, and a piece of it that is small enough for the kernel of one pixel per thread: the same bits
+    wherever the piece holds the footprints and their slopes' neighbours."""
+    mcdi, n = cuda_lib, 17
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    cams = t(guides[2][:1].copy())
+    pos, nrm = (t(np.tile(a[:1], (1, n, n, 1))) for a in guides[:2])  # 680 x 816 pixels
+    H, W = pos.shape[1:3]
+    gen = torch.Generator(device="cuda").manual_seed(radius + K)
+    g = torch.randn((K, H, W, 4), generator=gen, device="cuda")
+    out, wsum = torch.empty_like(g), torch.empty((1, H, W), device="cuda")
+    mcdi.bilateral_fwd(pos, nrm, cams, g, 0.5, out, wsum, radius=radius)
+    mcdi.bilateral_bwd(pos, nrm, cams, wsum, g, 0.5, out, radius=radius)
+    ys, xs, m = slice(200, 333), slice(311, 400), radius + 1
+    cut = lambda a: a[:, ys, xs].contiguous()
+    piece = torch.empty_like(cut(g))
+    mcdi.bilateral_bwd(cut(pos), cut(nrm), cams, cut(wsum), cut(g), 0.5, piece, radius=radius)
+    torch.cuda.synchronize()
+    assert torch.equal(piece[:, m:-m, m:-m], cut(out)[:, m:-m, m:-m])
+    assert (piece != cut(g)).any()

@@ -352,7 +352,8 @@ __global__ void __launch_bounds__(32 * kMaxWarps) bilateral_bwd_kernel(const flo
     const int threads = blockDim.x;
     const Tile T(R, threads >> 5);
     const int view = blockIdx.z;
-    const int x0 = blockIdx.x * kTileW, y0 = blockIdx.y * kRows * (threads >> 5);
+    const int tiles_x = (W + kTileW - 1) / kTileW, tile_y = blockIdx.x / tiles_x;  // (rows of tiles may outnumber a grid's y)
+    const int x0 = (blockIdx.x - tile_y * tiles_x) * kTileW, y0 = tile_y * kRows * (threads >> 5);
     Guide* sg = reinterpret_cast<Guide*>(smem);
     const int cplane = T.cw * T.ch;
     float4* sc = smem + T.gw * T.gh;                          // K planes of g / W
@@ -469,7 +470,7 @@ cudaError_t launch_bwd(const float4* pos, const float4* nrm, const mcdi_camera* 
                         (size_t)(2 * R + 2) * (2 * R + 1) * sizeof(float2);
     e = allow_smem((const void*)bilateral_bwd_kernel<K>, smem);
     if (e != cudaSuccess) return e;
-    const dim3 grid((W + kTileW - 1) / kTileW, (H + kRows * warps - 1) / (kRows * warps), N);
+    const dim3 grid(((W + kTileW - 1) / kTileW) * ((H + kRows * warps - 1) / (kRows * warps)), 1, N);
     launch_k(bilateral_bwd_kernel<K>, grid, 32 * warps, smem, s, pos, nrm, cams, N, H, W, wsum, g_out, inv2s2, R, g_in);
     return cudaGetLastError();
 }

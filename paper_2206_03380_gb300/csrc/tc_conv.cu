@@ -1203,6 +1203,22 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn(const char** why) {
     return fn;
 }
 
+// The driver's encoder.  It wants a context that is current in the calling thread,
+// which the runtime binds only with a thread's first call that needs one: a thread
+// that starts with a convolution binds it here and encodes again.
+struct Encoder {
+    PFN_cuTensorMapEncodeTiled_v12000 fn;
+    explicit operator bool() const { return fn != nullptr; }
+    template <typename... Args>
+    CUresult operator()(Args... args) const {
+        const CUresult r = fn(args...);
+        if (r != CUDA_ERROR_INVALID_CONTEXT && r != CUDA_ERROR_NOT_INITIALIZED) return r;
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || cudaSetDevice(dev) != cudaSuccess) return r;
+        return fn(args...);
+    }
+};
+
 struct DeviceLimits {
     int sms = 0;
     uint32_t rows_smem_max = 0;  // dynamic shared memory one row-tile CTA may request
@@ -1305,7 +1321,7 @@ size_t conv_smem_bytes(int cout_pad) {
 
 bool encode_plane_rows_map(CUtensorMap* map, const void* base, int W, int H, long long n_planes, int box_px,
                            int box_rows, int box_planes, const char** why) {
-    auto enc = encode_fn(why);
+    const Encoder enc{encode_fn(why)};
     if (!enc) return false;
     // BF16 8-channel planes [plane][H][W][16 B] as rows of 8-byte elements (two per pixel), so that a box
     // row of box_px pixels is one contiguous run for the copy engine
@@ -1366,7 +1382,7 @@ static bool plan_halo(const ConvParams& p, HaloPlan* out) {
 }
 
 bool conv_make_desc(ConvDesc* d, const void* x, const void* w, const char** why) {
-    auto enc = encode_fn(why);
+    const Encoder enc{encode_fn(why)};
     if (!enc) return false;
     const ConvParams& p = d->p;
     d->p.x = x;

@@ -444,11 +444,6 @@ __global__ void __launch_bounds__(32 * kMaxWarps) bilateral_bwd_kernel(const flo
     }
 }
 
-cudaError_t allow_smem(const void* kernel, size_t smem) {
-    return smem > 48 * 1024 ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                            : cudaSuccess;
-}
-
 template <int K>
 cudaError_t launch_bwd(const float4* pos, const float4* nrm, const mcdi_camera* cams, int N, int H, int W,
                        const float* wsum, const float4* g_out, float inv2s2, int R, float4* g_in, cudaStream_t s) {

@@ -80,4 +80,23 @@ inline cudaError_t launch_k_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 
     return launch_k_impl(true, kernel, grid, block, smem, stream, std::forward<Args>(args)...);
 }
 
+// Lets launches of the kernel ask for `bytes` of dynamic shared memory.  Beyond the
+// default 48 KB a kernel has to be allowed it beforehand, once for the context, not
+// per launch: the allowance is therefore always raised to all that the device gives
+// a block, whatever this call needs, so that another thread's call with other sizes
+// cannot lower it between this one and its launch.
+inline cudaError_t allow_smem(const void* kernel, size_t bytes) {
+    if (bytes <= 48 * 1024) return cudaSuccess;
+    int dev = 0, optin = 0;
+    cudaFuncAttributes fa{};
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kernel);
+    if (e != cudaSuccess) return e;
+    const size_t room = (size_t)optin > fa.sharedSizeBytes ? (size_t)optin - fa.sharedSizeBytes : 0;
+    if (bytes > room) return cudaErrorInvalidValue;
+    if ((size_t)fa.maxDynamicSharedSizeBytes >= room) return cudaSuccess;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room);
+}
+
 }  // namespace mcdi

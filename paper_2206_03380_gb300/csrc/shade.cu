@@ -401,18 +401,11 @@ cudaError_t launch_primary_cast(const void* nodes, const void* tris, int n_tris,
     return cudaGetLastError();
 }
 
-// dynamic shared memory beyond the default limit (large probes) has to be asked for
-template <class K>
-static cudaError_t allow_smem(K* kernel, size_t bytes) {
-    if (bytes <= 48 * 1024) return cudaSuccess;
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 cudaError_t launch_shade_fwd(const ShadeArgs& a, float4* c_d, float4* kd_out, float4* c_s, uint32_t* vis_mask,
                              cudaStream_t stream) {
     const long long P = (long long)a.N * a.H * a.W;
     const size_t smem = sizeof(FwdShared) + (size_t)(a.Hp + 1) * sizeof(float);
-    const cudaError_t e = allow_smem(shade_fwd_kernel, smem);
+    const cudaError_t e = allow_smem((const void*)shade_fwd_kernel, smem);
     if (e != cudaSuccess) return e;
     launch_k(shade_fwd_kernel, grid_for(P, 32), kShadeThreads, smem, stream, a, c_d, kd_out, c_s, vis_mask);
     return cudaGetLastError();
@@ -431,7 +424,7 @@ cudaError_t launch_shade_bwd(const ShadeArgs& a, const float4* g_cd, const float
         return cudaGetLastError();
     }
     const size_t smem_rt = smem + sizeof(BlockRays<kBwdChunk>);
-    const cudaError_t e = allow_smem(shade_bwd_kernel<true>, smem_rt);
+    const cudaError_t e = allow_smem((const void*)shade_bwd_kernel<true>, smem_rt);
     if (e != cudaSuccess) return e;
     launch_k(shade_bwd_kernel<true>, grid_for(count, 32), kShadeThreads, smem_rt, stream, a, g_cd, g_kdout, g_cs,
              vis_mask, g_kd, g_korm, g_nrm, g_env, first, first + count);

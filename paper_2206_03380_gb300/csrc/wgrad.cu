@@ -462,7 +462,7 @@ cudaError_t launch_wgrad(const WgradConv* conv, int n, void* scratch, unsigned* 
         off += align256(P.partial_bytes);
         if (P.smem > smem) smem = P.smem;
     }
-    cudaError_t e = cudaFuncSetAttribute(wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem((const void*)wgrad_kernel, smem);
     if (e != cudaSuccess) return e;
     e = launch_k(wgrad_kernel, blocks, kWgThreads, smem, s, B);
     if (e != cudaSuccess) return e;

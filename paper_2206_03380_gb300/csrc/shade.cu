@@ -46,18 +46,6 @@ CastTiles cast_tiles(int H, int W) {
     return T;
 }
 
-// Whether a ray from o may use the four-wide nodes: a plane's distance is off by
-// up to 3 u |plane - o| and half a quantisation step, and the child boxes are a
-// whole step (at least 2^-17 of the largest coordinate m of the root box) wider
-// on each side, so |o| may be 2^-18 m / 3 u - m = 20 m; 16 m is taken.
-__device__ __forceinline__ bool wide_cast_ok(const BvhNode* __restrict__ nodes, f3 o) {
-    const float4 a = __ldg(&nodes->a), b = __ldg(&nodes->b), c = __ldg(&nodes->c);
-    const float mx = fmaxf(fmaxf(fabsf(a.x), fabsf(a.y)), fmaxf(fabsf(b.x), fabsf(b.y)));
-    const float my = fmaxf(fmaxf(fabsf(a.z), fabsf(a.w)), fmaxf(fabsf(b.z), fabsf(b.w)));
-    const float mz = fmaxf(fmaxf(fabsf(c.x), fabsf(c.y)), fmaxf(fabsf(c.z), fabsf(c.w)));
-    return fmaxf(fabsf(o.x), fmaxf(fabsf(o.y), fabsf(o.z))) <= 16.0f * fmaxf(mx, fmaxf(my, mz));
-}
-
 __global__ void __launch_bounds__(kShadeThreads) primary_cast_kernel(
     const BvhNode* __restrict__ nodes, const TriRecord* __restrict__ tris, int n_tris, const float* __restrict__ verts,
     const float* __restrict__ vnrm, const int* __restrict__ tri_idx, int n_verts, const mcdi_camera* __restrict__ cams,
@@ -83,7 +71,7 @@ __global__ void __launch_bounds__(kShadeThreads) primary_cast_kernel(
     const RayInv ray = make_ray(o, d);
     float t, u = 0.f, v = 0.f;
     int leaf = kWideOverflow;
-    if (n_tris > 0 && wide_cast_ok(nodes, o))  // the same for the whole CTA: one view
+    if (n_tris > 0 && largest(o) <= wide_reach(nodes))  // the same for the whole CTA: one view
         leaf = closest_hit_wide(wide_nodes(nodes, n_tris), tris, n_tris, ray, live ? 0 : -1,
                                 stack + (threadIdx.x >> 1) * (kCastStack + 1), &t, &u, &v);
     if (!inside) return;

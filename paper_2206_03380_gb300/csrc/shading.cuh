@@ -212,6 +212,26 @@ __device__ __forceinline__ float qbyte(uint32_t w, int k) {
     return __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7540u + (uint32_t)k));
 }
 
+// The largest coordinate (in magnitude) that a ray's origin o may have for the
+// four-wide nodes' boxes to hold what they should, or a negative number where no
+// ray may use them.  With m the largest coordinate of the root box, P a child box's
+// plane and a its node's origin, the computed distance to the plane (wide_visit)
+// differs from (P - o) / d, in units of the axis, by at most
+//   u |P - o| (1 / d) + u |o| (its product) + u |a - o| (the difference)
+//   + u (2^23 s + |a - o|) (B') + u |P - o| (the last sum)  <=  s / 2 + u (5 |o| + 4 m).
+// The child boxes are a step s >= 2^-17 m wider on each side, so |o| may be 12 m; 11
+// m is taken.  And no product may overflow: 1 / d goes up to 1e20 (make_ray) and
+// 2^23 s to 1.4e5 m, so m up to 1e12 (an infinite vertex makes m infinite).
+__device__ __forceinline__ float wide_reach(const BvhNode* __restrict__ nodes) {
+    const float4 a = __ldg(&nodes->a), b = __ldg(&nodes->b), c = __ldg(&nodes->c);
+    const float mx = fmaxf(fmaxf(fabsf(a.x), fabsf(a.y)), fmaxf(fabsf(b.x), fabsf(b.y)));
+    const float my = fmaxf(fmaxf(fabsf(a.z), fabsf(a.w)), fmaxf(fabsf(b.z), fabsf(b.w)));
+    const float mz = fmaxf(fmaxf(fabsf(c.x), fabsf(c.y)), fmaxf(fabsf(c.z), fabsf(c.w)));
+    const float m = fmaxf(mx, fmaxf(my, mz));
+    return m <= 1e12f ? 11.0f * m : -1.0f;
+}
+__device__ __forceinline__ float largest(f3 o) { return fmaxf(fabsf(o.x), fmaxf(fabsf(o.y), fabsf(o.z))); }
+
 // Slab tests of the four child boxes of a four-wide node; bit k of the result
 // is set when the ray (t >= 0, no far limit) meets child k's box.  Per axis
 // the near plane is the low one for a non-negative direction, the high one

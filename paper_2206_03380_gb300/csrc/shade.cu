@@ -30,19 +30,27 @@ __device__ __forceinline__ f3 cam_origin(const mcdi_camera* cams, int view) {
 // ---------------------------------------------------------------- G-buffer
 // A warp casts 4 x 4 pixels (or 16 x 1, 8 x 2, .. 1 x 16 where a narrow image
 // would leave lanes out), so that its rays visit the same nodes; a CTA's four
-// warps lie 2 x 2 (or in a row or a column).
+// warps lie 2 x 2 (or in a row or a column).  A view whose camera is too far for
+// the four-wide nodes is cast with a ray per lane: in small images both lanes of a
+// pair cast the same one (the rays' latency is all that counts), in large ones every
+// other CTA takes two tiles.  Measured, camera 12 m away (this way / the other; the
+// former kernel of 32 consecutive pixels a warp): 320 x 320: 148 / 199 us (154), 400 x
+// 300: 139 / 146 (132), 512 x 512: 167 / 181 (160).
+constexpr int kCastJoin = 20;  // CTAs per SM from which the image counts as large
 struct CastTiles {
     int log_w, log_wx;  // log2 of the warp tile's width and of the warps side by side
     int nx, ny;         // CTAs per view
+    bool join;          // whether a CTA whose view is cast with a ray per lane takes two tiles
 };
-CastTiles cast_tiles(int H, int W) {
-    CastTiles T{2, 1, 0, 0};
+CastTiles cast_tiles(int N, int H, int W, int sms) {
+    CastTiles T{2, 1, 0, 0, false};
     while (T.log_w < 4 && (8 >> T.log_w) >= H) ++T.log_w;
     while (T.log_w > 0 && (1 << (T.log_w - 1)) >= W) --T.log_w;
     if ((1 << T.log_w) >= W) T.log_wx = 0;
     else if ((16 >> T.log_w) >= H) T.log_wx = 2;
     T.nx = ((W - 1) >> (T.log_w + T.log_wx)) + 1;
     T.ny = ((H - 1) >> (6 - T.log_w - T.log_wx)) + 1;
+    T.join = (long long)N * T.nx * T.ny > (long long)kCastJoin * sms;
     return T;
 }
 
@@ -55,23 +63,31 @@ __global__ void __launch_bounds__(kShadeThreads) primary_cast_kernel(
     pdl_prologue();
     __shared__ float2 stack[(kCastStack + 1) * kShadeThreads / 2];
     const int per_view = T.nx * T.ny;
-    const int view = blockIdx.x / per_view, tile = blockIdx.x - view * per_view;
-    const int warp = threadIdx.x >> 5, ray_of_warp = (threadIdx.x & 31) >> 1;
+    const int view = blockIdx.x / per_view;
+    int tile = blockIdx.x - view * per_view, warp = threadIdx.x >> 5, ray_of_warp = (threadIdx.x & 31) >> 1;
+    const mcdi_camera& C = cams[view];
+    const f3 o = mk(C.origin[0], C.origin[1], C.origin[2]);
+    const bool pairs = n_tris > 0 && largest(o) <= wide_reach(nodes);  // the same for the whole CTA: one view
+    const bool joined = !pairs && T.join;
+    if (joined) {  // a ray per lane: every other CTA takes two tiles, half a warp a warp's tile
+        if (tile & 1) return;
+        tile += threadIdx.x >> 6;
+        warp = (threadIdx.x >> 4) & 3;
+        ray_of_warp = threadIdx.x & 15;
+    }
     const int ty = tile / T.nx, tx = tile - ty * T.nx;
     const int wx = warp & ((1 << T.log_wx) - 1), wy = warp >> T.log_wx;
     const int x = (((tx << T.log_wx) + wx) << T.log_w) + (ray_of_warp & ((1 << T.log_w) - 1));
     const int y = (((ty << (2 - T.log_wx)) + wy) << (4 - T.log_w)) + (ray_of_warp >> T.log_w);
-    const bool inside = x < W && y < H;
+    const bool inside = tile < per_view && x < W && y < H;
     const long long idx = ((long long)view * H + y) * W + x;
-    const mcdi_camera& C = cams[view];
-    const f3 o = mk(C.origin[0], C.origin[1], C.origin[2]);
     const f3 d = camera_dir(C, x, y, W, H);
     // a degenerate camera's NaN passes every box test (minimum and maximum drop it) and no triangle's: a miss
     const bool live = inside && finite_ray(o, d);
     const RayInv ray = make_ray(o, d);
     float t, u = 0.f, v = 0.f;
     int leaf = kWideOverflow;
-    if (n_tris > 0 && largest(o) <= wide_reach(nodes))  // the same for the whole CTA: one view
+    if (pairs)
         leaf = closest_hit_wide(wide_nodes(nodes, n_tris), tris, n_tris, ray, live ? 0 : -1,
                                 stack + (threadIdx.x >> 1) * (kCastStack + 1), &t, &u, &v);
     if (!inside) return;
@@ -81,10 +97,13 @@ __global__ void __launch_bounds__(kShadeThreads) primary_cast_kernel(
         gbuffer_hit(__float_as_int(__ldg(&tris[leaf].v0.w)), u, v, verts, vnrm, tri_idx, n_verts,
                     reinterpret_cast<const float*>(tex_kd), reinterpret_cast<const float*>(tex_korm), S, uv_ox, uv_oz,
                     uv_s, &P, &Nn, &KD, &KORM);
-    // the pair's lanes computed the same; each writes two of the four
+    // a pair's lanes computed the same: each writes two of the four
     const bool odd = threadIdx.x & 1;
     (odd ? gb_nrm : gb_pos)[idx] = odd ? Nn : P;
     (odd ? gb_korm : gb_kd)[idx] = odd ? KORM : KD;
+    if (!joined) return;
+    (odd ? gb_pos : gb_nrm)[idx] = odd ? P : Nn;
+    (odd ? gb_kd : gb_korm)[idx] = odd ? KD : KORM;
 }
 
 // ---------------------------------------------------------------- forward
@@ -380,7 +399,10 @@ cudaError_t launch_primary_cast(const void* nodes, const void* tris, int n_tris,
                                 int H, int W, const float* tex_kd, const float* tex_korm, int tex_size, float uv_ox,
                                 float uv_oz, float uv_s, float* gb_pos, float* gb_nrm, float* gb_kd, float* gb_korm,
                                 cudaStream_t stream) {
-    const CastTiles T = cast_tiles(H, W);
+    int dev = 0, sms = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const CastTiles T = cast_tiles(N, H, W, sms);
     launch_k(primary_cast_kernel, (unsigned)T.nx * (unsigned)T.ny * (unsigned)N, kShadeThreads, 0, stream,
              static_cast<const BvhNode*>(nodes), static_cast<const TriRecord*>(tris), n_tris, verts, vnrm, tri_idx,
              n_verts, cams, N, H, W, T, reinterpret_cast<const float4*>(tex_kd), reinterpret_cast<const float4*>(tex_korm),

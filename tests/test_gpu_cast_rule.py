@@ -63,3 +63,28 @@ def test_cameras_around_the_distance_line(cuda_lib, orc, far):
     tol = 64 * 2.0 ** -24 * np.linalg.norm(eye)
     off = np.abs(g[:, :3] - o[:, :3]).max(1) > 10 * tol
     assert (both & off).sum() <= 0.02 * both.sum() + 3
+
+
+def test_far_cameras_of_large_and_small_images(cuda_lib):
+    """A ray per lane in one tile per CTA (few pixels) and in two (many), with an odd number of tiles per view: the
+    same pixels, all of them."""
+    sc = scenes.parity_scene()
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    pad = lambda a: t(np.concatenate([a, np.zeros(a.shape[:2] + (1,), np.float32)], -1)) if a.shape[-1] == 3 else t(a)
+    eye = np.array([0.2, 0.62, 1.0]) * 20 * float(np.abs(sc.verts).max())
+    verts, vnrm, tris, kd, korm = t(sc.verts), t(sc.vnrm), t(sc.tris), pad(sc.tex_kd), pad(sc.tex_korm)
+    bvh = cuda_lib.Bvh.allocate(len(sc.tris)).build(verts, tris)
+    cam = scenes.look_at(tuple(eye), (0, -0.2, 0), (0, 1, 0), np.degrees(2.4 / np.linalg.norm(eye)), 1.0).astype(np.float32)
+
+    def cast(views, h, w):
+        gb = cuda_lib.GBuffer.allocate(views, h, w)
+        for p in (gb.pos, gb.nrm, gb.kd, gb.korm):
+            p.fill_(float("nan"))
+        cuda_lib.primary_cast(bvh, verts, vnrm, tris, t(np.stack([cam] * views)), h, w, kd, korm, sc.uvmap, gb)
+        torch.cuda.synchronize()
+        return torch.cat([gb.pos, gb.nrm, gb.kd, gb.korm], -1)
+
+    one = cast(1, 99, 71)  # 13 x 9 tiles of 8 x 8
+    many = cast(41, 99, 71)  # the same view, in enough CTAs to join tiles
+    assert torch.isfinite(one).all() and (one[..., 3] > 0).float().mean() > 0.5
+    assert torch.equal(many, one.expand_as(many))

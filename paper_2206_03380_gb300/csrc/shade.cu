@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(kShadeThreads) primary_cast_kernel(
     int tile = blockIdx.x - view * per_view, warp = threadIdx.x >> 5, ray_of_warp = (threadIdx.x & 31) >> 1;
     const mcdi_camera& C = cams[view];
     const f3 o = mk(C.origin[0], C.origin[1], C.origin[2]);
-    const bool pairs = n_tris > 0 && largest(o) <= wide_reach(nodes);  // the same for the whole CTA: one view
+    const bool pairs = largest(o) <= wide_reach(nodes, n_tris);  // the same for the whole CTA: one view
     const bool joined = !pairs && T.join;
     if (joined) {  // a ray per lane: every other CTA takes two tiles, half a warp a warp's tile
         if (tile & 1) return;
@@ -152,6 +152,7 @@ __global__ void __launch_bounds__(kShadeThreads) shade_fwd_kernel(ShadeArgs a, f
     }
     f3 cd = mk(0.f, 0.f, 0.f), cs = cd;
     uint32_t word = 0;
+    const float reach = wide_reach(a.nodes, a.n_tris);
     for (int j0 = 0; j0 < spp; j0 += kFwdChunk) {
         const int n = min(kFwdChunk, spp - j0);
         S.rays.clear();
@@ -186,7 +187,7 @@ __global__ void __launch_bounds__(kShadeThreads) shade_fwd_kernel(ShadeArgs a, f
             S.cs[jj * 32 + lane] = ds;
         }
         __syncthreads();
-        trace_rays(a.nodes, static_cast<const TriRecord*>(a.tris), a.n_tris, S.rays.stacks, S.rays);
+        trace_rays(a.nodes, static_cast<const TriRecord*>(a.tris), a.n_tris, reach, S.rays.stacks, S.rays);
         __syncthreads();
         if (quarter == 0) {
             for (int jj = 0; jj < n; ++jj) {
@@ -269,7 +270,9 @@ __global__ void __launch_bounds__(kShadeThreads, 6) shade_bwd_kernel(ShadeArgs a
     const float so = sqrtf(fmaf(a2, ico2 - 1.0f, 1.0f)), lo = 0.5f * (so - 1.0f);
     const float dlo_dco = (-2.0f * a2 * ico2 / px.co) / (4.0f * so), dlo_da = 2.0f * px.alpha * (ico2 - 1.0f) / (4.0f * so);
     BlockRays<kBwdChunk>* rays = nullptr;
+    float reach = 0.0f;
     if constexpr (kRetrace) {
+        reach = wide_reach(a.nodes, a.n_tris);
         rays = reinterpret_cast<BlockRays<kBwdChunk>*>(s_part + kBwdQuarters * kBwdPartials * 32);
         const f3 o = covered ? fma_rn(px.n, a.ray_eps, px.p) : mk(0.f, 0.f, 0.f);
         if (quarter == 0) rays->origin[lane] = make_float4(o.x, o.y, o.z, 0.f);
@@ -291,7 +294,7 @@ __global__ void __launch_bounds__(kShadeThreads, 6) shade_bwd_kernel(ShadeArgs a
             rays->append(active, j - j0, wi);
         }
         __syncthreads();
-        trace_rays(a.nodes, static_cast<const TriRecord*>(a.tris), a.n_tris, rays->stacks, *rays);
+        trace_rays(a.nodes, static_cast<const TriRecord*>(a.tris), a.n_tris, reach, rays->stacks, *rays);
         __syncthreads();
     }
     for (int j = covered ? j0 + quarter : j1; j < j1; j += kBwdQuarters) {

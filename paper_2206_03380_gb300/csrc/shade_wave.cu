@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(kTraceThreads, kTraceBlocksPerSM) wave_trace_k
     ListRays rays{wave_buffers(ws, P, slots), 0u, (uint32_t)P, (uint32_t)__cvta_generic_to_shared(s_ray + threadIdx.x),
                   (uint32_t)__cvta_generic_to_shared(s_slot + threadIdx.x)};
     rays.n = *((volatile unsigned*)rays.B.counter);
-    trace_rays(nodes, tris, n_tris, s_stacks, rays);
+    trace_rays(nodes, tris, n_tris, wide_reach(nodes, n_tris), s_stacks, rays);
 }
 
 __global__ void __launch_bounds__(kGenThreads) wave_accum_kernel(ShadeArgs a, const void* ws,
@@ -271,6 +271,7 @@ __global__ void __launch_bounds__(kTraceThreads) wave_stats_kernel(const void* _
     const long long n_rays = (long long)B.counter[0];
     unsigned long long c[5] = {0, 0, 0, 0, 0};
     const WideNode* wn = wide_nodes(nodes, n_tris > 0 ? n_tris : 1);
+    const float reach = wide_reach(nodes, n_tris);
     int stack[kWideStack];
     for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < n_rays;
          k += (long long)gridDim.x * blockDim.x) {
@@ -281,7 +282,8 @@ __global__ void __launch_bounds__(kTraceThreads) wave_stats_kernel(const void* _
         bool blocked = false, overflow = false;
         unsigned tests = 0;
         int node = 0, sp = 0;
-        for (int it = 0; it < 2 * n_tris && node >= 0; ++it) {
+        const int visits = largest(r.o) <= reach ? 2 * n_tris : 0;
+        for (int it = 0; it < visits && node >= 0; ++it) {
             ++c[1];
             node = wide_step<1, true>(wn, tris, n_tris, r, node, stack, sp, overflow, &tests);
         }

@@ -213,8 +213,8 @@ __device__ __forceinline__ float qbyte(uint32_t w, int k) {
 }
 
 // The largest coordinate (in magnitude) that a ray's origin o may have for the
-// four-wide nodes' boxes to hold what they should, or a negative number where no
-// ray may use them.  With m the largest coordinate of the root box, P a child box's
+// four-wide nodes' boxes to hold what they should, or a negative number where no ray
+// may use them (then and beyond, the two-child or depth-first nodes decide).  With m the largest coordinate of the root box, P a child box's
 // plane and a its node's origin, the computed distance to the plane (wide_visit)
 // differs from (P - o) / d, in units of the axis, by at most
 //   u |P - o| (1 / d) + u |o| (its product) + u |a - o| (the difference)
@@ -222,7 +222,9 @@ __device__ __forceinline__ float qbyte(uint32_t w, int k) {
 // The child boxes are a step s >= 2^-17 m wider on each side, so |o| may be 12 m; 11
 // m is taken.  And no product may overflow: 1 / d goes up to 1e20 (make_ray) and
 // 2^23 s to 1.4e5 m, so m up to 1e12 (an infinite vertex makes m infinite).
-__device__ __forceinline__ float wide_reach(const BvhNode* __restrict__ nodes) {
+__device__ __forceinline__ float wide_reach(const void* __restrict__ root, int n_tris) {
+    if (n_tris <= 0) return -1.0f;
+    const BvhNode* nodes = static_cast<const BvhNode*>(root);
     const float4 a = __ldg(&nodes->a), b = __ldg(&nodes->b), c = __ldg(&nodes->c);
     const float mx = fmaxf(fmaxf(fabsf(a.x), fabsf(a.y)), fmaxf(fabsf(b.x), fabsf(b.y)));
     const float my = fmaxf(fmaxf(fabsf(a.z), fabsf(a.w)), fmaxf(fabsf(b.z), fabsf(b.w)));

@@ -369,7 +369,8 @@ __global__ void __launch_bounds__(kGradThreads) shadow_edge_grad_kernel(
             if (threadIdx.x == 0) rays.find_parts(a.nodes, a.n_tris);
             __syncthreads();
         }
-        trace_rays(a.nodes, static_cast<const TriRecord*>(a.tris), a.n_tris, rays.stacks, rays);
+        trace_rays(a.nodes, static_cast<const TriRecord*>(a.tris), a.n_tris, wide_reach(a.nodes, a.n_tris), rays.stacks,
+                   rays);
         __syncthreads();
         const unsigned n = rays.n;
         for (unsigned i = threadIdx.x; i < n; i += kGradThreads) {

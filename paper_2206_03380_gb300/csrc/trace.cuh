@@ -33,8 +33,8 @@ struct TraceStacks {  // a CTA's columns: one thread's entries in one bank
 // instead, with rounds forced by waiting lanes, takes a round at nearly every
 // step with a quarter of its lanes, or leaves lanes idle.)
 //
-// A ray whose pending nodes outgrow the stack is decided by the stackless walk
-// of the depth-first copy instead.
+// A ray whose pending nodes outgrow the stack, or whose origin lies beyond `reach`
+// (wide_reach), is decided by the stackless walk of the depth-first copy instead.
 //
 // R supplies the rays: R.count() of them, the same for all warps; R.take(n)
 // (lane 0) reserves the next n and returns the first; R.start(i, id, o, d,
@@ -44,7 +44,7 @@ struct TraceStacks {  // a CTA's columns: one thread's entries in one bank
 // the one before); R.blocked(id) records a hit.
 template <class R>
 __device__ __forceinline__ void trace_rays(const void* __restrict__ nodes, const TriRecord* __restrict__ tris,
-                                           int n_tris, TraceStacks& st, R& rays) {
+                                           int n_tris, float reach, TraceStacks& st, R& rays) {
     constexpr int kStep = 4 * kTraceThreads;
     if (n_tris <= 0) return;  // nothing can block a ray
     const unsigned n_rays = rays.count();
@@ -76,6 +76,7 @@ __device__ __forceinline__ void trace_rays(const void* __restrict__ nodes, const
                 inv = make_ray(o, d).inv;
                 oi = mk(-o.x * inv.x, -o.y * inv.y, -o.z * inv.z);
                 lmark = la;
+                if (!(largest(o) <= reach)) na = nroom + kStep;  // as if its pending nodes had outgrown the stack
             }
             more = base + (unsigned)__popc(idle) < n_rays;
         } else if (!__any_sync(full, node >= 0 || la != lbase)) {
@@ -115,7 +116,7 @@ __device__ __forceinline__ void trace_rays(const void* __restrict__ nodes, const
                     }
                 }
             }
-            if (node >= 0 && na > nroom) {  // more pending nodes than the stack holds
+            if (node >= 0 && na > nroom) {  // more pending nodes than the stack holds, or not for these nodes
                 f3 o, d;
                 rays.load(cur, o, d);
                 if (any_hit_threaded(nodes, tris, n_tris, make_ray(o, d))) rays.blocked(cur);

@@ -11,10 +11,10 @@ namespace mcdi {
 
 // ---------------------------------------------------------------- fixed roundings
 // What decides a sample (its direction, its probe texel, whether a triangle
-// blocks its ray) is written with every rounding spelled out, so that all the
-// kernels that draw a sample or trace its ray, whatever is compiled around it,
-// decide it alike: a sum of products as one fused multiply-add per product
-// after the first, a + b (p q) as one.
+// blocks its ray) is written with every rounding spelled out, so that the kernels
+// that draw a sample or trace its ray decide it alike whatever is compiled around
+// it: a sum of products as one fused multiply-add per product after the first, a +
+// b (p q) as one.  One difference is kept: the adjoint's GGX samples (sample_ggx).
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
 __device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
@@ -711,8 +711,12 @@ __device__ __forceinline__ float ggx_lambda(float c, float a2) {
 }
 
 // Heitz 2018 visible-normal sample, returns the reflected light direction.  The
-// adjoint sums wo's projections in another order than the forward kernels (a
-// last bit of the direction, a texel or two of a million samples).
+// adjoint sums wo's projections in another order than the forward kernels: its
+// direction may differ in the last bits, and in one or two of a million samples (more
+// with a finer probe) it reads the neighbouring texel.  That is rounding either way,
+// but a smooth lobe's gradients are so steep in the direction that the forward's
+// order moves them by up to 1.5e-3 of their norm, further than results may move: the
+// adjoint keeps its own.
 template <bool kAdjoint>
 __device__ __forceinline__ f3 sample_ggx(f3 n, f3 b1, f3 b2, f3 wo, float alpha, float u0, float u1) {
     const f3 lo = kAdjoint ? mk(dot_rn(wo, b1), dot_rn(wo, b2), dot_rn(wo, n))

@@ -461,9 +461,9 @@ MCDI_API mcdi_status mcdi_denoise_wgrad(int precision, int n_img, int H, int W, 
  * 8 ints to rec (host memory, room for cap records; later ones are dropped):
  *   {pass (0 forward, 1 input gradient), convolution index 0..14 (the order of
  *    mcdi_denoise_pack_weights), level (0 = full resolution), row-tile form
- *    (1) or one CTA per 128-pixel tile (0), output rows per row tile R (0 in
- *    the tile form), ReLU-mask prefetching variant (0/1), 2x2 max-pool written
- *    from the epilogue (0/1), E4M3 operands (0/1)};
+ *    (1), halo-tile form (2) or one CTA per 128-pixel tile (0), output rows
+ *    per row tile R (0 in the other forms), ReLU-mask words loaded ahead (0/1),
+ *    2x2 max-pool written from the epilogue (0/1), E4M3 operands (0/1)};
  * *count (host) is reset to 0 by this call and counts the records written.
  * mcdi_denoise_record_plan(NULL, 0, NULL) stops recording.  The records say
  * which kernel variants a launch configuration runs. */

@@ -511,7 +511,7 @@ static cudaError_t run_conv(Unet& u, int level, const bf16* x, int x_slot, int c
         r[0] = w.dgrad ? 1 : 0;
         r[1] = w.i;
         r[2] = level;
-        r[3] = d.rows_form ? 1 : 0;
+        r[3] = d.halo_form ? 2 : d.rows_form ? 1 : 0;
         r[4] = d.rows_form ? d.rp.rows : 0;
         r[5] = conv_mask_prefetch(d) ? 1 : 0;
         r[6] = d.p.pool_out != nullptr ? 1 : 0;

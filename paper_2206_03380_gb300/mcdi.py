@@ -568,7 +568,8 @@ def unflatten_unet_params(flat):
 class denoise_plan_recorder:
     """Context manager: records the launch plan of every convolution the denoiser
     launches from this thread inside the block; ``records`` then holds one dict per
-    convolution (pass, conv, level, rows_form, rows, mask_prefetch, pool_fused, e4m3)."""
+    convolution (pass, conv, level, rows_form: 1 row tiles, 2 halo tiles, 0 neither; rows,
+    mask_prefetch, pool_fused, e4m3)."""
 
     KEYS = ("pass", "conv", "level", "rows_form", "rows", "mask_prefetch", "pool_fused", "e4m3")
 

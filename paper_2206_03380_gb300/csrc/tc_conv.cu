@@ -16,7 +16,8 @@
 //   warp 0 lane 0  issues the TMA loads      (waits "empty", arms "full"),
 //   warp 1 lane 0  issues the MMAs           (waits "full", commits to "empty"),
 //   all 4 warps    run the epilogue: tcgen05.ld of their 32 TMEM lanes, bias,
-//                  ReLU / gradient mask, BF16 (or FP32) stores.
+//                  ReLU, BF16 stores (kStore only: the denoiser's own layers all
+//                  fit one of the other forms).
 // Every wait is bounded (2 s of %globaltimer); on a timeout the kernel sets
 // *err, stops issuing work, drains its own copies in flight and frees TMEM.
 #include <stdio.h>
@@ -25,6 +26,7 @@
 
 #include <cudaTypedefs.h>
 
+#include "common.cuh"
 #include "tc_conv.cuh"
 #include "tcgen05.cuh"
 
@@ -150,132 +152,19 @@ __device__ __forceinline__ size_t plane_off(int img, int G, int g, int H, int W,
     return ((((size_t)img * G + g) * H + y) * W + x) * 8;
 }
 
-// the ReLU mask words of 16 channels (two 8-channel groups) of one pixel
-__device__ __forceinline__ void load_mask16(const ConvParams& p, int c0, int img, int x, int y, uint4* m) {
-    const __nv_bfloat16* mk = p.mask + plane_off(img, p.mask_ctotal >> 3, (p.mask_coff + c0) >> 3, p.H, p.W, y, x);
-    m[0] = __ldg(reinterpret_cast<const uint4*>(mk));
-    m[1] = __ldg(reinterpret_cast<const uint4*>(mk + (size_t)p.H * p.W * 8));
-}
-
-// bias / activation / mask and store of 16 output channels (two 8-channel
-// groups) of one pixel; pre: the pixel's mask words are already in (ma, mb)
-template <bool kPoolBwd>
-__device__ __forceinline__ void epilogue16(const ConvParams& p, const uint32_t* v, int c0, int img, int x, int y,
-                                           const float* bias16, float dq, float* amax, bool pre = false,
-                                           uint4 ma = uint4{}, uint4 mb = uint4{}, uint32_t* keep = nullptr) {
+// bias / activation and store of 16 output channels (two 8-channel groups) of one
+// pixel, in the general form
+__device__ __forceinline__ void store_act16(const ConvParams& p, const uint32_t* v, int c0, int img, int x, int y,
+                                            const float* bias16, float dq) {
     float f[16];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) f[i] = __uint_as_float(v[i]) * dq;
-    const size_t hw = (size_t)p.H * p.W;
-    if constexpr (kPoolBwd) {  // the instantiation for kDgradPoolBwd (its loads would crowd the others' registers)
-        // (y, x) is a pooled pixel: its window is (2y + dy, 2x + dx) at twice the size
-        const int H2 = 2 * p.H, W2 = 2 * p.W;
-        auto bf = [](uint32_t w, int hi) {  // BF16 half of a packed pair as float
-            return __uint_as_float(hi ? (w & 0xffff0000u) : (w << 16));
-        };
-#pragma unroll
-        for (int gg = 0; gg < 2; ++gg) {
-            const size_t e0 =
-                plane_off(img, p.mask_ctotal >> 3, ((p.mask_coff + c0) >> 3) + gg, H2, W2, 2 * y, 2 * x);
-            uint32_t we[4][4];  // the window's E values, packed BF16 pairs
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const uint4 t = __ldg(reinterpret_cast<const uint4*>(p.mask + e0 + ((size_t)(k >> 1) * W2 + (k & 1)) * 8));
-                we[k][0] = t.x, we[k][1] = t.y, we[k][2] = t.z, we[k][3] = t.w;
-            }
-            int arg[8];
-#pragma unroll
-            for (int c = 0; c < 8; ++c) {  // the window's first maximum, in window order
-                arg[c] = 0;
-                float best = bf(we[0][c >> 1], c & 1);
-#pragma unroll
-                for (int k = 1; k < 4; ++k) {
-                    const float e = bf(we[k][c >> 1], c & 1);
-                    if (e > best) best = e, arg[c] = k;
-                }
-            }
-            const size_t o0 = plane_off(img, p.out_ctotal >> 3, ((p.out_coff + c0) >> 3) + gg, H2, W2, 2 * y, 2 * x);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const size_t off = ((size_t)(k >> 1) * W2 + (k & 1)) * 8;
-                const uint4 t = __ldg(reinterpret_cast<const uint4*>(p.gskip + e0 + off));
-                const uint32_t wg[4] = {t.x, t.y, t.z, t.w};
-                float o[8];
-#pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    const float gp = __bfloat162float(__float2bfloat16_rn(f[8 * gg + c]));  // as stored unfused
-                    const float v = bf(wg[c >> 1], c & 1) + (arg[c] == k ? gp : 0.0f);
-                    o[c] = bf(we[k][c >> 1], c & 1) > 0.0f ? v : 0.0f;
-                    *amax = fmaxf(*amax, fabsf(o[c]));
-                }
-                store8_bf16(p.out + o0 + off, o);
-            }
-        }
-        return;
-    } else {
-    if (p.mode == kDgradMask || p.mode == kDgradPlain) {
-        if (p.mode == kDgradMask) {
-            uint4 mm[2] = {ma, mb};
-            if (!pre) load_mask16(p, c0, img, x, y, mm);
-            const uint4 m0 = mm[0], m1 = mm[1];
-            const uint32_t mw[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const __nv_bfloat162 h = *reinterpret_cast<const __nv_bfloat162*>(&mw[i]);
-                if (!(__bfloat162float(h.x) > 0.0f)) f[2 * i] = 0.0f;
-                if (!(__bfloat162float(h.y) > 0.0f)) f[2 * i + 1] = 0.0f;
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < 16; ++i) *amax = fmaxf(*amax, fabsf(f[i]));
-        __nv_bfloat16* o = p.out + plane_off(img, p.out_ctotal >> 3, (p.out_coff + c0) >> 3, p.H, p.W, y, x);
-        store8_bf16(o, f);
-        store8_bf16(o + hw * 8, f + 8);
-        return;
-    }
-#pragma unroll
     for (int i = 0; i < 16; ++i) {
-        f[i] += bias16 ? bias16[i] : 0.0f;
+        f[i] = __fadd_rn(__fmul_rn(__uint_as_float(v[i]), dq), bias16 ? bias16[i] : 0.0f);
         if (p.relu) f[i] = fmaxf(f[i], 0.0f);
-        *amax = fmaxf(*amax, fabsf(f[i]));
     }
-    if (keep) {  // the 16 stored values as packed BF16 pairs
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            __nv_bfloat162 h = __floats2bfloat162_rn(f[2 * i], f[2 * i + 1]);
-            keep[i] = *reinterpret_cast<uint32_t*>(&h);
-        }
-    }
-    if (p.mode == kStoreF32) {
-        p.out_f32[((size_t)img * p.H + y) * p.W + x] = make_float4(f[0], f[1], f[2], 0.0f);
-    } else if (p.mode == kStoreUp2) {
-        const int W2 = 2 * p.W, H2 = 2 * p.H;
-        __nv_bfloat16* o = p.out + plane_off(img, p.out_ctotal >> 3, (p.out_coff + c0) >> 3, H2, W2, 2 * y, 2 * x);
-        const size_t hw2 = (size_t)H2 * W2 * 8;
-#pragma unroll
-        for (int j = 0; j < 2; ++j)
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                __nv_bfloat16* q = o + ((size_t)j * W2 + i) * 8;
-                store8_bf16(q, f);
-                store8_bf16(q + hw2, f + 8);
-            }
-    } else {
-        __nv_bfloat16* o = p.out + plane_off(img, p.out_ctotal >> 3, (p.out_coff + c0) >> 3, p.H, p.W, y, x);
-        store8_bf16(o, f);
-        store8_bf16(o + hw * 8, f + 8);
-    }
-    }
-}
-
-// Publish a thread's running max |value| of the stored output: rounded to BF16
-// like the stored values (rounding is monotonic, so this is the max over the
-// stored tensor), reduced over the warp, one atomic per warp while the maximum grows.
-__device__ __forceinline__ void publish_amax(unsigned* out_amax, float m, unsigned mask) {
-    if (out_amax == nullptr) return;
-    const unsigned b = __float_as_uint(__bfloat162float(__float2bfloat16_rn(m)));
-    const unsigned w = __reduce_max_sync(mask, b);
-    if ((threadIdx.x & 31) == __ffs(mask) - 1 && w) atomicMax(out_amax, w);
+    __nv_bfloat16* o = p.out + plane_off(img, p.out_ctotal >> 3, (p.out_coff + c0) >> 3, p.H, p.W, y, x);
+    store8_bf16(o, f);
+    store8_bf16(o + (size_t)p.H * p.W * 8, f + 8);
 }
 
 // accumulator scale: 1 for BF16; (amax_x / 448) (amax_w / 448) for E4M3
@@ -285,7 +174,7 @@ __device__ __forceinline__ float dequant_factor(const ConvParams& p) {
     return (__ldg(p.x_amax) * (1.0f / 448.0f)) * (__ldg(p.w_amax) * (1.0f / 448.0f));
 }
 
-template <bool FP8, bool PB>
+template <bool FP8>
 __global__ void __launch_bounds__(kConvThreads) conv_tc_kernel(const __grid_constant__ CUtensorMap tmap_x,
                                                                const __grid_constant__ CUtensorMap tmap_w,
                                                                const ConvParams p) {
@@ -390,16 +279,14 @@ __global__ void __launch_bounds__(kConvThreads) conv_tc_kernel(const __grid_cons
     const int x = x0 + xx, y = y0 + yy;
     const bool valid = acc_ok && x < p.W && y < p.H;
     const float dq = dequant_factor(p);
-    float amax = 0.0f;
     for (int c0 = 0; c0 < p.cout_pad; c0 += 16) {
         uint32_t v[16];
         // collective load of 16 accumulator columns of this warp's 32 lanes
         tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
         if (valid && c0 < p.cout_valid)
-            epilogue16<PB>(p, v, c0, img, x, y, p.bias ? p.bias + c0 : nullptr, dq, &amax);
+            store_act16(p, v, c0, img, x, y, p.bias ? p.bias + c0 : nullptr, dq);
         __syncwarp();
     }
-    publish_amax(p.out_amax, amax, 0xffffffffu);
 
     // ---- teardown
     tc_fence_before();
@@ -473,15 +360,6 @@ __device__ __forceinline__ uint32_t max_bf16(uint32_t a, uint32_t b) {
     const __nv_bfloat162 m = __hmax2(as_bf162(a), as_bf162(b));
     return *reinterpret_cast<const uint32_t*>(&m);
 }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) {
-    float2 r;
-    asm("{\n\t.reg .b64 ra, rb, rd;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
-        "add.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
-        : "=f"(r.x), "=f"(r.y)
-        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-    return r;
-}
-
 // accumulators (times dq for E4M3 operands) plus bias, rounded to BF16
 template <bool FP8>
 __device__ __forceinline__ void bias_pack16(const uint32_t* v, float dq, const float* bias, uint32_t* h) {
@@ -1428,6 +1306,10 @@ bool conv_make_desc(ConvDesc* d, const void* x, const void* w, const char** why)
         return false;
     }
     d->rows_form = plan_rows(d->p, &d->rp);
+    if (!d->rows_form && (p.mode != kStore || p.out_amax != nullptr)) {  // what the general form can do
+        *why = "layer outside the row-tile and halo-tile forms";
+        return false;
+    }
     if (d->rows_form) {
         const RowPlan& rp = d->rp;
         d->p.tiles_y = (p.H + rp.rows - 1) / rp.rows;
@@ -1491,8 +1373,7 @@ cudaError_t conv_launch(const ConvDesc& d, cudaStream_t stream) {
     std::call_once(once, [] {
         const int lim = (int)device_limits().rows_smem_max;
         const int tile = (int)conv_smem_bytes(256);
-        const void* generic[4] = {(const void*)conv_tc_kernel<false, false>, (const void*)conv_tc_kernel<true, false>,
-                                  (const void*)conv_tc_kernel<false, true>, (const void*)conv_tc_kernel<true, true>};
+        const void* generic[2] = {(const void*)conv_tc_kernel<false>, (const void*)conv_tc_kernel<true>};
         for (const void* f : generic)
             if (attr_err == cudaSuccess)
                 attr_err = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, tile);
@@ -1524,14 +1405,8 @@ cudaError_t conv_launch(const ConvDesc& d, cudaStream_t stream) {
     }
     const int n_tiles = d.p.n_img * d.p.tiles_y * d.p.tiles_x;
     const size_t smem = conv_smem_bytes(d.p.cout_pad);
-    const bool pb = d.p.mode == kDgradPoolBwd;
-    if (d.p.fp8) {
-        if (pb) launch_k(conv_tc_kernel<true, true>, n_tiles, kConvThreads, smem, stream, d.tmap_x, d.tmap_w, d.p);
-        else launch_k(conv_tc_kernel<true, false>, n_tiles, kConvThreads, smem, stream, d.tmap_x, d.tmap_w, d.p);
-    } else {
-        if (pb) launch_k(conv_tc_kernel<false, true>, n_tiles, kConvThreads, smem, stream, d.tmap_x, d.tmap_w, d.p);
-        else launch_k(conv_tc_kernel<false, false>, n_tiles, kConvThreads, smem, stream, d.tmap_x, d.tmap_w, d.p);
-    }
+    if (d.p.fp8) launch_k(conv_tc_kernel<true>, n_tiles, kConvThreads, smem, stream, d.tmap_x, d.tmap_w, d.p);
+    else launch_k(conv_tc_kernel<false>, n_tiles, kConvThreads, smem, stream, d.tmap_x, d.tmap_w, d.p);
     return cudaGetLastError();
 }
 

@@ -83,8 +83,10 @@ MCDI_API mcdi_status mcdi_build_envmap_cdf(const float* env, int W, int H, float
  * and `tri_records` (16-byte aligned), opaque layouts valid until the caller
  * frees them; `scratch` is
  * overwritten.  Build = Morton codes -> LSD radix sort -> Karras hierarchy ->
- * bottom-up bounds -> a depth-first copy with escape links, which shadow rays
- * traverse without a stack.  Deterministic for a given input.
+ * bottom-up bounds -> four-wide nodes with 8-bit child boxes, which rays
+ * traverse, and a depth-first copy with escape links for the rays those boxes
+ * do not hold for (origins far outside the mesh, infinite bounds, deep
+ * stacks).  Deterministic for a given input.
  * ------------------------------------------------------------------------ */
 MCDI_API mcdi_status mcdi_bvh_sizes(int n_tris, size_t* node_bytes, size_t* tri_bytes, size_t* scratch_bytes);
 MCDI_API mcdi_status mcdi_build_bvh(const float* verts, int n_verts, const int* tris, int n_tris, void* nodes,

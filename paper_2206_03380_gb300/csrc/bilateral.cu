@@ -241,9 +241,9 @@ size_t bilateral_smem(int R, int K) {
 // A CTA owns a tile of one view, 32 pixels wide, each thread two pixels of a
 // column; guides and the upstream gradients divided by W(p) over the tile plus its
 // halo are staged in shared memory, and from the guides every staged pixel's
-// slopes.  What bounds it is three things at about the same level, per weight and
-// warp: some 45 issued instructions, 3 MUFU operations and shared-memory
-// wavefronts (16 per neighbour for two images), then the staging's latency.  So a
+// slopes.  What bounds it is three things at about the same level, per pair of
+// weights and warp: some 50 issued instructions, 4 MUFU operations and 15
+// shared-memory wavefronts (for two images), then the staging's latency.  So a
 // neighbour loaded once meets two pixels, their arithmetic goes in packed pairs,
 // the spatial factors come from a table, the division takes no branch, and
 // uncovered neighbours (zero normal and gradients) take none either.  Every

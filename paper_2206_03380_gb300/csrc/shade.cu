@@ -1,7 +1,8 @@
 // Shading kernels: the G-buffer ray cast, the forward MIS estimator and its
-// hand-written adjoint (Sec. 3.1, Sec. 4.1, Sec. 4.2).  One thread shades one
-// pixel with all of its samples; G-buffer planes are read and outputs written
-// as coalesced float4.
+// hand-written adjoint (Sec. 3.1, Sec. 4.1, Sec. 4.2).  The ray cast walks the
+// tree with a pair of lanes per pixel; forward and adjoint shade 32 consecutive
+// pixels per CTA, their samples split over its four warps.  G-buffer planes are
+// read and outputs written as float4.
 #include "common.cuh"
 #include "internal.h"
 #include "shading.cuh"

@@ -214,9 +214,10 @@ __device__ __forceinline__ float qbyte(uint32_t w, int k) {
 
 // The largest coordinate (in magnitude) that a ray's origin o may have for the
 // four-wide nodes' boxes to hold what they should, or a negative number where no ray
-// may use them (then and beyond, the two-child or depth-first nodes decide).  With m the largest coordinate of the root box, P a child box's
-// plane and a its node's origin, the computed distance to the plane (wide_visit)
-// differs from (P - o) / d, in units of the axis, by at most
+// may use them; the two-child or the depth-first nodes decide then and beyond.  With
+// m the largest coordinate of the root box, P a child box's plane and a its node's
+// origin, the computed distance to the plane (wide_visit) differs from (P - o) / d, in
+// units of the axis, by at most
 //   u |P - o| (1 / d) + u |o| (its product) + u |a - o| (the difference)
 //   + u (2^23 s + |a - o|) (B') + u |P - o| (the last sum)  <=  s / 2 + u (5 |o| + 4 m).
 // The child boxes are a step s >= 2^-17 m wider on each side, so |o| may be 12 m; 11
@@ -474,12 +475,15 @@ __device__ __forceinline__ float tri_hit_rn(f3 o, f3 d, const TriRecord* __restr
 // two-child nodes 175), 190k triangles, 133 x 77: 86 (71; 127; 115), 157k
 // triangles, 64 x 64: 79 (63; 119; 108).  A persistent tracer that refills lanes
 // leaves too few in flight: 208 to 340.
+// A triangle is decided as closest_hit decides it, bit for bit; only where two lie at
+// the same or nearly the same distance (a shared edge, faces that touch) may the pair,
+// which meets them in another order, take the other one: on a mesh of 1.2M triangles
+// the planes then differ by 3e-8 of their norm, 1e-5 at most.
 // The whole warp calls it and stays together (node: 0, or -1 for a pair without a
 // ray).  An empty slot's box is inverted, which rejects every finite ray; its link
-// is checked all the same before it becomes a triangle's
-// index.  Pending nodes and their entry distances are a row of shared memory per
-// ray.  Returns the leaf, the same in both lanes, or kWideOverflow: more pending
-// nodes than the row holds.
+// is checked all the same before it becomes a triangle's index.  Pending nodes and
+// their entry distances are a row of shared memory per ray.  Returns the leaf, the
+// same in both lanes, or kWideOverflow: more pending nodes than the row holds.
 constexpr int kCastStack = 24;
 constexpr int kWideOverflow = -2;
 __device__ __forceinline__ int closest_hit_wide(const WideNode* __restrict__ wn, const TriRecord* __restrict__ tris,
